@@ -45,15 +45,47 @@ struct Phys {
   double gamma_d, rho_floor_d, p_floor_d;  // FP64 copies for the floor branch
 };
 
-// Correctly rounded reciprocal (the host build, used only by host-side unit
-// harnesses, divides).
-MHD_HD double rcp(double x) {
+// Single-precision seeds of the FP64 reciprocal and square root below (the
+// host build, used only by host-side unit harnesses, divides).
+MHD_HD float seed_rcp(float x) {
 #ifdef __CUDA_ARCH__
-  return __drcp_rn(x);
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
 #else
-  return 1.0 / x;
+  return 1.0f / x;
 #endif
 }
+MHD_HD float seed_rsqrt(float x) {
+#ifdef __CUDA_ARCH__
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+#else
+  return 1.0f / sqrtf(x);
+#endif
+}
+MHD_HD uint32_t f32_bits(float x) {
+#ifdef __CUDA_ARCH__
+  return __float_as_uint(x);
+#else
+  uint32_t b;
+  memcpy(&b, &x, sizeof(b));
+  return b;
+#endif
+}
+MHD_HD float bits_f32(uint32_t b) {
+#ifdef __CUDA_ARCH__
+  return __uint_as_float(b);
+#else
+  float x;
+  memcpy(&x, &b, sizeof(x));
+  return x;
+#endif
+}
+MHD_HD uint32_t mulhi_u(uint32_t a, uint32_t b) { return (uint32_t)(((uint64_t)a * b) >> 32); }
+MHD_HD int32_t mulhi_s(int32_t a, int32_t b) { return (int32_t)(((int64_t)a * b) >> 32); }
+
 // FP32 mode: hardware-approximate reciprocal and square root (a few ulp;
 // the FP32 bulk path's error budget is ~1e-5 relative).
 MHD_HD float rcp(float x) {
@@ -93,7 +125,6 @@ MHD_HD T dot3_rn(T a0, T b0, T a1, T b1, T a2, T b2) {
 
 MHD_HD double trsqrt(double x) { return rsqrt(x); }
 MHD_HD float trsqrt(float x) { return rsqrtf(x); }
-MHD_HD double tsqrt(double x) { return sqrt(x); }
 MHD_HD float tsqrt(float x) {
 #ifdef __CUDA_ARCH__
   return x > 0.0f ? x * rsqrtf(x) : 0.0f;
@@ -126,6 +157,86 @@ MHD_HD double bits2d(long long b) {
   double x;
   memcpy(&x, &b, sizeof(x));
   return x;
+#endif
+}
+
+// FP64 reciprocal and square root without FP64 instructions.  The SM's FP64
+// unit issues 1.68 lanes per clock against 128 for the integer and FP32
+// pipes, which idle beside it.  Clocks per warp and SM with the pipes full:
+// CUDA's correctly rounded reciprocal 83.5, this one 21.8; CUDA's square root
+// 141, this one 26.2 (a fused multiply-add takes 15.6).  A single-precision seed of the significand (relative
+// error < 2^-21) is corrected in 64-bit fixed point: the residual against the
+// full significand is exact to 2^-62, and the first- and second-order terms of
+// the correction leave less than 2^-61, so the rounded result is within 0.51
+// ulp.  Both need a biased exponent in [64, 1982] (in_fixed_range); other
+// operands (zero, subnormal, extreme, infinite, NaN, negative for the root)
+// take the CUDA function behind a branch.
+MHD_HD bool in_fixed_range(uint32_t hi) { return ((hi >> 20) & 0x7ffu) - 64u < 1919u; }
+
+MHD_HD double rcp_fixed(double x) {
+  const uint64_t b = (uint64_t)dbits(x);
+  const uint32_t hi = (uint32_t)(b >> 32), lo = (uint32_t)b;
+  // significand in [1, 2): xh 2^-31 + xl 2^-63
+  const uint32_t xh = 0x80000000u | (hi << 11) | (lo >> 21), xl = lo << 11;
+  const float r0 = seed_rcp(bits_f32(0x3f800000u | ((xh >> 8) & 0x7fffffu)));
+  const float r = fminf(fmaxf(r0, 0.5f), 0.99999994f);
+  const uint32_t y = (f32_bits(r) << 8) | 0x80000000u;  // seed, units 2^-32
+  const int32_t yh = (int32_t)(y >> 1);                 // the same, units 2^-31
+  // e = 1 - x y and the corrections y e, y e^2, units 2^-62
+  const int64_t e = (int64_t)(0x4000000000000000ull -
+                              ((uint64_t)xh * (uint32_t)yh + mulhi_u(xl, (uint32_t)yh)));
+  const int64_t c = (((int64_t)(int32_t)(e >> 32) * yh) << 1) + mulhi_u((uint32_t)e, y);
+  const int32_t c2 = mulhi_s((int32_t)(c >> 11), (int32_t)(e >> 11)) >> 8;
+  const uint64_t q = ((uint64_t)(uint32_t)yh << 31) + (uint64_t)c + (uint64_t)(int64_t)c2;
+  const uint64_t m = (q + 0x100u) >> 9;  // [2^52, 2^53]
+  const uint64_t ex = (uint64_t)(2044u - ((hi >> 20) & 0x7ffu)) << 52;
+  return bits2d((int64_t)((m + ex) | (b & 0x8000000000000000ull)));
+}
+
+MHD_HD double sqrt_fixed(double x) {
+  const uint64_t b = (uint64_t)dbits(x);
+  const uint32_t hi = (uint32_t)(b >> 32);
+  const uint32_t odd = ((hi >> 20) & 1u) ^ 1u;  // odd exponent: significand in [2, 4)
+  // m in [1, 4), units 2^-62
+  const uint64_t m = ((b & 0x000fffffffffffffull) | 0x0010000000000000ull) << (10 + odd);
+  const float f = bits_f32((0x3f800000u + (odd << 23)) | (uint32_t)((b >> 29) & 0x7fffffu));
+  const float y0 = fminf(fmaxf(seed_rsqrt(f), 0.5f), 0.99999994f);
+  const float s0 = fminf(fmaxf(f * y0, 1.0f), 1.9999999f);
+  const uint32_t t = (f32_bits(s0) << 8) | 0x80000000u;                  // units 2^-31
+  const int32_t yh = (int32_t)(((f32_bits(y0) << 8) | 0x80000000u) >> 1);  // units 2^-31
+  // sqrt(m) = t + d + d (e - d y / 2) with r = m - t^2, d = r y / 2, e = 1 - t y
+  const int64_t r = (int64_t)(m - (uint64_t)t * t);
+  const int64_t d = (int64_t)(int32_t)(r >> 32) * yh + mulhi_u((uint32_t)r, (uint32_t)yh);
+  const int64_t e = (int64_t)(0x4000000000000000ull - (uint64_t)t * (uint32_t)yh);
+  const int32_t ds = (int32_t)(d >> 12);  // units 2^-50
+  const int32_t g = (int32_t)(e >> 12) - mulhi_s(ds, yh);
+  const uint64_t q = ((uint64_t)t << 31) + (uint64_t)d + (uint64_t)(int64_t)(mulhi_s(ds, g) >> 6);
+  const uint64_t s = (q + 0x200u) >> 10;  // [2^52, 2^53]
+  const uint64_t ex = (uint64_t)((((hi >> 20) + 1023u) >> 1) - 1u) << 52;
+  return bits2d((int64_t)(s + ex));
+}
+
+// (The CUDA functions as volatile asm: otherwise the compiler evaluates them
+// for every operand and selects afterwards.)
+MHD_HD double rcp(double x) {
+#ifdef __CUDA_ARCH__
+  double r = rcp_fixed(x);
+  if (!in_fixed_range((uint32_t)__double2hiint(x)))
+    asm volatile("rcp.rn.f64 %0, %1;" : "=d"(r) : "d"(x));
+  return r;
+#else
+  return 1.0 / x;
+#endif
+}
+MHD_HD double tsqrt(double x) {
+#ifdef __CUDA_ARCH__
+  const uint32_t hi = (uint32_t)__double2hiint(x);
+  double s = sqrt_fixed(x);
+  if (!in_fixed_range(hi) || (int)hi < 0)
+    asm volatile("sqrt.rn.f64 %0, %1;" : "=d"(s) : "d"(x));
+  return s;
+#else
+  return sqrt(x);
 #endif
 }
 
@@ -315,21 +426,20 @@ MHD_HD long long sign_bit_of(bool negative) {
 MHD_HD double sign_mul(double x, long long sbit) { return bits2d(dbits(x) ^ sbit); }
 MHD_HD float sign_mul(float x, long long sbit) { return sbit ? -x : x; }
 
-// Fast magnetosonic speed squared from 1/rho, gamma p, |B|^2 and B_n^2:
-// with g = gamma p / rho, a = g + |B|^2 / rho and c_an^2 = B_n^2 / rho,
-// c_f^2 = (a + sqrt(a^2 - 4 g c_an^2)) / 2.
+// Twice the fast magnetosonic speed squared from 1/rho, gamma p, |B|^2 and
+// B_n^2: with g = gamma p / rho, a = g + |B|^2 / rho and c_an^2 = B_n^2 / rho,
+// 2 c_f^2 = a + sqrt(a^2 - 4 g c_an^2).
 template <class T>
-MHD_HD T fast_speed2(T rho_i, T gp, T b2, T bn2) {
+MHD_HD T fast_speed2x(T rho_i, T gp, T b2, T bn2) {
   const T g = mul_rn(gp, rho_i);
   const T a = fma_rn(b2, rho_i, g);
-  const T disc = pos_part(fma_rn(a, a, neg4(g * (bn2 * rho_i))));
-  return half_of(a + tsqrt(disc));
+  return a + tsqrt(pos_part(fma_rn(a, a, neg4(g * (bn2 * rho_i)))));
 }
 
-// Fast magnetosonic speed (see fast_speed2).
+// Fast magnetosonic speed (see fast_speed2x).
 template <class T>
 MHD_HD T fast_speed(T rho_i, T gp, T b2, T bn2) {
-  return tsqrt(fast_speed2(rho_i, gp, b2, bn2));
+  return tsqrt(half_of(fast_speed2x(rho_i, gp, b2, bn2)));
 }
 
 // max over active directions of |v_d| + c_f,d for one conservative cell.
@@ -708,6 +818,14 @@ __device__ __forceinline__ void glm_hlld_flux_f32x2(const float vl[kNV], const f
 // is written with mul_rn / fma_rn / dot3_rn, so the flux rounds the same in
 // every kernel and at every call site it is inlined into (the results of
 // decomposed and undecomposed runs must agree bit for bit).
+// FP64 is bound by the SM's FP64 unit, so the solver is arranged for few FP64
+// operations: about 95 per face, 130 where a lane of the warp is inside the
+// Alfven fan (the form that builds both sides' star and double-star states and
+// adds up the wave jumps took about 280 with CUDA's divisions and roots).
+// Orszag-Tang 256^3 FP64: 76.4 -> 47.4 ms per step, of which the fixed-point
+// reciprocals and roots 11.  Against a quadruple-precision evaluation its
+// error is at most that of the longer form (2e-16 to 3e-15 rms of the flux,
+// random, smooth, Mach-20, low- and high-beta and degenerate face states).
 template <int dir, class T>
 MHD_HD void glm_hlld_flux(const T vl[kNV], const T vr[kNV], T ch, T half_chi,
                           const Phys<T>& ph, T F[kNV]) {
@@ -736,134 +854,122 @@ MHD_HD void glm_hlld_flux(const T vl[kNV], const T vr[kNV], T ch, T half_chi,
   // GLM: exact solution of the linear (B_n, psi) interface problem
   const T bx = fma_rn(half, bnL + bnR, -mul_rn(half_chi, vr[kPSI] - vl[kPSI]));
   const T psis = fma_rn(half, vl[kPSI] + vr[kPSI], -mul_rn(half * ch, bnR - bnL));
-  const T bx2 = bx * bx;
+  const T bx2 = mul_rn(bx, bx);
 
-  // outer states
+  // total pressures; c_max, the larger fast speed: one square root of the
+  // larger c_f^2 (sqrt is monotone)
   const T b2L = fma_rn(bzL, bzL, fma_rn(byL, byL, bx2));
   const T b2R = fma_rn(bzR, bzR, fma_rn(byR, byR, bx2));
   const T ptL = fma_rn(half, b2L, pL), ptR = fma_rn(half, b2R, pR);
-  // (rho / 2 by half_of: an exponent move in FP64, the same value as 0.5 * rho)
-  const T eL = fma_rn(half, b2L,
-                      fma_rn(half_of(rL), dot3_rn(uL, uL, vL, vL, wL, wL), mul_rn(pL, ph.gm1i)));
-  const T eR = fma_rn(half, b2R,
-                      fma_rn(half_of(rR), dot3_rn(uR, uR, vR, vR, wR, wR), mul_rn(pR, ph.gm1i)));
-  // 1/rho of both sides from one reciprocal; only max(c_fL, c_fR) is used,
-  // so one square root of max(c_fL^2, c_fR^2) (sqrt is monotone and
-  // correctly rounded: the same value)
-  const T qr = rcp(rL * rR);
-  const T cf2L = fast_speed2(rR * qr, ph.gamma * pL, b2L, bx2);
-  const T cf2R = fast_speed2(rL * qr, ph.gamma * pR, b2R, bx2);
+  const T cf2L = fast_speed2x(rcp(rL), mul_rn(ph.gamma, pL), b2L, bx2);
+  const T cf2R = fast_speed2x(rcp(rR), mul_rn(ph.gamma, pR), b2R, bx2);
+  const T cmax = tsqrt(half_of(tmax2(cf2L, cf2R)));
 
-  // wave-speed estimates (MK05 Eq. 67), contact speed and total pressure
-  const T cmax = tsqrt(tmax2(cf2L, cf2R));
+  // wave-speed estimates (MK05 Eq. 67) and contact speed (Eq. 38, written as
+  // u_L plus a correction)
   const T SL = tmin2(uL, uR) - cmax;
   const T SR = tmax2(uL, uR) + cmax;
-  const T dL = (SL - uL) * rL, dR = (SR - uR) * rR;
-  const T Di = rcp(dR - dL);
-  const T SM = (fma_rn(dR, uR, -mul_rn(dL, uL)) - ptR + ptL) * Di;
-  const T pts = fma_rn(mul_rn(dL, dR), uR - uL, fma_rn(dR, ptL, -mul_rn(dL, ptR))) * Di;
+  const T SuL = SL - uL, SuR = SR - uR;
+  const T dL = mul_rn(SuL, rL), dR = mul_rn(SuR, rR);
+  const T SM = fma_rn(fma_rn(dR, uR - uL, ptL - ptR), rcp(dR - dL), uL);
 
-  // single-star states (MK05 Eqs. 43-48), degenerate when
-  // |rho (S-u)(S-S_M) - Bx^2| < 1e-8 p_t*; paired reciprocals of S-S_M and
-  // of the two denominators
-  const T smL = SL - SM, smR = SR - SM;
-  const T denL = fma_rn(dL, smL, -bx2), denR = fma_rn(dR, smR, -bx2);
-  const bool degL = abs_lt(denL, T(1e-8) * pts);
-  const bool degR = abs_lt(denR, T(1e-8) * pts);
-  const T dnL = degL ? T(1) : denL, dnR = degR ? T(1) : denR;
-  const T ps = smL * smR, pd = dnL * dnR;
-  const T q4 = rcp(ps * pd);  // one reciprocal for the four divisors
-  const T qs = pd * q4, qd = ps * q4;
-  const T smiL = smR * qs, smiR = smL * qs;
-  const T deniL = dnR * qd, deniR = dnL * qd;
-  T rsL, vsL, wsL, bysL, bzsL, esL, vbsL, vbL;
-  T rsR, vsR, wsR, bysR, bzsR, esR, vbsR, vbR;
-  {
-    rsL = dL * smiL;
-    const T fv = bx * (SM - uL) * deniL;
-    const T fb = fma_rn(dL, SL - uL, -bx2) * deniL;
-    vsL = degL ? vL : fma_rn(-byL, fv, vL);
-    wsL = degL ? wL : fma_rn(-bzL, fv, wL);
-    bysL = degL ? byL : byL * fb;
-    bzsL = degL ? bzL : bzL * fb;
-    vbL = dot3_rn(uL, bx, vL, byL, wL, bzL);
-    vbsL = dot3_rn(SM, bx, vsL, bysL, wsL, bzsL);
-    esL = fma_rn(bx, vbL - vbsL,
-                   fma_rn(pts, SM, fma_rn(SL - uL, eL, -mul_rn(ptL, uL)))) *
-          smiL;
-  }
-  {
-    rsR = dR * smiR;
-    const T fv = bx * (SM - uR) * deniR;
-    const T fb = fma_rn(dR, SR - uR, -bx2) * deniR;
-    vsR = degR ? vR : fma_rn(-byR, fv, vR);
-    wsR = degR ? wR : fma_rn(-bzR, fv, wR);
-    bysR = degR ? byR : byR * fb;
-    bzsR = degR ? bzR : bzR * fb;
-    vbR = dot3_rn(uR, bx, vR, byR, wR, bzR);
-    vbsR = dot3_rn(SM, bx, vsR, bysR, wsR, bzsR);
-    esR = fma_rn(bx, vbR - vbsR,
-                   fma_rn(pts, SM, fma_rn(SR - uR, eR, -mul_rn(ptR, uR)))) *
-          smiR;
-  }
-
-  // Fan region: side a = L if (S_L > 0) or (S_R >= 0 and S_M >= 0), else R
-  // (sign tests on the integer pipe in FP64: gt0 / lt0 / ge0).  The side's
-  // outer and single-star values are picked here, before the double-star
-  // states, so that the other side's outer state is no longer live there.
+  // The upwind side a: L if (S_L > 0) or (S_R >= 0 and S_M >= 0), else R
+  // (sign tests on the integer pipe in FP64: gt0 / lt0 / ge0); o: the other
+  // side, which enters only through the double-star states.
   const bool sup = gt0(SL) || lt0(SR);
   const bool useL = gt0(SL) || (!lt0(SR) && ge0(SM));
   const T r = useL ? rL : rR, u = useL ? uL : uR, v = useL ? vL : vR, w = useL ? wL : wR;
-  const T by = useL ? byL : byR, bz = useL ? bzL : bzR, e = useL ? eL : eR;
-  const T pt = useL ? ptL : ptR;
-  const T rs = useL ? rsL : rsR, vs = useL ? vsL : vsR, ws = useL ? wsL : wsR;
-  const T bys = useL ? bysL : bysR, bzs = useL ? bzsL : bzsR, es = useL ? esL : esR;
-  const T vbs = useL ? vbsL : vbsR;
-  const T vb = useL ? vbL : vbR;  // v . B of the side's outer state
-  // the flux terms of the outer and single-star states (the Alfven-fan
-  // terms are added below), so that the outer state dies here
-  const T c1 = sup ? T(0) : (useL ? SL : SR);
-  T f[7];
-  {
-    const T ru = mul_rn(r, u), rv = mul_rn(r, v), rw = mul_rn(r, w);
-    f[0] = fma_rn(c1, rs - r, ru);
-    f[1] = fma_rn(c1, fma_rn(rs, SM, -ru), fma_rn(ru, u, pt) - bx2);
-    f[2] = fma_rn(c1, fma_rn(rs, vs, -rv), fma_rn(rv, u, -mul_rn(bx, by)));
-    f[3] = fma_rn(c1, fma_rn(rs, ws, -rw), fma_rn(rw, u, -mul_rn(bx, bz)));
-    f[4] = fma_rn(c1, bys - by, fma_rn(by, u, -mul_rn(bx, v)));
-    f[5] = fma_rn(c1, bzs - bz, fma_rn(bz, u, -mul_rn(bx, w)));
-    f[6] = fma_rn(c1, es - e, fma_rn(e + pt, u, -mul_rn(bx, vb)));
+  const T by = useL ? byL : byR, bz = useL ? bzL : bzR, b2 = useL ? b2L : b2R;
+  const T p = useL ? pL : pR, pt = useL ? ptL : ptR;
+  const T S = useL ? SL : SR, Su = useL ? SuL : SuR, d = useL ? dL : dR;
+
+  // single-star state of side a (MK05 Eqs. 43-48), degenerate when
+  // den = rho (S-u)(S-S_M) - Bx^2 is below 1e-8 p_t*; p_t* = p_t + rho (S-u)
+  // (S_M-u); B* = B (1 + rho (S-u)(S_M-u) / den); one reciprocal for the two
+  // divisors
+  const T du = SM - u;
+  const T pts = fma_rn(d, du, pt);
+  const T sm = S - SM;
+  const T den = fma_rn(d, sm, -bx2);
+  const bool deg = abs_lt(den, mul_rn(T(1e-8), pts));
+  const T dn = deg ? T(1) : den;
+  const T q = rcp(mul_rn(sm, dn));
+  const T smi = mul_rn(dn, q), deni = mul_rn(sm, q);
+  const T rs = mul_rn(d, smi);
+  const T k0 = mul_rn(du, deni);
+  const T fv = mul_rn(bx, k0), fb = mul_rn(d, k0);
+  const T vs = deg ? v : fma_rn(-by, fv, v);
+  const T ws = deg ? w : fma_rn(-bz, fv, w);
+  const T bys = deg ? by : fma_rn(by, fb, by);
+  const T bzs = deg ? bz : fma_rn(bz, fb, bz);
+  const T vb = dot3_rn(u, bx, v, by, w, bz);
+  const T vbs = dot3_rn(SM, bx, vs, bys, ws, bzs);
+  // (rho / 2 by half_of: an exponent move in FP64, the same value as 0.5 * rho)
+  const T e = fma_rn(half, b2, fma_rn(half_of(r), dot3_rn(u, u, v, v, w, w), mul_rn(p, ph.gm1i)));
+  const T es = mul_rn(fma_rn(bx, vb - vbs,
+                             fma_rn(pts, SM, fma_rn(Su, e, -mul_rn(pt, u)))), smi);
+
+  // The state on the interface: outer where the flow is supersonic, else
+  // single-star, else (below) double-star.
+  const T rF = sup ? r : rs, uF = sup ? u : SM, ptF = sup ? pt : pts;
+  const T ru = mul_rn(rF, uF);
+  T vF = sup ? v : vs, wF = sup ? w : ws, byF = sup ? by : bys, bzF = sup ? bz : bzs;
+  T eF = sup ? e : es, vbF = sup ? vb : vbs;
+
+  // Inside the Alfven fan (S*_L <= 0 <= S*_R, Eq. 51: rho* S_M^2 <= B_x^2) the
+  // double-star states (Eqs. 59-63).  With s = sign(B_x) on side L and
+  // -sign(B_x) on side R, Eqs. 59-62 are a step X from the single-star state
+  // of side a: v** = v* + X, B** = B* + s sqrt(rho*) X, X = (sqrt(rho*_o)
+  // (v*_o - v*) + s (B*_o - B*)) / (sqrt(rho*) + sqrt(rho*_o)).  Skipped where
+  // no lane of the warp is inside the fan.
+  if (!sup && !lt_ieee(bx2, mul_rn(ru, SM))) {
+    const T uo = useL ? uR : uL, vo = useL ? vR : vL, wo = useL ? wR : wL;
+    const T byo = useL ? byR : byL, bzo = useL ? bzR : bzL;
+    const T So = useL ? SR : SL, dO = useL ? dR : dL;
+    const T smo = So - SM;
+    const T deno = fma_rn(dO, smo, -bx2);
+    const bool dego = abs_lt(deno, mul_rn(T(1e-8), pts));
+    const T dno = dego ? T(1) : deno;
+    const T qo = rcp(mul_rn(smo, dno));
+    const T denio = mul_rn(smo, qo);
+    const T rso = mul_rn(dO, mul_rn(dno, qo));
+    const T k0o = mul_rn(SM - uo, denio);
+    const T fvo = mul_rn(bx, k0o), fbo = mul_rn(dO, k0o);
+    const T vso = dego ? vo : fma_rn(-byo, fvo, vo);
+    const T wso = dego ? wo : fma_rn(-bzo, fvo, wo);
+    const T byso = dego ? byo : fma_rn(byo, fbo, byo);
+    const T bzso = dego ? bzo : fma_rn(bzo, fbo, bzo);
+    const T sqa = tsqrt(rs), sqo = tsqrt(rso);
+    const T isum = rcp(sqa + sqo);
+    const long long sg = sign_bit_of(ge0(bx) != useL);
+    const T Xv = mul_rn(fma_rn(sqo, vso - vs, sign_mul(byso - bys, sg)), isum);
+    const T Xw = mul_rn(fma_rn(sqo, wso - ws, sign_mul(bzso - bzs, sg)), isum);
+    const T sqs = sign_mul(sqa, sg);
+    vF = vs + Xv;
+    wF = ws + Xw;
+    byF = fma_rn(sqs, Xv, bys);
+    bzF = fma_rn(sqs, Xw, bzs);
+    vbF = dot3_rn(SM, bx, vF, byF, wF, bzF);
+    eF = fma_rn(sqs, vbF - vbs, es);
   }
 
-  // Alfven waves (MK05 Eq. 51) and double-star states (Eqs. 59-63);
-  // 1/sqrt(rho*) by rsqrt, sqrt(rho*) = rho* / sqrt(rho*)
-  const T iqL = trsqrt(rsL), iqR = trsqrt(rsR);
-  const T sqL = rsL * iqL, sqR = rsR * iqR;
-  const T abx = tabs(bx);
-  const T SLs = fma_rn(-abx, iqL, SM);
-  const T SRs = fma_rn(abx, iqR, SM);
-  // sign(B_x) applied as a sign flip (sign_mul), not a multiplication
-  const long long sg = sign_bit_of(!ge0(bx));
-  const T isum = rcp(sqL + sqR);
-  const T sqLR = mul_rn(sqL, sqR);
-  const T vss = (fma_rn(sqR, vsR, mul_rn(sqL, vsL)) + sign_mul(bysR - bysL, sg)) * isum;
-  const T wss = (fma_rn(sqR, wsR, mul_rn(sqL, wsL)) + sign_mul(bzsR - bzsL, sg)) * isum;
-  const T byss = fma_rn(sqLR, sign_mul(vsR - vsL, sg), fma_rn(sqR, bysL, mul_rn(sqL, bysR))) * isum;
-  const T bzss = fma_rn(sqLR, sign_mul(wsR - wsL, sg), fma_rn(sqR, bzsL, mul_rn(sqL, bzsR))) * isum;
-  const T vbss = dot3_rn(SM, bx, vss, byss, wss, bzss);
-
-  // F = F_a + c1 (U*_a - U_a) + c2 (U**_a - U*_a) with c1 = S_a unless the
-  // interface is supersonic, c2 = S*_a inside the Alfven fan.
-  const bool inner = !sup && (useL ? !gt0(SLs) : !lt0(SRs));
-  const T sq = useL ? -sqL : sqR;
-  const T ess = fma_rn(sq, sign_mul(vbs - vbss, sg), es);
-  const T c2 = inner ? (useL ? SLs : SRs) : T(0);
-  const T c2rs = mul_rn(c2, rs);
-  f[2] = fma_rn(c2rs, vss - vs, f[2]);
-  f[3] = fma_rn(c2rs, wss - ws, f[3]);
-  f[4] = fma_rn(c2, byss - bys, f[4]);
-  f[5] = fma_rn(c2, bzss - bzs, f[5]);
-  f[6] = fma_rn(c2, ess - es, f[6]);
+  // HLLD's fan fluxes F_a + S_a (U*_a - U_a) + S*_a (U**_a - U*_a) (Eqs.
+  // 64-66) are, by the jump relations that define the star states, the physical
+  // flux of the state on the interface with normal velocity S_M and total
+  // pressure p_t* -- except the induction terms of a degenerate star state,
+  // which keeps B* = B: there B (u - S_M) is left over.
+  T f[7];
+  f[0] = ru;
+  f[1] = fma_rn(ru, uF, ptF - bx2);
+  f[2] = fma_rn(ru, vF, -mul_rn(bx, byF));
+  f[3] = fma_rn(ru, wF, -mul_rn(bx, bzF));
+  f[4] = fma_rn(byF, uF, -mul_rn(bx, vF));
+  f[5] = fma_rn(bzF, uF, -mul_rn(bx, wF));
+  f[6] = fma_rn(eF + ptF, uF, -mul_rn(bx, vbF));
+  if (deg && !sup) {
+    f[4] = fma_rn(-by, du, f[4]);
+    f[5] = fma_rn(-bz, du, f[5]);
+  }
 
   F[kRHO] = f[0];
   F[kPRS] = f[6];
