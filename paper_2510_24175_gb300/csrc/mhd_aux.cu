@@ -12,6 +12,7 @@ Phys<T> make_phys(const Grid& g) {
   ph.gamma = T(g.gamma);
   ph.gm1 = T(g.gamma - 1.0);
   ph.gm1i = T(1.0 / (g.gamma - 1.0));
+  ph.gm1im1 = T(1.0 / (g.gamma - 1.0) - 1.0);
   ph.rho_floor = T(g.rho_floor);
   ph.p_floor = T(g.p_floor);
   ph.gamma_d = g.gamma;

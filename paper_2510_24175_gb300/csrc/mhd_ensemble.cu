@@ -110,12 +110,14 @@ __device__ __forceinline__ void ens_stage(const EnsArgs& a, unsigned char* smem,
     const int bx = (int)(j % B.ntx);
     const int by = (int)((j / B.ntx) % B.nty);
     const int bz = (int)(j / ((long long)B.ntx * B.nty));
-    // (no interior prefetch: the persistent kernel's registers are capped at
-    // 128 for two CTAs per SM, and the prefetch registers spill there)
-    stage_tile<float, TY, kEnsNW, STAGE, true, false, false, false>(p, sc, bx, by, bz, smem, wmax);
+    stage_tile<float, TY, kEnsNW, STAGE, true>(p, sc, bx, by, bz, smem, wmax);
   }
 }
 
+// 8 warps per CTA, two CTAs per SM: with 12 and 16 warps per CTA (80 and 64
+// registers, the per-box kernel's shape) the persistent kernel, which also keeps
+// a box's parameters, spills 500 bytes a thread and takes 56.0 and 56.6 ms for
+// five steps of 64 boxes against 49.5.
 template <int TY>
 __global__ void __launch_bounds__(kEnsNW * 32, 2) ensemble_kernel(const EnsArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];

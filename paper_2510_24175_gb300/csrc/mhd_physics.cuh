@@ -40,6 +40,7 @@ struct Phys {
   T gamma;      // adiabatic index
   T gm1;        // gamma - 1
   T gm1i;       // 1 / (gamma - 1)
+  T gm1im1;     // 1 / (gamma - 1) - 1
   T rho_floor;
   T p_floor;
   double gamma_d, rho_floor_d, p_floor_d;  // FP64 copies for the floor branch
@@ -329,6 +330,74 @@ MHD_HD long long half_bits(long long b) {
   return (b >> 1) + ((b & 1) & ((b >> 1) & 1));
 }
 
+// -4x and x/2 with IEEE results; FP64 moves the exponent field on the
+// integer pipe (twice_bits / half_bits, exact including subnormals and
+// overflow).
+MHD_HD double neg4(double x) {
+  const long long b = dbits(x), sign = b & (long long)0x8000000000000000ull;
+  return bits2d(twice_bits(twice_bits(b ^ sign)) | (sign ^ (long long)0x8000000000000000ull));
+}
+MHD_HD float neg4(float x) { return -4.0f * x; }
+MHD_HD double half_of(double x) {
+  const long long b = dbits(x), sign = b & (long long)0x8000000000000000ull;
+  return bits2d(half_bits(b ^ sign) | sign);
+}
+MHD_HD float half_of(float x) { return 0.5f * x; }
+
+// x * s for a sign factor s = +1 / -1 given by its sign bit (0, or the top
+// bit of a 64-bit pattern): FP64 flips the sign bit of x on the integer pipe
+// (the product by +-1 is exact, so the result is the same, NaN payloads
+// aside); FP32 negates.
+MHD_HD long long sign_bit_of(bool negative) {
+  return negative ? (long long)0x8000000000000000ull : 0ll;
+}
+MHD_HD double sign_mul(double x, long long sbit) { return bits2d(dbits(x) ^ sbit); }
+
+// Two FP32 values in one register pair.  The packed instructions (FFMA2 / FMUL2
+// / FADD2) do two values' arithmetic in one issue slot, each rounded as the
+// scalar instruction rounds it.
+struct f2 {
+  float2 v;
+  MHD_HD f2() {}
+  MHD_HD f2(float a) : v(make_float2(a, a)) {}
+  MHD_HD f2(float a, float b) : v(make_float2(a, b)) {}
+  MHD_HD explicit f2(float2 a) : v(a) {}
+};
+#if defined(__CUDA_ARCH__) && __CUDA_ARCH__ >= 1000
+MHD_HD f2 fma_rn(f2 a, f2 b, f2 c) { return f2(__ffma2_rn(a.v, b.v, c.v)); }
+MHD_HD f2 mul_rn(f2 a, f2 b) { return f2(__fmul2_rn(a.v, b.v)); }
+MHD_HD f2 operator+(f2 a, f2 b) { return f2(__fadd2_rn(a.v, b.v)); }
+#else
+MHD_HD f2 fma_rn(f2 a, f2 b, f2 c) { return f2(fmaf(a.v.x, b.v.x, c.v.x), fmaf(a.v.y, b.v.y, c.v.y)); }
+MHD_HD f2 mul_rn(f2 a, f2 b) { return f2(mul_rn(a.v.x, b.v.x), mul_rn(a.v.y, b.v.y)); }
+MHD_HD f2 operator+(f2 a, f2 b) { return f2(a.v.x + b.v.x, a.v.y + b.v.y); }
+#endif
+// (a - b is fma(b, -1, a): the product is exact, so it rounds once)
+MHD_HD f2 operator-(f2 a, f2 b) { return fma_rn(b, f2(-1.0f), a); }
+MHD_HD f2 tabs(f2 a) { return f2(fabsf(a.v.x), fabsf(a.v.y)); }
+MHD_HD f2 rcp(f2 a) { return f2(rcp(a.v.x), rcp(a.v.y)); }
+
+// x * (+1 or -1): sign_of(m) is the factor -1 where m holds.  FP64: the sign
+// bit (sign_mul); FP32: a product.
+MHD_HD long long sign_of(bool m, double) { return sign_bit_of(m); }
+MHD_HD float sign_of(bool m, float) { return m ? -1.0f : 1.0f; }
+MHD_HD float sign_mul(float x, float s) { return mul_rn(x, s); }
+
+// Reciprocal and square root inside the Riemann solver.  FP32: the hardware
+// approximations (one instruction each; subnormal operands count as zero).
+MHD_HD double rcp_h(double x) { return rcp(x); }
+MHD_HD double sqrt_h(double x) { return tsqrt(x); }
+MHD_HD float rcp_h(float x) { return seed_rcp(x); }
+MHD_HD float sqrt_h(float x) {
+#ifdef __CUDA_ARCH__
+  float y;
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+#else
+  return sqrtf(x);
+#endif
+}
+
 // Pressure floor.  FP64: plain comparison.  FP32: when the FP32 pressure is
 // within the cancellation-dominated range (internal energy below 1e-3 of the
 // total, or below the floor) p is recomputed in FP64 from the promoted
@@ -361,18 +430,17 @@ MHD_HD float pressure_floor(float p, const float u[kNV], float rho,
 // Conservative -> primitive (step 2 of the stage).  Floors by replacement,
 // density first, then pressure; activations are flagged.
 template <class T>
-MHD_HD void cons_to_prim(const T u[kNV], T v[kNV], const Phys<T>& ph,
-                                             unsigned& flags) {
+MHD_HD void cons_to_prim(const T u[kNV], T v[kNV], const Phys<T>& ph, unsigned& flags) {
   T rho = u[kRHO];
   if (lt_ieee(rho, ph.rho_floor)) {
     rho = ph.rho_floor;
     flags |= kFloorRho;
   }
   const T ri = rcp(rho);
-  const T vx = u[kVX] * ri, vy = u[kVY] * ri, vz = u[kVZ] * ri;
-  const T kin = T(0.5) * dot3_rn(u[kVX], vx, u[kVY], vy, u[kVZ], vz);
+  const T vx = mul_rn(u[kVX], ri), vy = mul_rn(u[kVY], ri), vz = mul_rn(u[kVZ], ri);
+  const T k2 = dot3_rn(u[kVX], vx, u[kVY], vy, u[kVZ], vz);
   const T b2 = dot3_rn(u[kBX], u[kBX], u[kBY], u[kBY], u[kBZ], u[kBZ]);
-  T p = ph.gm1 * (u[kPRS] - kin - T(0.5) * b2);
+  T p = mul_rn(ph.gm1, fma_rn(T(-0.5), b2, fma_rn(T(-0.5), k2, u[kPRS])));
   p = pressure_floor(p, u, rho, ph, flags);
   v[kRHO] = rho;
   v[kVX] = vx;
@@ -402,30 +470,6 @@ MHD_HD void prim_to_cons(const T v[kNV], T u[kNV], const Phys<T>& ph) {
   u[kPSI] = v[kPSI];
 }
 
-// -4x and x/2 with IEEE results; FP64 moves the exponent field on the
-// integer pipe (twice_bits / half_bits, exact including subnormals and
-// overflow).
-MHD_HD double neg4(double x) {
-  const long long b = dbits(x), sign = b & (long long)0x8000000000000000ull;
-  return bits2d(twice_bits(twice_bits(b ^ sign)) | (sign ^ (long long)0x8000000000000000ull));
-}
-MHD_HD float neg4(float x) { return -4.0f * x; }
-MHD_HD double half_of(double x) {
-  const long long b = dbits(x), sign = b & (long long)0x8000000000000000ull;
-  return bits2d(half_bits(b ^ sign) | sign);
-}
-MHD_HD float half_of(float x) { return 0.5f * x; }
-
-// x * s for a sign factor s = +1 / -1 given by its sign bit (0, or the top
-// bit of a 64-bit pattern): FP64 flips the sign bit of x on the integer pipe
-// (the product by +-1 is exact, so the result is the same, NaN payloads
-// aside); FP32 negates.
-MHD_HD long long sign_bit_of(bool negative) {
-  return negative ? (long long)0x8000000000000000ull : 0ll;
-}
-MHD_HD double sign_mul(double x, long long sbit) { return bits2d(dbits(x) ^ sbit); }
-MHD_HD float sign_mul(float x, long long sbit) { return sbit ? -x : x; }
-
 // Twice the fast magnetosonic speed squared from 1/rho, gamma p, |B|^2 and
 // B_n^2: with g = gamma p / rho, a = g + |B|^2 / rho and c_an^2 = B_n^2 / rho,
 // 2 c_f^2 = a + sqrt(a^2 - 4 g c_an^2).
@@ -433,27 +477,28 @@ template <class T>
 MHD_HD T fast_speed2x(T rho_i, T gp, T b2, T bn2) {
   const T g = mul_rn(gp, rho_i);
   const T a = fma_rn(b2, rho_i, g);
-  return a + tsqrt(pos_part(fma_rn(a, a, neg4(g * (bn2 * rho_i)))));
+  return a + sqrt_h(pos_part(fma_rn(a, a, neg4(mul_rn(g, mul_rn(bn2, rho_i))))));
 }
 
 // Fast magnetosonic speed (see fast_speed2x).
 template <class T>
 MHD_HD T fast_speed(T rho_i, T gp, T b2, T bn2) {
-  return tsqrt(half_of(fast_speed2x(rho_i, gp, b2, bn2)));
+  return sqrt_h(half_of(fast_speed2x(rho_i, gp, b2, bn2)));
 }
 
 // max over active directions of |v_d| + c_f,d for one conservative cell.
 template <class T>
-MHD_HD T cell_max_speed(const T u[kNV], const Phys<T>& ph, int ndim,
-                                            unsigned& flags) {
+MHD_HD T cell_max_speed(const T u[kNV], const Phys<T>& ph, int ndim, unsigned& flags) {
   T v[kNV];
   cons_to_prim(u, v, ph, flags);
   const T ri = rcp(v[kRHO]);
-  const T gp = ph.gamma * v[kPRS];
+  const T gp = mul_rn(ph.gamma, v[kPRS]);
   const T b2 = dot3_rn(v[kBX], v[kBX], v[kBY], v[kBY], v[kBZ], v[kBZ]);
-  T lam = tabs(v[kVX]) + fast_speed(ri, gp, b2, v[kBX] * v[kBX]);
-  if (ndim > 1) lam = nan_max(lam, tabs(v[kVY]) + fast_speed(ri, gp, b2, v[kBY] * v[kBY]));
-  if (ndim > 2) lam = nan_max(lam, tabs(v[kVZ]) + fast_speed(ri, gp, b2, v[kBZ] * v[kBZ]));
+  T lam = tabs(v[kVX]) + fast_speed(ri, gp, b2, mul_rn(v[kBX], v[kBX]));
+  if (ndim > 1)
+    lam = nan_max(lam, tabs(v[kVY]) + fast_speed(ri, gp, b2, mul_rn(v[kBY], v[kBY])));
+  if (ndim > 2)
+    lam = nan_max(lam, tabs(v[kVZ]) + fast_speed(ri, gp, b2, mul_rn(v[kBZ], v[kBZ])));
   // NaN anywhere in the cell (psi included) makes the speed NaN
   if (is_nan(v[kPSI]) || is_nan(lam)) lam = T(NAN);
   return lam;
@@ -613,34 +658,52 @@ MHD_HD double limited_slope<double>(double dm, double dp, int lim) {
   return bits2d(mb | (a & ~mask));
 }
 
-// PLM face states around one interface from four consecutive cells q0..q3
-// (the interface lies between q1 and q2).  c[j] points at variable 0 of cell
-// j; variables are vstride apart.  Writes the left state (from q1) and the
-// right state (from q2).
-template <class T>
-MHD_HD void plm_face_pair(const T* c0, const T* c1, const T* c2,
-                                              const T* c3, int vstride, int lim, T vl[kNV],
-                                              T vr[kNV]) {
-  T s1[kNV], s2[kNV];
-#pragma unroll
-  for (int k = 0; k < kNV; ++k) {
-    const T q0 = c0[k * vstride], q1 = c1[k * vstride], q2 = c2[k * vstride],
-            q3 = c3[k * vstride];
-    s1[k] = limited_slope(q1 - q0, q2 - q1, lim);
-    s2[k] = limited_slope(q2 - q1, q3 - q2, lim);
-    vl[k] = q1;
-    vr[k] = q2;
-  }
-  // zero-slope fallback per cell if a face density or pressure is <= 0
-  const bool ok1 = gt0(vl[kRHO] - T(0.5) * tabs(s1[kRHO])) &&
-                   gt0(vl[kPRS] - T(0.5) * tabs(s1[kPRS]));
-  const bool ok2 = gt0(vr[kRHO] - T(0.5) * tabs(s2[kRHO])) &&
-                   gt0(vr[kPRS] - T(0.5) * tabs(s2[kPRS]));
-#pragma unroll
-  for (int k = 0; k < kNV; ++k) {
-    if (ok1) vl[k] = vl[k] + T(0.5) * s1[k];
-    if (ok2) vr[k] = vr[k] - T(0.5) * s2[k];
-  }
+// Half the limited slope, the step from the cell value to its faces: MC
+// min(|dm|, |dp|, |dm+dp|/4), minmod min(|dm|, |dp|)/2, with the common sign, 0
+// when the signs differ.  FP32: with the central value c between dm and dp, the
+// smallest of the three where it is positive, the largest where it is negative.
+MHD_HD float min3(float a, float b, float c) {
+#if defined(__CUDA_ARCH__) && __CUDA_ARCH__ >= 1000
+  float d;
+  asm("min.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
+#else
+  return fminf(fminf(a, b), c);
+#endif
+}
+MHD_HD float max3(float a, float b, float c) {
+#if defined(__CUDA_ARCH__) && __CUDA_ARCH__ >= 1000
+  float d;
+  asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
+#else
+  return fmaxf(fmaxf(a, b), c);
+#endif
+}
+MHD_HD float half_slope_mc(float dm, float dp) {
+  const float c = mul_rn(0.25f, dm + dp);
+  return fmaxf(min3(dm, dp, c), 0.0f) + fminf(max3(dm, dp, c), 0.0f);
+}
+MHD_HD float half_slope_minmod(float dm, float dp) {
+  return mul_rn(0.5f, fmaxf(fminf(dm, dp), 0.0f) + fminf(fmaxf(dm, dp), 0.0f));
+}
+// FP64: the same value as half of limited_slope, decided and scaled on the
+// integer pipe; |dm| + |dp| is the only FP64 operation.
+MHD_HD double half_slope_mc(double dm, double dp) {
+  const long long a = dbits(dm), b = dbits(dp);
+  const long long mask = 0x7fffffffffffffffll;
+  const long long am = a & mask, bm = b & mask;
+  const long long mb = am < bm ? am : bm;
+  const long long qr = half_bits(half_bits(dbits(bits2d(am) + bits2d(bm))));
+  const long long h = (qr < mb ? qr : mb) | (a & ~mask);
+  return (a ^ b) < 0 || am == 0 || bm == 0 ? 0.0 : bits2d(h);
+}
+MHD_HD double half_slope_minmod(double dm, double dp) {
+  const long long a = dbits(dm), b = dbits(dp);
+  const long long mask = 0x7fffffffffffffffll;
+  const long long am = a & mask, bm = b & mask;
+  const long long h = half_bits(am < bm ? am : bm) | (a & ~mask);
+  return (a ^ b) < 0 || am == 0 || bm == 0 ? 0.0 : bits2d(h);
 }
 
 // Picks component (dir + j) % 3 of a 3-vector given as scalars (dir is a
@@ -650,167 +713,6 @@ MHD_HD T rot3(int dir, int j, T a, T b, T c) {
   const int m = (dir + j) % 3;
   return m == 0 ? a : (m == 1 ? b : c);
 }
-
-#if defined(__CUDA_ARCH__) && __CUDA_ARCH__ >= 1000
-// Packed FP32 (FFMA2 / FMUL2 / FADD2: two lanes per instruction, each lane
-// rounded as the scalar instruction).  x - y is fma(y, -1, x): the product is
-// exact, so it rounds once, as a subtraction does.
-__device__ __forceinline__ float2 pk(float a, float b) { return make_float2(a, b); }
-__device__ __forceinline__ float2 pk1(float a) { return make_float2(a, a); }
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
-__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 sub2(float2 a, float2 b) {
-  return __ffma2_rn(b, make_float2(-1.0f, -1.0f), a);
-}
-__device__ __forceinline__ float2 swap2(float2 a) { return make_float2(a.y, a.x); }
-
-// FP32 GLM + HLLD (the same steps as glm_hlld_flux) with the two sides'
-// identical operations -- outer states, fast speeds, single-star states --
-// and the two tangential components' ones -- double-star states, flux
-// terms -- paired in packed instructions: .x the left state (or the first
-// tangential component), .y the right one (or the second).  Every operation
-// is written out (no contraction is left to the compiler), so the flux rounds
-// the same in every kernel it is inlined into.
-template <int dir>
-__device__ __forceinline__ void glm_hlld_flux_f32x2(const float vl[kNV], const float vr[kNV],
-                                                    float ch, float half_chi,
-                                                    const Phys<float>& ph, float F[kNV]) {
-  const float2 H = pk1(0.5f);
-  const float2 u = pk(rot3(dir, 0, vl[kVX], vl[kVY], vl[kVZ]), rot3(dir, 0, vr[kVX], vr[kVY], vr[kVZ]));
-  const float2 v = pk(rot3(dir, 1, vl[kVX], vl[kVY], vl[kVZ]), rot3(dir, 1, vr[kVX], vr[kVY], vr[kVZ]));
-  const float2 w = pk(rot3(dir, 2, vl[kVX], vl[kVY], vl[kVZ]), rot3(dir, 2, vr[kVX], vr[kVY], vr[kVZ]));
-  const float2 by = pk(rot3(dir, 1, vl[kBX], vl[kBY], vl[kBZ]), rot3(dir, 1, vr[kBX], vr[kBY], vr[kBZ]));
-  const float2 bz = pk(rot3(dir, 2, vl[kBX], vl[kBY], vl[kBZ]), rot3(dir, 2, vr[kBX], vr[kBY], vr[kBZ]));
-  const float bnL = rot3(dir, 0, vl[kBX], vl[kBY], vl[kBZ]);
-  const float bnR = rot3(dir, 0, vr[kBX], vr[kBY], vr[kBZ]);
-  const float2 r = pk(vl[kRHO], vr[kRHO]), p = pk(vl[kPRS], vr[kPRS]);
-
-  // GLM: exact solution of the linear (B_n, psi) interface problem
-  const float bx = fmaf(0.5f, __fadd_rn(bnL, bnR), -__fmul_rn(half_chi, __fsub_rn(vr[kPSI], vl[kPSI])));
-  const float psis = fmaf(0.5f, __fadd_rn(vl[kPSI], vr[kPSI]),
-                          -__fmul_rn(__fmul_rn(0.5f, ch), __fsub_rn(bnR, bnL)));
-  const float bx2 = __fmul_rn(bx, bx);
-  const float2 BX = pk1(bx), BX2 = pk1(bx2);
-
-  // outer states
-  const float2 b2 = fma2(bz, bz, fma2(by, by, BX2));
-  const float2 pt = fma2(H, b2, p);
-  const float2 vv = fma2(w, w, fma2(v, v, mul2(u, u)));
-  const float2 e = fma2(H, b2, fma2(mul2(H, r), vv, mul2(p, pk1(ph.gm1i))));
-  // 1/rho of both sides from one reciprocal; fast speeds squared
-  const float qr = rcp(__fmul_rn(r.x, r.y));
-  const float2 ri = mul2(swap2(r), pk1(qr));
-  const float2 gp = mul2(pk1(ph.gamma), p);
-  const float2 g = mul2(gp, ri);
-  const float2 a = fma2(b2, ri, g);
-  const float2 disc2 = fma2(a, a, mul2(pk1(-4.0f), mul2(g, mul2(BX2, ri))));
-  const float dL = fmaxf(disc2.x, 0.0f), dR = fmaxf(disc2.y, 0.0f);
-  const float2 dsc = pk(dL, dR);
-  const float2 rq = pk(dL > 0.0f ? rsqrtf(dL) : 0.0f, dR > 0.0f ? rsqrtf(dR) : 0.0f);
-  const float2 cf2 = mul2(H, fma2(dsc, rq, a));
-  // wave-speed estimates, contact speed and total pressure
-  const float c2m = fmaxf(cf2.x, cf2.y);
-  const float cmax = c2m > 0.0f ? __fmul_rn(c2m, rsqrtf(c2m)) : 0.0f;
-  const float2 S = add2(pk(fminf(u.x, u.y), fmaxf(u.x, u.y)), pk(-cmax, cmax));
-  const float2 Su = sub2(S, u);
-  const float2 d = mul2(Su, r);
-  const float Di = rcp(__fsub_rn(d.y, d.x));
-  const float SM =
-      __fmul_rn(__fadd_rn(__fsub_rn(fmaf(d.y, u.y, -__fmul_rn(d.x, u.x)), pt.y), pt.x), Di);
-  const float pts = __fmul_rn(fmaf(__fmul_rn(d.x, d.y), __fsub_rn(u.y, u.x),
-                                   fmaf(d.y, pt.x, -__fmul_rn(d.x, pt.y))), Di);
-  const float2 SMv = pk1(SM);
-
-  // single-star states, degenerate when |rho (S-u)(S-S_M) - Bx^2| < 1e-8 p_t*;
-  // paired reciprocals of S-S_M and of the two denominators
-  const float2 sm = sub2(S, SMv);
-  const float2 den = fma2(d, sm, pk1(-bx2));
-  const float thr = __fmul_rn(1e-8f, pts);
-  const bool degL = fabsf(den.x) < thr, degR = fabsf(den.y) < thr;
-  const float2 dn = pk(degL ? 1.0f : den.x, degR ? 1.0f : den.y);
-  const float ps = __fmul_rn(sm.x, sm.y), pd = __fmul_rn(dn.x, dn.y);
-  const float q4 = rcp(__fmul_rn(ps, pd));
-  const float qs = __fmul_rn(pd, q4), qd = __fmul_rn(ps, q4);
-  const float2 smi = mul2(swap2(sm), pk1(qs));
-  const float2 deni = mul2(swap2(dn), pk1(qd));
-  const float2 rs = mul2(d, smi);
-  const float2 fv = mul2(mul2(BX, sub2(SMv, u)), deni);
-  const float2 fb = mul2(fma2(d, Su, pk1(-bx2)), deni);
-  const float2 vs0 = fma2(pk(-by.x, -by.y), fv, v), ws0 = fma2(pk(-bz.x, -bz.y), fv, w);
-  const float2 bys0 = mul2(by, fb), bzs0 = mul2(bz, fb);
-  const float2 vs = pk(degL ? v.x : vs0.x, degR ? v.y : vs0.y);
-  const float2 ws = pk(degL ? w.x : ws0.x, degR ? w.y : ws0.y);
-  const float2 bys = pk(degL ? by.x : bys0.x, degR ? by.y : bys0.y);
-  const float2 bzs = pk(degL ? bz.x : bzs0.x, degR ? bz.y : bzs0.y);
-  const float2 vb = fma2(w, bz, fma2(v, by, mul2(u, BX)));
-  const float2 vbs = fma2(ws, bzs, fma2(vs, bys, mul2(SMv, BX)));
-  const float2 es = mul2(fma2(BX, sub2(vb, vbs),
-                              fma2(pk1(pts), SMv, fma2(Su, e, pk(-__fmul_rn(pt.x, u.x),
-                                                                 -__fmul_rn(pt.y, u.y))))),
-                         smi);
-
-  // fan region: side a = L if (S_L > 0) or (S_R >= 0 and S_M >= 0), else R
-  const bool sup = S.x > 0.0f || S.y < 0.0f;
-  const bool useL = S.x > 0.0f || (!(S.y < 0.0f) && SM >= 0.0f);
-  const float ra = useL ? r.x : r.y, ua = useL ? u.x : u.y;
-  const float2 vw = useL ? pk(v.x, w.x) : pk(v.y, w.y);
-  const float2 bb = useL ? pk(by.x, bz.x) : pk(by.y, bz.y);
-  const float ea = useL ? e.x : e.y, pta = useL ? pt.x : pt.y;
-  const float rsa = useL ? rs.x : rs.y, esa = useL ? es.x : es.y;
-  const float2 vws = useL ? pk(vs.x, ws.x) : pk(vs.y, ws.y);
-  const float2 bbs = useL ? pk(bys.x, bzs.x) : pk(bys.y, bzs.y);
-  const float vbsa = useL ? vbs.x : vbs.y, vba = useL ? vb.x : vb.y;
-  const float c1 = sup ? 0.0f : (useL ? S.x : S.y);
-  const float2 C1 = pk1(c1), UA = pk1(ua);
-  // flux of the outer state plus the single-star jump
-  const float ru = __fmul_rn(ra, ua);
-  const float2 rvw = mul2(pk1(ra), vw);
-  float f0 = fmaf(c1, __fsub_rn(rsa, ra), ru);
-  float f1 = fmaf(c1, fmaf(rsa, SM, -ru), __fsub_rn(fmaf(ru, ua, pta), bx2));
-  float2 f23 = fma2(C1, fma2(pk1(rsa), vws, pk(-rvw.x, -rvw.y)),
-                    fma2(rvw, UA, pk(-__fmul_rn(bx, bb.x), -__fmul_rn(bx, bb.y))));
-  float2 f45 = fma2(C1, sub2(bbs, bb), fma2(bb, UA, pk(-__fmul_rn(bx, vw.x), -__fmul_rn(bx, vw.y))));
-  float f6 = fmaf(c1, __fsub_rn(esa, ea), fmaf(__fadd_rn(ea, pta), ua, -__fmul_rn(bx, vba)));
-
-  // Alfven waves and double-star states; 1/sqrt(rho*) by rsqrt
-  const float2 iq = pk(rsqrtf(rs.x), rsqrtf(rs.y));
-  const float2 sq = mul2(rs, iq);
-  const float abx = fabsf(bx);
-  const float2 Ss = fma2(pk(-abx, abx), iq, SMv);  // (S_L*, S_R*)
-  const float sg = bx >= 0.0f ? 1.0f : -1.0f;
-  const float isum = rcp(__fadd_rn(sq.x, sq.y));
-  const float sqLR = __fmul_rn(sq.x, sq.y);
-  const float2 SG = pk1(sg), IS = pk1(isum), SQL = pk1(sq.x), SQR = pk1(sq.y);
-  // (v**, w**) and (By**, Bz**)
-  const float2 vwR = pk(vs.y, ws.y), vwL = pk(vs.x, ws.x);
-  const float2 bbR = pk(bys.y, bzs.y), bbL = pk(bys.x, bzs.x);
-  const float2 vwss = mul2(fma2(sub2(bbR, bbL), SG, fma2(SQR, vwR, mul2(SQL, vwL))), IS);
-  const float2 bbss = mul2(fma2(pk1(sqLR), mul2(sub2(vwR, vwL), SG), fma2(SQR, bbL, mul2(SQL, bbR))), IS);
-  const float vbss = fmaf(vwss.y, bbss.y, fmaf(vwss.x, bbss.x, __fmul_rn(SM, bx)));
-
-  // inside the Alfven fan: c2 = S*_a
-  const bool inner = !sup && (useL ? !(Ss.x > 0.0f) : !(Ss.y < 0.0f));
-  const float sqa = useL ? -sq.x : sq.y;
-  const float ess = fmaf(sqa, __fmul_rn(__fsub_rn(vbsa, vbss), sg), esa);
-  const float c2 = inner ? (useL ? Ss.x : Ss.y) : 0.0f;
-  const float c2rs = __fmul_rn(c2, rsa);
-  f23 = fma2(pk1(c2rs), sub2(vwss, vws), f23);
-  f45 = fma2(pk1(c2), sub2(bbss, bbs), f45);
-  f6 = fmaf(c2, __fsub_rn(ess, esa), f6);
-
-  F[kRHO] = f0;
-  F[kPRS] = f6;
-  F[kPSI] = __fmul_rn(__fmul_rn(ch, ch), bx);
-  // un-rotate: component m gets rotated slot j = (m - dir) mod 3
-#pragma unroll
-  for (int m = 0; m < 3; ++m) {
-    const int j = (m - dir + 3) % 3;
-    F[kVX + m] = j == 0 ? f1 : (j == 1 ? f23.x : f23.y);
-    F[kBX + m] = j == 0 ? psis : (j == 1 ? f45.x : f45.y);
-  }
-}
-#endif
 
 // GLM interface step + HLLD along direction dir (0, 1, 2; template
 // argument) for primitive face states vl, vr.  ch: cleaning speed;
@@ -829,12 +731,6 @@ __device__ __forceinline__ void glm_hlld_flux_f32x2(const float vl[kNV], const f
 template <int dir, class T>
 MHD_HD void glm_hlld_flux(const T vl[kNV], const T vr[kNV], T ch, T half_chi,
                           const Phys<T>& ph, T F[kNV]) {
-#if defined(__CUDA_ARCH__) && __CUDA_ARCH__ >= 1000
-  if constexpr (sizeof(T) == 4) {  // FP32 on the device: the packed form
-    glm_hlld_flux_f32x2<dir>(vl, vr, ch, half_chi, ph, F);
-    return;
-  }
-#endif
   const T half = T(0.5);
   // rotate: u normal, (v, w) tangential in cyclic order; by, bz likewise
   const T uL = rot3(dir, 0, vl[kVX], vl[kVY], vl[kVZ]);
@@ -852,18 +748,19 @@ MHD_HD void glm_hlld_flux(const T vl[kNV], const T vr[kNV], T ch, T half_chi,
   const T rL = vl[kRHO], pL = vl[kPRS], rR = vr[kRHO], pR = vr[kPRS];
 
   // GLM: exact solution of the linear (B_n, psi) interface problem
-  const T bx = fma_rn(half, bnL + bnR, -mul_rn(half_chi, vr[kPSI] - vl[kPSI]));
-  const T psis = fma_rn(half, vl[kPSI] + vr[kPSI], -mul_rn(half * ch, bnR - bnL));
+  const T bx = fma_rn(half, bnL + bnR, mul_rn(-half_chi, vr[kPSI] - vl[kPSI]));
+  const T psis = fma_rn(half, vl[kPSI] + vr[kPSI], mul_rn(T(-0.5) * ch, bnR - bnL));
   const T bx2 = mul_rn(bx, bx);
+  const T nbx = -bx, nbx2 = -bx2;
 
   // total pressures; c_max, the larger fast speed: one square root of the
   // larger c_f^2 (sqrt is monotone)
   const T b2L = fma_rn(bzL, bzL, fma_rn(byL, byL, bx2));
   const T b2R = fma_rn(bzR, bzR, fma_rn(byR, byR, bx2));
   const T ptL = fma_rn(half, b2L, pL), ptR = fma_rn(half, b2R, pR);
-  const T cf2L = fast_speed2x(rcp(rL), mul_rn(ph.gamma, pL), b2L, bx2);
-  const T cf2R = fast_speed2x(rcp(rR), mul_rn(ph.gamma, pR), b2R, bx2);
-  const T cmax = tsqrt(half_of(tmax2(cf2L, cf2R)));
+  const T cf2L = fast_speed2x(rcp_h(rL), mul_rn(ph.gamma, pL), b2L, bx2);
+  const T cf2R = fast_speed2x(rcp_h(rR), mul_rn(ph.gamma, pR), b2R, bx2);
+  const T cmax = sqrt_h(half_of(tmax2(cf2L, cf2R)));
 
   // wave-speed estimates (MK05 Eq. 67) and contact speed (Eq. 38, written as
   // u_L plus a correction)
@@ -871,50 +768,49 @@ MHD_HD void glm_hlld_flux(const T vl[kNV], const T vr[kNV], T ch, T half_chi,
   const T SR = tmax2(uL, uR) + cmax;
   const T SuL = SL - uL, SuR = SR - uR;
   const T dL = mul_rn(SuL, rL), dR = mul_rn(SuR, rR);
-  const T SM = fma_rn(fma_rn(dR, uR - uL, ptL - ptR), rcp(dR - dL), uL);
+  const T SM0 = fma_rn(fma_rn(dR, uR - uL, ptL - ptR), rcp_h(dR - dL), uL);
 
   // The upwind side a: L if (S_L > 0) or (S_R >= 0 and S_M >= 0), else R
   // (sign tests on the integer pipe in FP64: gt0 / lt0 / ge0); o: the other
-  // side, which enters only through the double-star states.
+  // side, which enters only through the double-star states.  Where the flow is
+  // supersonic the interface takes side a's outer state: S_M = u there makes
+  // the star state below the outer one (rho and E are selected: their
+  // quotients round).
   const bool sup = gt0(SL) || lt0(SR);
-  const bool useL = gt0(SL) || (!lt0(SR) && ge0(SM));
-  const T r = useL ? rL : rR, u = useL ? uL : uR, v = useL ? vL : vR, w = useL ? wL : wR;
-  const T by = useL ? byL : byR, bz = useL ? bzL : bzR, b2 = useL ? b2L : b2R;
+  const bool useL = gt0(SL) || (!lt0(SR) && ge0(SM0));
+  const T r = useL ? rL : rR, u = useL ? uL : uR;
+  const T v = useL ? vL : vR, w = useL ? wL : wR;
+  const T by = useL ? byL : byR, bz = useL ? bzL : bzR;
   const T p = useL ? pL : pR, pt = useL ? ptL : ptR;
   const T S = useL ? SL : SR, Su = useL ? SuL : SuR, d = useL ? dL : dR;
+  const T SM = sup ? u : SM0;
 
-  // single-star state of side a (MK05 Eqs. 43-48), degenerate when
-  // den = rho (S-u)(S-S_M) - Bx^2 is below 1e-8 p_t*; p_t* = p_t + rho (S-u)
-  // (S_M-u); B* = B (1 + rho (S-u)(S_M-u) / den); one reciprocal for the two
-  // divisors
+  // single-star state of side a (MK05 Eqs. 43-48), degenerate (v*, B* equal to
+  // the outer state) when |den| < 1e-8 p_t*, den = rho (S-u)(S-S_M) - Bx^2;
+  // p_t* = p_t + rho (S-u)(S_M-u), B* = B (1 + rho (S-u)(S_M-u) / den); one
+  // reciprocal for the two divisors
   const T du = SM - u;
   const T pts = fma_rn(d, du, pt);
   const T sm = S - SM;
-  const T den = fma_rn(d, sm, -bx2);
-  const bool deg = abs_lt(den, mul_rn(T(1e-8), pts));
+  const T den = fma_rn(d, sm, nbx2);
+  const T thr = mul_rn(T(1e-8), pts);
+  const bool deg = abs_lt(den, thr);
   const T dn = deg ? T(1) : den;
-  const T q = rcp(mul_rn(sm, dn));
-  const T smi = mul_rn(dn, q), deni = mul_rn(sm, q);
-  const T rs = mul_rn(d, smi);
-  const T k0 = mul_rn(du, deni);
-  const T fv = mul_rn(bx, k0), fb = mul_rn(d, k0);
-  const T vs = deg ? v : fma_rn(-by, fv, v);
-  const T ws = deg ? w : fma_rn(-bz, fv, w);
-  const T bys = deg ? by : fma_rn(by, fb, by);
-  const T bzs = deg ? bz : fma_rn(bz, fb, bz);
+  const T q = rcp_h(mul_rn(sm, dn));
+  const T smi = mul_rn(dn, q);
+  const T rs = sup ? r : mul_rn(d, smi);
+  const T k0 = deg ? T(0) : mul_rn(du, mul_rn(sm, q));
+  const T fv = mul_rn(nbx, k0), fb = mul_rn(d, k0);
+  const T vs = fma_rn(by, fv, v), ws = fma_rn(bz, fv, w);
+  const T bys = fma_rn(by, fb, by), bzs = fma_rn(bz, fb, bz);
   const T vb = dot3_rn(u, bx, v, by, w, bz);
   const T vbs = dot3_rn(SM, bx, vs, bys, ws, bzs);
-  // (rho / 2 by half_of: an exponent move in FP64, the same value as 0.5 * rho)
-  const T e = fma_rn(half, b2, fma_rn(half_of(r), dot3_rn(u, u, v, v, w, w), mul_rn(p, ph.gm1i)));
-  const T es = mul_rn(fma_rn(bx, vb - vbs,
-                             fma_rn(pts, SM, fma_rn(Su, e, -mul_rn(pt, u)))), smi);
-
-  // The state on the interface: outer where the flow is supersonic, else
-  // single-star, else (below) double-star.
-  const T rF = sup ? r : rs, uF = sup ? u : SM, ptF = sup ? pt : pts;
-  const T ru = mul_rn(rF, uF);
-  T vF = sup ? v : vs, wF = sup ? w : ws, byF = sup ? by : bys, bzF = sup ? bz : bzs;
-  T eF = sup ? e : es, vbF = sup ? vb : vbs;
+  // E = rho v^2 / 2 + p / (gamma-1) + B^2 / 2, the last two from p_t; E* (S-S_M)
+  // = (S-u) E + (p_t* S_M - p_t u) + Bx (v.B - v*.B*).  (rho / 2 by half_of: an
+  // exponent move in FP64, the same value as 0.5 * rho)
+  const T e = fma_rn(half_of(r), dot3_rn(u, u, v, v, w, w), fma_rn(p, ph.gm1im1, pt));
+  const T ns = fma_rn(bx, vb - vbs, fma_rn(Su, e, mul_rn(du, fma_rn(d, SM, pt))));
+  const T es = sup ? e : mul_rn(ns, smi);
 
   // Inside the Alfven fan (S*_L <= 0 <= S*_R, Eq. 51: rho* S_M^2 <= B_x^2) the
   // double-star states (Eqs. 59-63).  With s = sign(B_x) on side L and
@@ -922,26 +818,25 @@ MHD_HD void glm_hlld_flux(const T vl[kNV], const T vr[kNV], T ch, T half_chi,
   // of side a: v** = v* + X, B** = B* + s sqrt(rho*) X, X = (sqrt(rho*_o)
   // (v*_o - v*) + s (B*_o - B*)) / (sqrt(rho*) + sqrt(rho*_o)).  Skipped where
   // no lane of the warp is inside the fan.
+  const T ru = mul_rn(rs, SM);
+  T vF = vs, wF = ws, byF = bys, bzF = bzs, eF = es, vbF = vbs;
   if (!sup && !lt_ieee(bx2, mul_rn(ru, SM))) {
     const T uo = useL ? uR : uL, vo = useL ? vR : vL, wo = useL ? wR : wL;
     const T byo = useL ? byR : byL, bzo = useL ? bzR : bzL;
     const T So = useL ? SR : SL, dO = useL ? dR : dL;
     const T smo = So - SM;
-    const T deno = fma_rn(dO, smo, -bx2);
-    const bool dego = abs_lt(deno, mul_rn(T(1e-8), pts));
+    const T deno = fma_rn(dO, smo, nbx2);
+    const bool dego = abs_lt(deno, thr);
     const T dno = dego ? T(1) : deno;
-    const T qo = rcp(mul_rn(smo, dno));
-    const T denio = mul_rn(smo, qo);
+    const T qo = rcp_h(mul_rn(smo, dno));
     const T rso = mul_rn(dO, mul_rn(dno, qo));
-    const T k0o = mul_rn(SM - uo, denio);
-    const T fvo = mul_rn(bx, k0o), fbo = mul_rn(dO, k0o);
-    const T vso = dego ? vo : fma_rn(-byo, fvo, vo);
-    const T wso = dego ? wo : fma_rn(-bzo, fvo, wo);
-    const T byso = dego ? byo : fma_rn(byo, fbo, byo);
-    const T bzso = dego ? bzo : fma_rn(bzo, fbo, bzo);
-    const T sqa = tsqrt(rs), sqo = tsqrt(rso);
-    const T isum = rcp(sqa + sqo);
-    const long long sg = sign_bit_of(ge0(bx) != useL);
+    const T k0o = dego ? T(0) : mul_rn(SM - uo, mul_rn(smo, qo));
+    const T fvo = mul_rn(nbx, k0o), fbo = mul_rn(dO, k0o);
+    const T vso = fma_rn(byo, fvo, vo), wso = fma_rn(bzo, fvo, wo);
+    const T byso = fma_rn(byo, fbo, byo), bzso = fma_rn(bzo, fbo, bzo);
+    const T sqa = sqrt_h(rs), sqo = sqrt_h(rso);
+    const T isum = rcp_h(sqa + sqo);
+    const auto sg = sign_of(ge0(bx) != useL, T(0));
     const T Xv = mul_rn(fma_rn(sqo, vso - vs, sign_mul(byso - bys, sg)), isum);
     const T Xw = mul_rn(fma_rn(sqo, wso - ws, sign_mul(bzso - bzs, sg)), isum);
     const T sqs = sign_mul(sqa, sg);
@@ -958,28 +853,25 @@ MHD_HD void glm_hlld_flux(const T vl[kNV], const T vr[kNV], T ch, T half_chi,
   // flux of the state on the interface with normal velocity S_M and total
   // pressure p_t* -- except the induction terms of a degenerate star state,
   // which keeps B* = B: there B (u - S_M) is left over.
-  T f[7];
-  f[0] = ru;
-  f[1] = fma_rn(ru, uF, ptF - bx2);
-  f[2] = fma_rn(ru, vF, -mul_rn(bx, byF));
-  f[3] = fma_rn(ru, wF, -mul_rn(bx, bzF));
-  f[4] = fma_rn(byF, uF, -mul_rn(bx, vF));
-  f[5] = fma_rn(bzF, uF, -mul_rn(bx, wF));
-  f[6] = fma_rn(eF + ptF, uF, -mul_rn(bx, vbF));
-  if (deg && !sup) {
-    f[4] = fma_rn(-by, du, f[4]);
-    f[5] = fma_rn(-bz, du, f[5]);
+  const T f1 = fma_rn(ru, SM, pts + nbx2);
+  const T f2 = fma_rn(ru, vF, mul_rn(nbx, byF));
+  const T f3 = fma_rn(ru, wF, mul_rn(nbx, bzF));
+  T f4 = fma_rn(byF, SM, mul_rn(nbx, vF));
+  T f5 = fma_rn(bzF, SM, mul_rn(nbx, wF));
+  if (deg) {
+    f4 = fma_rn(-by, du, f4);
+    f5 = fma_rn(-bz, du, f5);
   }
 
-  F[kRHO] = f[0];
-  F[kPRS] = f[6];
-  F[kPSI] = ch * ch * bx;
+  F[kRHO] = ru;
+  F[kPRS] = fma_rn(eF + pts, SM, mul_rn(nbx, vbF));
+  F[kPSI] = mul_rn(mul_rn(ch, ch), bx);
   // un-rotate: component m of a vector gets rotated slot j = (m - dir) mod 3
 #pragma unroll
   for (int m = 0; m < 3; ++m) {
     const int j = (m - dir + 3) % 3;
-    F[kVX + m] = j == 0 ? f[1] : (j == 1 ? f[2] : f[3]);
-    F[kBX + m] = j == 0 ? psis : (j == 1 ? f[4] : f[5]);
+    F[kVX + m] = j == 0 ? f1 : (j == 1 ? f2 : f3);
+    F[kBX + m] = j == 0 ? psis : (j == 1 ? f4 : f5);
   }
 }
 

@@ -154,9 +154,9 @@ struct CtCell {
   __device__ __forceinline__ void from_prims(const T* v, int st) {
     const T vx = v[kVX * st], vy = v[kVY * st], vz = v[kVZ * st];
     const T bx = v[kBX * st], by = v[kBY * st], bz = v[kBZ * st];
-    ex = vz * by - vy * bz;
-    ey = vx * bz - vz * bx;
-    ez = vy * bx - vx * by;
+    ex = fma_rn(vz, by, -mul_rn(vy, bz));
+    ey = fma_rn(vx, bz, -mul_rn(vz, bx));
+    ez = fma_rn(vy, bx, -mul_rn(vx, by));
     rho = v[kRHO * st];
   }
   // fx / fy: the x and y fluxes of the cell's lower faces (variables sx / sy
@@ -236,69 +236,37 @@ struct TileGeom {
   static constexpr int ITEMS = IT_X + IT_Y + IT_XE;
 };
 
-#if defined(__CUDA_ARCH__) && __CUDA_ARCH__ >= 1000
-// FP32 limited slopes of two variables at once: the one-sided differences,
-// their product, the doubled minimum and the halved sum in packed FP32; the
-// per-lane comparisons, minima and sign choices as limited_slope<float>
-// takes them (the same values).
-__device__ __forceinline__ float2 limited_slope2(float2 dm, float2 dp, int lim) {
-  const float2 pr = mul2(dm, dp);
-  float2 mag = pk(fminf(fabsf(dm.x), fabsf(dp.x)), fminf(fabsf(dm.y), fabsf(dp.y)));
-  if (lim == kLimMC) {
-    const float2 two = mul2(pk1(2.0f), mag);
-    const float2 sum = add2(dm, dp);
-    const float2 cen = mul2(pk1(0.5f), pk(fabsf(sum.x), fabsf(sum.y)));
-    mag = pk(fminf(two.x, cen.x), fminf(two.y, cen.y));
-  }
-  const bool okx = lim != kLimFlat && pr.x > 0.0f, oky = lim != kLimFlat && pr.y > 0.0f;
-  return pk(okx ? (dm.x > 0.0f ? mag.x : -mag.x) : 0.0f,
-            oky ? (dm.y > 0.0f ? mag.y : -mag.y) : 0.0f);
-}
-#endif
-
-// Limited slopes of the 9 primitives of one cell from its two neighbours
-// along a direction, with the zero-slope fallback when a face density or
-// pressure would be non-positive.  PAIRED: FP32 on the device pairs the
-// variables (0, 1) ... (6, 7) in packed instructions (the same values; fewer
-// instructions, more registers live).
-template <class T, bool PAIRED = true>
+// Half slopes of the 9 primitives of one cell from its two neighbours along a
+// direction, 0 for all of them when a face density or pressure would be
+// non-positive.  m, c, p: the cells (variables sm, sc, sp apart); h: variables
+// sh apart.
+template <class T>
 __device__ __forceinline__ void cell_slopes(const T* m, int sm, const T* c, int sc, const T* p,
-                                            int sp, int lim, T sig[kNV]) {
-#if defined(__CUDA_ARCH__) && __CUDA_ARCH__ >= 1000
-  if constexpr (PAIRED && sizeof(T) == 4) {
+                                            int sp, int lim, T* h, int sh) {
+  T sig[kNV];
+  if (lim == kLimMC) {
 #pragma unroll
-    for (int k = 0; k + 1 < kNV; k += 2) {
-      const float2 q = pk(c[k * sc], c[(k + 1) * sc]);
-      const float2 dm = sub2(q, pk(m[k * sm], m[(k + 1) * sm]));
-      const float2 dp = sub2(pk(p[k * sp], p[(k + 1) * sp]), q);
-      const float2 s2 = limited_slope2(dm, dp, lim);
-      sig[k] = s2.x;
-      sig[k + 1] = s2.y;
+    for (int k = 0; k < kNV; ++k) {
+      const T q = c[k * sc];
+      sig[k] = half_slope_mc(q - m[k * sm], p[k * sp] - q);
     }
-    {
-      const T q = c[(kNV - 1) * sc];
-      sig[kNV - 1] = limited_slope(q - m[(kNV - 1) * sm], p[(kNV - 1) * sp] - q, lim);
-    }
-    const bool ok = gt0(c[kRHO * sc] - T(0.5) * tabs(sig[kRHO])) &&
-                    gt0(c[kPRS * sc] - T(0.5) * tabs(sig[kPRS]));
-    if (!ok) {
+  } else if (lim == kLimMinmod) {
 #pragma unroll
-      for (int k = 0; k < kNV; ++k) sig[k] = T(0);
+    for (int k = 0; k < kNV; ++k) {
+      const T q = c[k * sc];
+      sig[k] = half_slope_minmod(q - m[k * sm], p[k * sp] - q);
     }
-    return;
+  } else {
+#pragma unroll
+    for (int k = 0; k < kNV; ++k) sig[k] = T(0);
   }
-#endif
-#pragma unroll
-  for (int k = 0; k < kNV; ++k) {
-    const T q = c[k * sc];
-    sig[k] = limited_slope(q - m[k * sm], p[k * sp] - q, lim);
-  }
-  const bool ok = gt0(c[kRHO * sc] - T(0.5) * tabs(sig[kRHO])) &&
-                  gt0(c[kPRS * sc] - T(0.5) * tabs(sig[kPRS]));
+  const bool ok = gt0(c[kRHO * sc] - tabs(sig[kRHO])) && gt0(c[kPRS * sc] - tabs(sig[kPRS]));
   if (!ok) {
 #pragma unroll
     for (int k = 0; k < kNV; ++k) sig[k] = T(0);
   }
+#pragma unroll
+  for (int k = 0; k < kNV; ++k) h[k * sh] = sig[k];
 }
 
 // One tile (bx, by, bz) of one RK stage; called by every thread of a CTA of
@@ -308,8 +276,7 @@ __device__ __forceinline__ void cell_slopes(const T* m, int sm, const T* c, int 
 // the face update), the face / cell electric fields go to p.ctf, and the last
 // stage has no damping and no wave-speed reduction (done after the face update).
 // HALO (3-D, not CT): ghost cells of kBcHalo sides from p.halo (halo_cell).
-template <class T, int TY, int NW, int STAGE, bool ZACT, bool CT = false, bool HALO = false,
-          bool PREFETCH = true>
+template <class T, int TY, int NW, int STAGE, bool ZACT, bool CT = false, bool HALO = false>
 __device__ __forceinline__ void stage_tile(const StageParams<T>& p, const StepScalars& sc,
                                            int bx, int by, int bz, unsigned char* smem_raw,
                                            double* wmax) {
@@ -325,7 +292,7 @@ __device__ __forceinline__ void stage_tile(const StageParams<T>& p, const StepSc
   T* sys = sxs + kNV * G::SXN;
   T* Fx = sys + kNV * G::SYN;
   T* Fy = Fx + kNV * G::FXN;
-  T* zS = Fy + kNV * G::FYN;  // per owner: z slope of cell k+1
+  T* zS = Fy + kNV * G::FYN;  // per owner: z half slope of cell k+1
   T* zP = zS + kNV * G::NINT;  // per owner: face state V_k + sigma_k / 2
   T* zF = zP + kNV * G::NINT;  // per owner: z flux at face k-1/2
 
@@ -364,6 +331,13 @@ __device__ __forceinline__ void stage_tile(const StageParams<T>& p, const StepSc
     if (fl & kFloorP) atomicAdd(&p.floor_cnt[1], 1ull);
     if (fl & kPressF64) atomicAdd(&p.floor_cnt[2], 1ull);
   };
+  // offset of tile cell (r, c) of plane zz, remapped into the grid
+  auto cell_off = [&](int zz, int r, int c) {
+    const int gz = ZACT ? remap(zz, nz, p.bc_lo[2], p.bc_hi[2]) : 0;
+    const int gx = remap(x0 + c, nx, p.bc_lo[0], p.bc_hi[0]);
+    const int gy = G::GY ? remap(y0 + r, ny, p.bc_lo[1], p.bc_hi[1]) : 0;
+    return (long long)gz * p.sz + (long long)gy * p.sy + gx;
+  };
   // cons -> prim of cell (r, c) of plane zz into dst (variables dst_stride
   // apart); own: an interior item of the tile (counted if the tile updates it)
   auto load_cell = [&](int zz, int r, int c, T* dst, int dst_stride, bool own) {
@@ -374,10 +348,7 @@ __device__ __forceinline__ void stage_tile(const StageParams<T>& p, const StepSc
 #pragma unroll
       for (int k = 0; k < kNV; ++k) u[k] = a[k * hs];
     } else {
-      const int gz = ZACT ? remap(zz, nz, p.bc_lo[2], p.bc_hi[2]) : 0;
-      const int gx = remap(x0 + c, nx, p.bc_lo[0], p.bc_hi[0]);
-      const int gy = G::GY ? remap(y0 + r, ny, p.bc_lo[1], p.bc_hi[1]) : 0;
-      const long long off = (long long)gz * p.sz + (long long)gy * p.sy + gx;
+      const long long off = cell_off(zz, r, c);
 #pragma unroll
       for (int k = 0; k < kNV; ++k) u[k] = p.win[k * p.sv + off];
     }
@@ -386,36 +357,6 @@ __device__ __forceinline__ void stage_tile(const StageParams<T>& p, const StepSc
     if (fl && own) count_floors(fl, zz, r, c);
 #pragma unroll
     for (int k = 0; k < kNV; ++k) dst[k * dst_stride] = v[k];
-  };
-  // FP32 kernels without halo faces or constrained transport, one thread per
-  // interior column (NT = NINT): each thread's interior item of the next
-  // iteration (plane k + 3) is fetched into registers one iteration ahead, so
-  // that its global-load latency overlaps this plane's slope, flux and update
-  // phases.  The same cells are read as without it, and converted by the same
-  // code.  (PREFETCH = false: not done, for callers short of registers.)
-  // The slopes are paired in packed FP32 where the prefetch is not done;
-  // with the prefetch, pairing them as well (still within the 128 registers
-  // of two CTAs per SM) ran slower than scalar slopes.
-  constexpr bool PREF = PREFETCH && ZACT && !HALO && !CT && sizeof(T) == 4 && NT == G::NINT;
-  T pre[kNV];
-  auto fetch_interior = [&](int zz) {
-    const int r = tid / TX, c = tid - (tid / TX) * TX;
-    const int gz = remap(zz, nz, p.bc_lo[2], p.bc_hi[2]);
-    const int gx = remap(x0 + c, nx, p.bc_lo[0], p.bc_hi[0]);
-    const int gy = G::GY ? remap(y0 + r, ny, p.bc_lo[1], p.bc_hi[1]) : 0;
-    const long long off = (long long)gz * p.sz + (long long)gy * p.sy + gx;
-#pragma unroll
-    for (int k = 0; k < kNV; ++k) pre[k] = p.win[k * p.sv + off];
-  };
-  auto convert_interior = [&](int zz) {
-    const int r = tid / TX, c = tid - (tid / TX) * TX;
-    T v[kNV];
-    unsigned fl = 0;
-    cons_to_prim(pre, v, ph, fl);
-    if (fl) count_floors(fl, zz, r, c);
-    T* dst = ring_plane(zz) + tid;
-#pragma unroll
-    for (int k = 0; k < kNV; ++k) dst[k * G::PS] = v[k];
   };
   // phase-A item: interior cell of plane zi or halo cell of plane zh
   auto load_item = [&](int it, int zi, int zh) {
@@ -434,28 +375,18 @@ __device__ __forceinline__ void stage_tile(const StageParams<T>& p, const StepSc
       load_cell(zh, r, c, yh + j, G::PS, false);
     }
   };
-  // primitives of cell (r, c) of the current plane (interior in ring slot,
-  // halo in the halo buffers); returns the pointer, stride in *st
-  auto cell_ptr = [&](const T* cur, int r, int c, int* st) -> const T* {
-    if (c < 0 || c >= TX) {
-      *st = G::PS;
-      return xh + r * 4 + (c < 0 ? c + 2 : c - TX + 2);
-    }
-    if (r < 0 || r >= TY) {
-      *st = G::PS;
-      return yh + (r < 0 ? r + 2 : r - TY + 2) * TX + c;
-    }
-    *st = G::PS;
+  // primitives of cell (r, c) of the current plane (interior in the ring slot,
+  // halo in the halo buffers; variables G::PS apart)
+  auto cell_ptr = [&](const T* cur, int r, int c) -> const T* {
+    if (c < 0 || c >= TX) return xh + r * 4 + (c < 0 ? c + 2 : c - TX + 2);
+    if (r < 0 || r >= TY) return yh + (r < 0 ? r + 2 : r - TY + 2) * TX + c;
     return cur + r * TX + c;
   };
   static_assert(!CT || ZACT, "constrained transport is 3-D only");
   static_assert(!HALO || (ZACT && !CT), "halo faces: 3-D GLM kernels only");
   // staggered normal field on the lower d-face of tile cell (r, c) of plane zz
   auto bface = [&](int d, int zz, int r, int c) -> T {
-    const int gz = remap(zz, nz, p.bc_lo[2], p.bc_hi[2]);
-    const int gx = remap(x0 + c, nx, p.bc_lo[0], p.bc_hi[0]);
-    const int gy = remap(y0 + r, ny, p.bc_lo[1], p.bc_hi[1]);
-    return p.bw[d][(long long)gz * p.sz + (long long)gy * p.sy + gx];
+    return p.bw[d][cell_off(zz, r, c)];
   };
   CtCell<T> ctc;
 
@@ -473,82 +404,53 @@ __device__ __forceinline__ void stage_tile(const StageParams<T>& p, const StepSc
 #pragma unroll 1
   for (int k = z0 - NWARM; k < z1; ++k) {
     const bool main = k >= z0;
-    // FP32 (two CTAs per SM): the item loops of phases A-C start at a
-    // thread index rotated by (k mod 4) whole warps.  A phase's items do not
-    // divide evenly among the warps; without the rotation the warps left with
-    // one item more are always the first ones, on the same schedulers in
-    // both CTAs of an SM, and rotated they change from plane to plane.
-    // Which thread takes an item does not change its result.
-    const int rtid = sizeof(T) == 4 ? (tid + 32 * (k & 3)) % NT : tid;
     // ---- A: loads ---------------------------------------------------------
     const int nload = main ? G::NLOAD : G::NINT;
-    if constexpr (PREF) {
-      // interior item (it = tid) from the registers fetched last iteration
-      if (k > z0 - NWARM) {
-        convert_interior(k + 2);
-      } else {
-        fetch_interior(k + 2);
-        convert_interior(k + 2);
-      }
-      for (int it = rtid + NT; it < nload; it += NT) load_item(it, k, k);
-    } else {
-      for (int it = rtid; it < nload; it += NT) {
-        if (ZACT && it < G::NINT)
-          load_item(it, k + 2, k);
-        else
-          load_item(it, k, k);
-      }
+    for (int it = tid; it < nload; it += NT) {
+      if (ZACT && it < G::NINT)
+        load_item(it, k + 2, k);
+      else
+        load_item(it, k, k);
     }
     __syncthreads();
-    if constexpr (PREF) {
-      if (k + 1 < z1) fetch_interior(k + 3);
-    }
     if (ZACT && k < z0 - 2) continue;
     const T* cur = ring_plane(k);
 
     // ---- B: slopes --------------------------------------------------------
-    for (int it = rtid; main && it < G::SXN + G::SYN; it += NT) {
-      T sig[kNV];
+    for (int it = tid; main && it < G::SXN + G::SYN; it += NT) {
       T* dst;
       int ds;
-      int s0, s1, s2;
       const T *m, *c, *pp;
       if (it < G::SXN) {
         const int r = it / (TX + 2), cc = it - r * (TX + 2) - 1;
-        m = cell_ptr(cur, r, cc - 1, &s0);
-        c = cell_ptr(cur, r, cc, &s1);
-        pp = cell_ptr(cur, r, cc + 1, &s2);
+        m = cell_ptr(cur, r, cc - 1);
+        c = cell_ptr(cur, r, cc);
+        pp = cell_ptr(cur, r, cc + 1);
         dst = sxs + it;
         ds = G::SXN;
       } else {
         const int j = it - G::SXN;
         const int rr = j / TX - 1, cc = j - (j / TX) * TX;
-        m = cell_ptr(cur, rr - 1, cc, &s0);
-        c = cell_ptr(cur, rr, cc, &s1);
-        pp = cell_ptr(cur, rr + 1, cc, &s2);
+        m = cell_ptr(cur, rr - 1, cc);
+        c = cell_ptr(cur, rr, cc);
+        pp = cell_ptr(cur, rr + 1, cc);
         dst = sys + j;
         ds = G::SYN;
       }
-      cell_slopes<T, !PREF>(m, s0, c, s1, pp, s2, lim, sig);
-#pragma unroll
-      for (int q = 0; q < kNV; ++q) dst[q * ds] = sig[q];
+      cell_slopes(m, G::PS, c, G::PS, pp, G::PS, lim, dst, ds);
     }
-    if (ZACT && owner) {
-      T sig[kNV];
-      cell_slopes<T, !PREF>(cur + oidx, G::PS, ring_plane(k + 1) + oidx, G::PS,
-                            ring_plane(k + 2) + oidx, G::PS, lim, sig);
-#pragma unroll
-      for (int q = 0; q < kNV; ++q) zS[q * G::NINT + oidx] = sig[q];
-    }
+    if (ZACT && owner)
+      cell_slopes(cur + oidx, G::PS, ring_plane(k + 1) + oidx, G::PS, ring_plane(k + 2) + oidx,
+                  G::PS, lim, zS + oidx, G::NINT);
     __syncthreads();
 
     // ---- C: fluxes --------------------------------------------------------
-    for (int it = rtid; main && it < G::ITEMS; it += NT) {
+    for (int it = tid; main && it < G::ITEMS; it += NT) {
       T vl[kNV], vr[kNV], F[kNV];
-      int dir;
       T* out;
       int os;
-      if (it < G::IT_X || it >= G::IT_X + G::IT_Y) {
+      const bool xdir = it < G::IT_X || it >= G::IT_X + G::IT_Y;
+      if (xdir) {
         int r, fi;
         if (it < G::IT_X) {
           r = it / TX;
@@ -557,40 +459,36 @@ __device__ __forceinline__ void stage_tile(const StageParams<T>& p, const StepSc
           r = it - (G::IT_X + G::IT_Y);
           fi = TX;
         }
-        int sa, sb;
-        const T* a = cell_ptr(cur, r, fi - 1, &sa);
-        const T* b = cell_ptr(cur, r, fi, &sb);
-        const T* ga = sxs + r * (TX + 2) + fi;      // slope of cell fi-1
-        const T* gb = ga + 1;                        // slope of cell fi
+        const T* a = cell_ptr(cur, r, fi - 1);
+        const T* b = cell_ptr(cur, r, fi);
+        const T* ga = sxs + r * (TX + 2) + fi;      // half slope of cell fi-1
+        const T* gb = ga + 1;                        // half slope of cell fi
 #pragma unroll
         for (int q = 0; q < kNV; ++q) {
-          vl[q] = a[q * sa] + T(0.5) * ga[q * G::SXN];
-          vr[q] = b[q * sb] - T(0.5) * gb[q * G::SXN];
+          vl[q] = a[q * G::PS] + ga[q * G::SXN];
+          vr[q] = b[q * G::PS] - gb[q * G::SXN];
         }
         if constexpr (CT) ct_face_field(vl, vr, 0, bface(0, k, r, fi));
-        dir = 0;
         out = Fx + r * (TX + 1) + fi;
         os = G::FXN;
       } else {
         const int j = it - G::IT_X;
         const int fj = j / TX, c = j - (j / TX) * TX;
-        int sa, sb;
-        const T* a = cell_ptr(cur, fj - 1, c, &sa);
-        const T* b = cell_ptr(cur, fj, c, &sb);
-        const T* ga = sys + fj * TX + c;             // slope of row fj-1
-        const T* gb = ga + TX;                       // slope of row fj
+        const T* a = cell_ptr(cur, fj - 1, c);
+        const T* b = cell_ptr(cur, fj, c);
+        const T* ga = sys + fj * TX + c;             // half slope of row fj-1
+        const T* gb = ga + TX;                       // half slope of row fj
 #pragma unroll
         for (int q = 0; q < kNV; ++q) {
-          vl[q] = a[q * sa] + T(0.5) * ga[q * G::SYN];
-          vr[q] = b[q * sb] - T(0.5) * gb[q * G::SYN];
+          vl[q] = a[q * G::PS] + ga[q * G::SYN];
+          vr[q] = b[q * G::PS] - gb[q * G::SYN];
         }
         if constexpr (CT) ct_face_field(vl, vr, 1, bface(1, k, fj, c));
-        dir = 1;
         out = Fy + j;
         os = G::FYN;
       }
       // warp-uniform branch to the compile-time direction
-      if (dir == 0)
+      if (xdir)
         glm_hlld_flux<0>(vl, vr, ch, half_chi, ph, F);
       else
         glm_hlld_flux<1>(vl, vr, ch, half_chi, ph, F);
@@ -605,7 +503,7 @@ __device__ __forceinline__ void stage_tile(const StageParams<T>& p, const StepSc
 #pragma unroll
         for (int q = 0; q < kNV; ++q) {
           vl[q] = zP[q * G::NINT + oidx];
-          vr[q] = c[q * G::PS] - T(0.5) * zS[q * G::NINT + oidx];
+          vr[q] = c[q * G::PS] - zS[q * G::NINT + oidx];
         }
         if constexpr (CT) {
           ct_face_field(vl, vr, 2, bface(2, k + 1, orow, ocol));
@@ -618,13 +516,13 @@ __device__ __forceinline__ void stage_tile(const StageParams<T>& p, const StepSc
           glm_hlld_flux<2>(vl, vr, ch, half_chi, ph, F);
 #pragma unroll
           for (int q = 0; q < kNV; ++q) {
-            dUz[q] = mul_rn(F[q] - zF[q * G::NINT + oidx], dtdz);
+            dUz[q] = F[q] - zF[q * G::NINT + oidx];
             zF[q * G::NINT + oidx] = F[q];
           }
         }
 #pragma unroll
         for (int q = 0; q < kNV; ++q)
-          zP[q * G::NINT + oidx] = c[q * G::PS] + T(0.5) * zS[q * G::NINT + oidx];
+          zP[q * G::NINT + oidx] = c[q * G::PS] + zS[q * G::NINT + oidx];
       }
     }
     __syncthreads();
@@ -648,7 +546,7 @@ __device__ __forceinline__ void stage_tile(const StageParams<T>& p, const StepSc
             const T* fy = Fy + q * G::FYN + orow * TX + ocol;
             du = fma_rn(fy[TX] - fy[0], dtdy, du);
           }
-          if constexpr (ZACT) du += dUz[q];
+          if constexpr (ZACT) du = fma_rn(dUz[q], dtdz, du);
           if (frozen) du = T(0);
           const T s1 = p.win[q * p.sv + off] - du;
           if constexpr (STAGE == 1) {
@@ -660,11 +558,12 @@ __device__ __forceinline__ void stage_tile(const StageParams<T>& p, const StepSc
         if constexpr (CT) {
 #pragma unroll
           for (int q = 0; q < kNV; ++q)
-            if (q != kBX && q != kBY && q != kBZ) p.uout[q * p.sv + off] = q == kPSI ? T(0) : unew[q];
+            if (q != kBX && q != kBY && q != kBZ)
+              p.uout[q * p.sv + off] = q == kPSI ? T(0) : unew[q];
           ctc.write(p.ctf, p.sv, off, Fx + orow * (TX + 1) + ocol, G::FXN,
                     Fy + orow * TX + ocol, G::FYN, ch);
         } else {
-          if constexpr (STAGE == 2) unew[kPSI] *= damp;
+          if constexpr (STAGE == 2) unew[kPSI] = mul_rn(unew[kPSI], damp);
 #pragma unroll
           for (int q = 0; q < kNV; ++q) p.uout[q * p.sv + off] = unew[q];
         }
@@ -698,7 +597,8 @@ __device__ __forceinline__ void stage_tile(const StageParams<T>& p, const StepSc
 }
 
 template <class T, int TY, int NW, int STAGE, bool ZACT, bool CT, bool HALO = false>
-__global__ void __launch_bounds__(NW * 32, 1) rk_stage_kernel(const StageParams<T> p) {
+__global__ void __launch_bounds__(NW * 32, sizeof(T) == 4 && ZACT ? 2 : 1)
+    rk_stage_kernel(const StageParams<T> p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ double wmax[NW];
   const StepScalars sc = *p.sc;

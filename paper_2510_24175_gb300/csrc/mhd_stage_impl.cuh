@@ -7,18 +7,19 @@
 
 namespace mhd {
 
-// Tile shapes: 3-D grids use 32 x 8 column tiles marching in z.  FP64 runs
-// 16 warps per CTA (one CTA per SM: 201 KB of shared memory): the SM's FP64
-// unit is shared by all its warps and one warp issues an FP64 instruction at
-// most every 64 clocks, so the unit saturates only when at least four warps
-// have FP64 work; 16 warps (8 helper warps, 8 column owners) keep more warps
-// busy through the phases than 13 and cap registers at 128 as 13 do (four
-// warps per scheduler).  FP32 runs 8 warps and two CTAs per SM.  2-D grids
-// use the same tile with a single plane; 1-D grids a 32-cell row.
+// Tile shapes: 3-D grids use 32 x 8 column tiles marching in z with 16 warps
+// per CTA (8 helper warps, 8 column owners).  FP64: one CTA per SM (211 KB of
+// shared memory); the SM's FP64 unit is shared by all its warps and one warp
+// issues an FP64 instruction at most every 64 clocks, so the unit saturates
+// only when at least four warps have FP64 work.  FP32: two CTAs per SM at 64
+// registers, 32 warps: the kernel is bound by latency and issue, and with 24
+// and 16 warps per SM (80 and 128 registers) it took 56.3 and 59.4 ms against
+// 55.1 for two steps of a 512^3 box.  2-D grids use the same tile with a single
+// plane; 1-D grids a 32-cell row.
 template <class T>
 struct StageShape3D {
   static constexpr int TY = 8;
-  static constexpr int NW = sizeof(T) == 8 ? 16 : 8;
+    static constexpr int NW = 16;
 };
 
 // The dynamic shared-memory limit of a kernel is set once per device (a
@@ -59,16 +60,15 @@ static cudaError_t launch_weno(const StageParams<T>& p, dim3 grid, cudaStream_t 
   return cudaGetLastError();
 }
 
-// WENO-Z tiles of 3-D grids.  FP64: 32 x 4 columns, 8 warps (the
-// face-value phase gives every warp two cells' worth of work), one CTA per
-// SM (166 KB of shared memory).  FP32: 32 x 8 columns, 16 warps (8 helper
-// warps, 8 column owners), one CTA per SM (154 KB): the three-deep y halo
-// is then 6 rows per 8 instead of per 4, and the kernel ran 8 % faster with
-// GLM and 5 % with constrained transport than with 32 x 4 tiles at two
-// 8-warp CTAs per SM.  2-D grids use 32 x 4 tiles with a single plane.
+// WENO-Z tiles of 3-D grids: 32 x 4 columns.  FP64: 8 warps (the face-value
+// phase gives every warp two cells' worth of work), one CTA per SM (167 KB of
+// shared memory).  FP32: 16 warps and two CTAs per SM at 64 registers; three
+// steps of a 256^3 box with constrained transport take 36.5 ms, 38.0 and 39.6
+// with 24 and 16 warps per SM, and 40.6 on 32 x 8 tiles with one CTA of 16 warps.
+// 2-D grids use 32 x 4 tiles with a single plane.
 template <class T>
 struct WenoShape3D {
-  static constexpr int TY = sizeof(T) == 8 ? 4 : 8;
+  static constexpr int TY = 4;
   static constexpr int NW = sizeof(T) == 8 ? 8 : 16;
 };
 

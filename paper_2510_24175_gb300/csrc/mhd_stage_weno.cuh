@@ -46,8 +46,8 @@ template <> struct WenoEps<float> { static constexpr float v = 1e-18f; };
 // product of the two faces' denominators serves both faces.  In FP32 these
 // products of epsilons underflow (a uniform variable has beta = 0), so FP32
 // takes the reciprocals 1 / e_k and one per face.
-template <class T>
-__device__ __forceinline__ void wenoz_pair(const T f[5], T& minus, T& plus) {
+__device__ __forceinline__ void wenoz_pair(const double f[5], double& minus, double& plus) {
+  using T = double;
   const T c12 = T(1.0 / 12.0), q4 = T(0.25), c39 = T(39);
   const T D0 = c12 * (f[0] + f[2] - T(2) * f[1]);
   const T D1 = c12 * (f[1] + f[3] - T(2) * f[2]);
@@ -61,106 +61,77 @@ __device__ __forceinline__ void wenoz_pair(const T f[5], T& minus, T& plus) {
   const T eps = T(0.25) * WenoEps<T>::v;
   const T tau = tabs(b0 - b2);
   const T e0 = b0 + eps, e1 = b1 + eps, e2 = b2 + eps;
-  T P0, P1, P2;
-  if constexpr (sizeof(T) == 8) {
-    const T E0 = e1 * e2, E2 = e0 * e1;
-    const T pi = e0 * E0;
-    P0 = pi + tau * E0, P1 = pi + tau * (e0 * e2), P2 = pi + tau * E2;
-  } else {
-    P0 = T(1) + tau * rcp(e0), P1 = T(1) + tau * rcp(e1), P2 = T(1) + tau * rcp(e2);
-  }
+  const T E0 = e1 * e2, E2 = e0 * e1;
+  const T pi = e0 * E0;
+  const T P0 = pi + tau * E0, P1 = pi + tau * (e0 * e2), P2 = pi + tau * E2;
   const T S1 = T(6) * P1, T0 = T(3) * P0, T2 = T(3) * P2;
   const T den_p = P0 + S1 + T2, den_m = P2 + S1 + T0;
   const T num_p = P0 * (D0 + G0) + S1 * (D1 - G1) + T2 * (D2 - G2);
   const T num_m = P2 * (D2 + G2) + S1 * (D1 + G1) + T0 * (D0 - G0);
-  if constexpr (sizeof(T) == 8) {
-    const T r = rcp(den_p * den_m);
-    plus = f[2] + num_p * den_m * r;
-    minus = f[2] + num_m * den_p * r;
-  } else {
-    plus = f[2] + num_p * rcp(den_p);
-    minus = f[2] + num_m * rcp(den_m);
-  }
+  const T r = rcp(den_p * den_m);
+  plus = f[2] + num_p * den_m * r;
+  minus = f[2] + num_m * den_p * r;
 }
 
-#if defined(__CUDA_ARCH__) && __CUDA_ARCH__ >= 1000
-// FP32 WENO-Z of two variables at once (.x, .y), the steps of wenoz_pair<float>
-// in packed FP32 with every operation written out; the reciprocals per lane.
-__device__ __forceinline__ void wenoz_pair2(const float2 f[5], float2& minus, float2& plus) {
-  const float2 C12 = pk1(1.0f / 12.0f), Q4 = pk1(0.25f), C39 = pk1(39.0f);
-  const float2 M2 = pk1(-2.0f), M4 = pk1(-4.0f), T3 = pk1(3.0f);
-  const float2 D0 = mul2(C12, fma2(M2, f[1], add2(f[0], f[2])));
-  const float2 D1 = mul2(C12, fma2(M2, f[2], add2(f[1], f[3])));
-  const float2 D2 = mul2(C12, fma2(M2, f[3], add2(f[2], f[4])));
-  const float2 G0 = mul2(Q4, fma2(T3, f[2], fma2(M4, f[1], f[0])));
-  const float2 G1 = mul2(Q4, sub2(f[1], f[3]));
-  const float2 G2 = mul2(Q4, add2(fma2(M4, f[3], mul2(T3, f[2])), f[4]));
-  const float2 b0 = fma2(G0, G0, mul2(mul2(C39, D0), D0));
-  const float2 b1 = fma2(G1, G1, mul2(mul2(C39, D1), D1));
-  const float2 b2 = fma2(G2, G2, mul2(mul2(C39, D2), D2));
-  const float2 EPS = pk1(0.25f * WenoEps<float>::v);
-  const float2 d02 = sub2(b0, b2);
-  const float2 tau = pk(fabsf(d02.x), fabsf(d02.y));
-  const float2 e0 = add2(b0, EPS), e1 = add2(b1, EPS), e2 = add2(b2, EPS);
-  const float2 ONE = pk1(1.0f);
-  const float2 P0 = fma2(tau, pk(rcp(e0.x), rcp(e0.y)), ONE);
-  const float2 P1 = fma2(tau, pk(rcp(e1.x), rcp(e1.y)), ONE);
-  const float2 P2 = fma2(tau, pk(rcp(e2.x), rcp(e2.y)), ONE);
-  const float2 S1 = mul2(pk1(6.0f), P1), T0 = mul2(T3, P0), T2 = mul2(T3, P2);
-  const float2 den_p = add2(add2(P0, S1), T2), den_m = add2(add2(P2, S1), T0);
-  const float2 num_p = fma2(T2, sub2(D2, G2), fma2(S1, sub2(D1, G1), mul2(P0, add2(D0, G0))));
-  const float2 num_m = fma2(T0, sub2(D0, G0), fma2(S1, add2(D1, G1), mul2(P2, add2(D2, G2))));
-  plus = fma2(num_p, pk(rcp(den_p.x), rcp(den_p.y)), f[2]);
-  minus = fma2(num_m, pk(rcp(den_m.x), rcp(den_m.y)), f[2]);
+// FP32: two variables at once, the same steps with every operation written out.
+__device__ __forceinline__ void wenoz_pair(const f2 f[5], f2& minus, f2& plus) {
+  using V = f2;
+  const V C12(1.0f / 12.0f), Q4(0.25f), C39(39.0f), M2(-2.0f), M4(-4.0f), T3(3.0f), ONE(1.0f);
+  const V D0 = mul_rn(C12, fma_rn(M2, f[1], f[0] + f[2]));
+  const V D1 = mul_rn(C12, fma_rn(M2, f[2], f[1] + f[3]));
+  const V D2 = mul_rn(C12, fma_rn(M2, f[3], f[2] + f[4]));
+  const V G0 = mul_rn(Q4, fma_rn(T3, f[2], fma_rn(M4, f[1], f[0])));
+  const V G1 = mul_rn(Q4, f[1] - f[3]);
+  const V G2 = mul_rn(Q4, fma_rn(M4, f[3], mul_rn(T3, f[2])) + f[4]);
+  const V b0 = fma_rn(G0, G0, mul_rn(mul_rn(C39, D0), D0));
+  const V b1 = fma_rn(G1, G1, mul_rn(mul_rn(C39, D1), D1));
+  const V b2 = fma_rn(G2, G2, mul_rn(mul_rn(C39, D2), D2));
+  const V EPS(0.25f * WenoEps<float>::v);
+  const V tau = tabs(b0 - b2);
+  const V P0 = fma_rn(tau, rcp(b0 + EPS), ONE);
+  const V P1 = fma_rn(tau, rcp(b1 + EPS), ONE);
+  const V P2 = fma_rn(tau, rcp(b2 + EPS), ONE);
+  const V S1 = mul_rn(V(6.0f), P1), T0 = mul_rn(T3, P0), T2 = mul_rn(T3, P2);
+  const V den_p = P0 + S1 + T2, den_m = P2 + S1 + T0;
+  const V num_p = fma_rn(T2, D2 - G2, fma_rn(S1, D1 - G1, mul_rn(P0, D0 + G0)));
+  const V num_m = fma_rn(T0, D0 - G0, fma_rn(S1, D1 + G1, mul_rn(P2, D2 + G2)));
+  plus = fma_rn(num_p, rcp(den_p), f[2]);
+  minus = fma_rn(num_m, rcp(den_m), f[2]);
 }
-#endif
-
 // Face values of all 9 primitives of one cell from five cells c[0..4]
 // (variables stride[j] apart); flat fallback on non-positive face density
-// or pressure.  FP32 on the device reconstructs the variables in pairs
-// (0, 1) ... (6, 7) in packed instructions.
+// or pressure.  FP32 reconstructs the variables in pairs (0, 1) ... (6, 7).
 template <class T>
 __device__ __forceinline__ void cell_weno(const T* const c[5], const int st[5], T M[kNV],
                                           T P[kNV]) {
-#if defined(__CUDA_ARCH__) && __CUDA_ARCH__ >= 1000
   if constexpr (sizeof(T) == 4) {
 #pragma unroll
     for (int k = 0; k + 1 < kNV; k += 2) {
-      float2 f[5];
+      f2 f[5], m, p;
 #pragma unroll
-      for (int j = 0; j < 5; ++j) f[j] = pk(c[j][k * st[j]], c[j][(k + 1) * st[j]]);
-      float2 m2, p2;
-      wenoz_pair2(f, m2, p2);
-      M[k] = m2.x;
-      M[k + 1] = m2.y;
-      P[k] = p2.x;
-      P[k + 1] = p2.y;
+      for (int j = 0; j < 5; ++j) f[j] = f2(c[j][k * st[j]], c[j][(k + 1) * st[j]]);
+      wenoz_pair(f, m, p);
+      M[k] = m.v.x;
+      M[k + 1] = m.v.y;
+      P[k] = p.v.x;
+      P[k + 1] = p.v.y;
     }
-    {
-      float2 f[5];
+    f2 f[5], m, p;
 #pragma unroll
-      for (int j = 0; j < 5; ++j) f[j] = pk1(c[j][(kNV - 1) * st[j]]);
-      float2 m2, p2;
-      wenoz_pair2(f, m2, p2);
-      M[kNV - 1] = m2.x;
-      P[kNV - 1] = p2.x;
-    }
-    const bool ok = M[kRHO] > T(0) && P[kRHO] > T(0) && M[kPRS] > T(0) && P[kPRS] > T(0);
-    if (!ok) {
+    for (int j = 0; j < 5; ++j) f[j] = f2(c[j][(kNV - 1) * st[j]]);
+    wenoz_pair(f, m, p);
+    M[kNV - 1] = m.v.x;
+    P[kNV - 1] = p.v.x;
+  } else {
 #pragma unroll
-      for (int k = 0; k < kNV; ++k) M[k] = P[k] = c[2][k * st[2]];
+    for (int k = 0; k < kNV; ++k) {
+      T f[5];
+#pragma unroll
+      for (int j = 0; j < 5; ++j) f[j] = c[j][k * st[j]];
+      wenoz_pair(f, M[k], P[k]);
     }
-    return;
   }
-#endif
-#pragma unroll
-  for (int k = 0; k < kNV; ++k) {
-    T f[5];
-#pragma unroll
-    for (int j = 0; j < 5; ++j) f[j] = c[j][k * st[j]];
-    wenoz_pair(f, M[k], P[k]);
-  }
-  const bool ok = M[kRHO] > T(0) && P[kRHO] > T(0) && M[kPRS] > T(0) && P[kPRS] > T(0);
+  const bool ok = gt0(M[kRHO]) && gt0(P[kRHO]) && gt0(M[kPRS]) && gt0(P[kPRS]);
   if (!ok) {
 #pragma unroll
     for (int k = 0; k < kNV; ++k) M[k] = P[k] = c[2][k * st[2]];
@@ -193,11 +164,8 @@ struct WenoGeom {
 };
 
 // CT: constrained transport, HALO: halo faces, as in stage_tile() (mhd_stage.cuh).
-// 3-D FP32 with 8-warp CTAs: two CTAs per SM (128 registers at most);
-// without the bound the packed reconstruction takes 132-150 registers and
-// runs one CTA per SM, 25-30 % slower.  (Larger CTAs run one per SM.)
 template <class T, int TY, int NW, int STAGE, bool ZACT, bool CT, bool HALO = false>
-__global__ void __launch_bounds__(NW * 32, (sizeof(T) == 4 && ZACT && NW <= 8) ? 2 : 1)
+__global__ void __launch_bounds__(NW * 32, sizeof(T) == 4 && ZACT ? 2 : 1)
     rk_stage_weno_kernel(const StageParams<T> p) {
   using G = WenoGeom<TY, ZACT>;
   constexpr int NT = NW * 32;
@@ -250,6 +218,13 @@ __global__ void __launch_bounds__(NW * 32, (sizeof(T) == 4 && ZACT && NW <= 8) ?
     if (fl & kFloorP) atomicAdd(&p.floor_cnt[1], 1ull);
     if (fl & kPressF64) atomicAdd(&p.floor_cnt[2], 1ull);
   };
+  // offset of tile cell (r, c) of plane zz, remapped into the grid
+  auto cell_off = [&](int zz, int r, int c) {
+    const int gz = ZACT ? remap3(zz, nz, p.bc_lo[2], p.bc_hi[2]) : 0;
+    const int gx = remap3(x0 + c, nx, p.bc_lo[0], p.bc_hi[0]);
+    const int gy = G::GY ? remap3(y0 + r, ny, p.bc_lo[1], p.bc_hi[1]) : 0;
+    return (long long)gz * p.sz + (long long)gy * p.sy + gx;
+  };
   auto load_cell = [&](int zz, int r, int c, T* dst, int dst_stride, bool own) {
     T u[kNV], v[kNV];
     if constexpr (HALO) {
@@ -258,10 +233,7 @@ __global__ void __launch_bounds__(NW * 32, (sizeof(T) == 4 && ZACT && NW <= 8) ?
 #pragma unroll
       for (int k = 0; k < kNV; ++k) u[k] = a[k * hs];
     } else {
-      const int gz = ZACT ? remap3(zz, nz, p.bc_lo[2], p.bc_hi[2]) : 0;
-      const int gx = remap3(x0 + c, nx, p.bc_lo[0], p.bc_hi[0]);
-      const int gy = G::GY ? remap3(y0 + r, ny, p.bc_lo[1], p.bc_hi[1]) : 0;
-      const long long off = (long long)gz * p.sz + (long long)gy * p.sy + gx;
+      const long long off = cell_off(zz, r, c);
 #pragma unroll
       for (int k = 0; k < kNV; ++k) u[k] = p.win[k * p.sv + off];
     }
@@ -303,10 +275,7 @@ __global__ void __launch_bounds__(NW * 32, (sizeof(T) == 4 && ZACT && NW <= 8) ?
   static_assert(!HALO || (ZACT && !CT), "halo faces: 3-D GLM kernels only");
   // staggered normal field on the lower d-face of tile cell (r, c) of plane zz
   auto bface = [&](int d, int zz, int r, int c) -> T {
-    const int gz = remap3(zz, nz, p.bc_lo[2], p.bc_hi[2]);
-    const int gx = remap3(x0 + c, nx, p.bc_lo[0], p.bc_hi[0]);
-    const int gy = remap3(y0 + r, ny, p.bc_lo[1], p.bc_hi[1]);
-    return p.bw[d][(long long)gz * p.sz + (long long)gy * p.sy + gx];
+    return p.bw[d][cell_off(zz, r, c)];
   };
   CtCell<T> ctc;
   // face values of the owned column's cell in plane zc (planes zc-2..zc+2)
@@ -446,7 +415,7 @@ __global__ void __launch_bounds__(NW * 32, (sizeof(T) == 4 && ZACT && NW <= 8) ?
           glm_hlld_flux<2>(vl, vr, ch, half_chi, ph, F);
 #pragma unroll
           for (int q = 0; q < kNV; ++q) {
-            dUz[q] = mul_rn(F[q] - zF[q * G::NINT + oidx], dtdz);
+            dUz[q] = F[q] - zF[q * G::NINT + oidx];
             zF[q * G::NINT + oidx] = F[q];
           }
         }
@@ -475,7 +444,7 @@ __global__ void __launch_bounds__(NW * 32, (sizeof(T) == 4 && ZACT && NW <= 8) ?
             const T* fy = Fy + q * G::FYN + orow * TX + ocol;
             du = fma_rn(fy[TX] - fy[0], dtdy, du);
           }
-          if constexpr (ZACT) du += dUz[q];
+          if constexpr (ZACT) du = fma_rn(dUz[q], dtdz, du);
           if (frozen) du = T(0);
           const T s1 = p.win[q * p.sv + off] - du;
           if constexpr (STAGE == 1) {
@@ -487,11 +456,12 @@ __global__ void __launch_bounds__(NW * 32, (sizeof(T) == 4 && ZACT && NW <= 8) ?
         if constexpr (CT) {
 #pragma unroll
           for (int q = 0; q < kNV; ++q)
-            if (q != kBX && q != kBY && q != kBZ) p.uout[q * p.sv + off] = q == kPSI ? T(0) : unew[q];
+            if (q != kBX && q != kBY && q != kBZ)
+              p.uout[q * p.sv + off] = q == kPSI ? T(0) : unew[q];
           ctc.write(p.ctf, p.sv, off, Fx + orow * (TX + 1) + ocol, G::FXN,
                     Fy + orow * TX + ocol, G::FYN, ch);
         } else {
-          if constexpr (STAGE == 2) unew[kPSI] *= damp;
+          if constexpr (STAGE == 2) unew[kPSI] = mul_rn(unew[kPSI], damp);
 #pragma unroll
           for (int q = 0; q < kNV; ++q) p.uout[q * p.sv + off] = unew[q];
         }
