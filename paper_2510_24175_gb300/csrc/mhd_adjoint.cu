@@ -52,7 +52,7 @@ __global__ void adj_prims_kernel(const double* __restrict__ W, double* __restric
 // One thread per face of direction DIR; faces f = 0..n_d along d (face f
 // separates cells f-1 and f).  Wp: the primitives of the stage input.
 template <int DIR>
-__global__ void __launch_bounds__(128) adj_faces_kernel(const double* __restrict__ Wp,
+__global__ void __launch_bounds__(128, 3) adj_faces_kernel(const double* __restrict__ Wp,
                                                         const double* __restrict__ x,
                                                         double* __restrict__ gV,
                                                         const FaceArgs a) {
@@ -122,15 +122,13 @@ __global__ void __launch_bounds__(128) adj_faces_kernel(const double* __restrict
 #pragma unroll
     for (int k = 0; k < kNV; ++k) {
       const unsigned ck = (unsigned)(codes >> (6 * k));
-      double dma, dpa, dmb, dpb;
-      slope_code_d(ck & 7u, dma, dpa);
-      slope_code_d((ck >> 3) & 7u, dmb, dpb);
-      const double ga = oka ? 0.5 * vlb[k] : 0.0;   // dJ/ds_a
-      const double gb = okb ? -0.5 * vrb[k] : 0.0;  // dJ/ds_b
-      const double g0 = -dma * ga;
-      const double g1 = vlb[k] + (dma - dpa) * ga - dmb * gb;
-      const double g2 = dpa * ga + vrb[k] + (dmb - dpb) * gb;
-      const double g3 = dpb * gb;
+      double hma, hpa, ca, hmb, hpb, cb;
+      slope_code_half(ck & 7u, oka, false, hma, hpa, ca);
+      slope_code_half((ck >> 3) & 7u, okb, true, hmb, hpb, cb);
+      const double g0 = -(hma * vlb[k]);
+      const double g1 = ca * vlb[k] + hmb * vrb[k];
+      const double g2 = hpa * vlb[k] + cb * vrb[k];
+      const double g3 = -(hpb * vrb[k]);
       // (zero tests on the integer pipe)
       if (nonzero(g0)) atomicAdd(&gV[k * a.sv + off[0]], g0);
       if (nonzero(g1)) atomicAdd(&gV[k * a.sv + off[1]], g1);

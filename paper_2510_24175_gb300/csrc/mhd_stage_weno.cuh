@@ -27,15 +27,15 @@ template <> struct WenoEps<double> { static constexpr double v = 1e-40; };
 template <> struct WenoEps<float> { static constexpr float v = 1e-18f; };
 
 // WENO-Z values of one variable at the cell's faces i-1/2 (minus) and i+1/2
-// (plus) from f[0..4] = cells i-2 .. i+2.  With the second differences
-// d_k and the one-sided first-difference combinations g_k of the three
-// candidate stencils, written as D_k = d_k/12 and G_k = g_k/4:
-//   * every candidate value is the cell value plus D_k +- G_k (the plus face
-//     takes D0+G0, D1-G1, D2-G2; the minus face, whose stencils are the
-//     mirrored ones, D2+G2, D1+G1, D0-G0);
-//   * the Jiang-Shu smoothness indicator is beta_k = 13/12 d_k^2 + 1/4 g_k^2
-//     = 4 (39 D_k^2 + G_k^2); the weights are invariant under a common scale
-//     of beta, tau and epsilon, so the code works with beta/4 and epsilon/4;
+// (plus) from f[0..4] = cells i-2 .. i+2.  With the second differences a_k
+// and the one-sided first-difference combinations g_k of the three candidate
+// stencils:
+//   * 12 x (candidate value - cell value) is a_k +- 3 g_k (the plus face takes
+//     a0+3g0, a1+3g1, a2-3g2; the minus face, whose stencils are the mirrored
+//     ones, a2+3g2, a1-3g1, a0-3g0, with g1 = d1 + d2);
+//   * the Jiang-Shu smoothness indicator is beta_k = (13/3 a_k^2 + g_k^2) / 4;
+//     the weights are invariant under a common scale of beta, tau and epsilon,
+//     so FP64 works with 4 beta and 4 epsilon;
 //   * the smoothness indicators are shared by both faces (the reversed
 //     stencils' are the same three in reverse order), and so is tau;
 //   * the normalised weights w_k = d_k (1 + tau / e_k) / sum_j (...),
@@ -43,34 +43,34 @@ template <> struct WenoEps<float> { static constexpr float v = 1e-18f; };
 //     the minus face).
 // FP64 multiplies the unnormalised weights by e0 e1 e2 (no reciprocal per
 // stencil): P_k = e0 e1 e2 + tau prod_{j != k} e_j, and one reciprocal of the
-// product of the two faces' denominators serves both faces.  In FP32 these
+// product of the two faces' denominators serves both faces: 51 FP64 operations
+// (61 from scaled second and first differences formed separately: the FP64
+// kernel is bound by its FP64 unit; one 256^3 SSP-RK3 step @@).  In FP32 these
 // products of epsilons underflow (a uniform variable has beta = 0), so FP32
-// takes the reciprocals 1 / e_k and one per face.
+// takes the reciprocals 1 / e_k and one per face, with D_k = a_k / 12 and
+// G_k = g_k / 4.
 __device__ __forceinline__ void wenoz_pair(const double f[5], double& minus, double& plus) {
-  using T = double;
-  const T c12 = T(1.0 / 12.0), q4 = T(0.25), c39 = T(39);
-  const T D0 = c12 * (f[0] + f[2] - T(2) * f[1]);
-  const T D1 = c12 * (f[1] + f[3] - T(2) * f[2]);
-  const T D2 = c12 * (f[2] + f[4] - T(2) * f[3]);
-  const T G0 = q4 * (f[0] - T(4) * f[1] + T(3) * f[2]);
-  const T G1 = q4 * (f[1] - f[3]);
-  const T G2 = q4 * (T(3) * f[2] - T(4) * f[3] + f[4]);
-  const T b0 = c39 * D0 * D0 + G0 * G0;
-  const T b1 = c39 * D1 * D1 + G1 * G1;
-  const T b2 = c39 * D2 * D2 + G2 * G2;
-  const T eps = T(0.25) * WenoEps<T>::v;
-  const T tau = tabs(b0 - b2);
-  const T e0 = b0 + eps, e1 = b1 + eps, e2 = b2 + eps;
-  const T E0 = e1 * e2, E2 = e0 * e1;
-  const T pi = e0 * E0;
-  const T P0 = pi + tau * E0, P1 = pi + tau * (e0 * e2), P2 = pi + tau * E2;
-  const T S1 = T(6) * P1, T0 = T(3) * P0, T2 = T(3) * P2;
-  const T den_p = P0 + S1 + T2, den_m = P2 + S1 + T0;
-  const T num_p = P0 * (D0 + G0) + S1 * (D1 - G1) + T2 * (D2 - G2);
-  const T num_m = P2 * (D2 + G2) + S1 * (D1 + G1) + T0 * (D0 - G0);
-  const T r = rcp(den_p * den_m);
-  plus = f[2] + num_p * den_m * r;
-  minus = f[2] + num_m * den_p * r;
+  const double d0 = f[1] - f[0], d1 = f[2] - f[1], d2 = f[3] - f[2], d3 = f[4] - f[3];
+  const double a0 = d1 - d0, a1 = d2 - d1, a2 = d3 - d2;
+  const double g0 = fma(3.0, d1, -d0), g1 = d1 + d2, g2 = fma(-3.0, d2, d3);
+  constexpr double c = 13.0 / 3.0, eps = 4.0 * WenoEps<double>::v;
+  const double e0 = fma(g0, g0, fma(c * a0, a0, eps));
+  const double e1 = fma(g1, g1, fma(c * a1, a1, eps));
+  const double e2 = fma(g2, g2, fma(c * a2, a2, eps));
+  const double tau = tabs(e0 - e2);
+  const double E0 = e1 * e2, E2 = e0 * e1;
+  const double pi = e0 * E0;
+  // P0, 2 P1, P2: the ideal weights are 1, 3 x 2, 3
+  const double P0 = fma(tau, E0, pi), P2 = fma(tau, E2, pi);
+  const double P1 = bits2d(twice_bits(dbits(fma(tau, e0 * e2, pi))));
+  const double den_p = fma(3.0, P1 + P2, P0), den_m = fma(3.0, P1 + P0, P2);
+  const double num_p = fma(3.0, fma(P1, fma(3.0, g1, a1), P2 * fma(-3.0, g2, a2)),
+                           P0 * fma(3.0, g0, a0));
+  const double num_m = fma(3.0, fma(P1, fma(-3.0, g1, a1), P0 * fma(-3.0, g0, a0)),
+                           P2 * fma(3.0, g2, a2));
+  const double r = rcp(den_p * den_m) * (1.0 / 12.0);
+  plus = fma(num_p, den_m * r, f[2]);
+  minus = fma(num_m, den_p * r, f[2]);
 }
 
 // FP32: two variables at once, the same steps with every operation written out.
