@@ -44,6 +44,7 @@ struct Phys {
   T rho_floor;
   T p_floor;
   double gamma_d, rho_floor_d, p_floor_d;  // FP64 copies for the floor branch
+  T one = T(1), nzero = T(-0.0);  // operands of add_f / sub_f / mul_f
 };
 
 // Single-precision seeds of the FP64 reciprocal and square root below (the
@@ -118,10 +119,23 @@ MHD_HD float mul_rn(float a, float b) {
 }
 MHD_HD double fma_rn(double a, double b, double c) { return fma(a, b, c); }
 MHD_HD float fma_rn(float a, float b, float c) { return fmaf(a, b, c); }
+// Sums, differences and products as fused multiply-adds with the constants 1
+// and -0 (exact, so each rounds once, as the plain operation does).  The FP64
+// unit takes a fused multiply-add with three register operands every 16.8
+// clocks per SM, but an addition, a multiplication or a fused multiply-add with
+// a constant operand only every 19.9.  The kernels therefore hold ph.one and
+// ph.nzero in registers whose values the compiler cannot see (fp64_registers);
+// elsewhere they are plain constants.  FP32 uses the plain operations.
+MHD_HD double add_f(double a, double b, const Phys<double>& ph) { return fma(a, ph.one, b); }
+MHD_HD double sub_f(double a, double b, const Phys<double>& ph) { return fma(-b, ph.one, a); }
+MHD_HD double mul_f(double a, double b, const Phys<double>& ph) { return fma(a, b, ph.nzero); }
+MHD_HD float add_f(float a, float b, const Phys<float>&) { return a + b; }
+MHD_HD float sub_f(float a, float b, const Phys<float>&) { return a - b; }
+MHD_HD float mul_f(float a, float b, const Phys<float>&) { return mul_rn(a, b); }
 // a0 b0 + a1 b1 + a2 b2, rounded as fma(a2, b2, fma(a1, b1, a0 b0))
 template <class T>
-MHD_HD T dot3_rn(T a0, T b0, T a1, T b1, T a2, T b2) {
-  return fma_rn(a2, b2, fma_rn(a1, b1, mul_rn(a0, b0)));
+MHD_HD T dot3_f(T a0, T b0, T a1, T b1, T a2, T b2, const Phys<T>& ph) {
+  return fma_rn(a2, b2, fma_rn(a1, b1, mul_f(a0, b0, ph)));
 }
 
 MHD_HD double trsqrt(double x) { return rsqrt(x); }
@@ -398,6 +412,10 @@ MHD_HD float sqrt_h(float x) {
 #endif
 }
 
+// x / 2 + y: FP64 halves by half_of, FP32 in one fused multiply-add.
+MHD_HD double half_plus(double x, double y, const Phys<double>& ph) { return add_f(half_of(x), y, ph); }
+MHD_HD float half_plus(float x, float y, const Phys<float>&) { return fma_rn(0.5f, x, y); }
+
 // Pressure floor.  FP64: plain comparison.  FP32: when the FP32 pressure is
 // within the cancellation-dominated range (internal energy below 1e-3 of the
 // total, or below the floor) p is recomputed in FP64 from the promoted
@@ -437,10 +455,11 @@ MHD_HD void cons_to_prim(const T u[kNV], T v[kNV], const Phys<T>& ph, unsigned& 
     flags |= kFloorRho;
   }
   const T ri = rcp(rho);
-  const T vx = mul_rn(u[kVX], ri), vy = mul_rn(u[kVY], ri), vz = mul_rn(u[kVZ], ri);
-  const T k2 = dot3_rn(u[kVX], vx, u[kVY], vy, u[kVZ], vz);
-  const T b2 = dot3_rn(u[kBX], u[kBX], u[kBY], u[kBY], u[kBZ], u[kBZ]);
-  T p = mul_rn(ph.gm1, fma_rn(T(-0.5), b2, fma_rn(T(-0.5), k2, u[kPRS])));
+  const T vx = mul_f(u[kVX], ri, ph), vy = mul_f(u[kVY], ri, ph), vz = mul_f(u[kVZ], ri, ph);
+  const T k2 = dot3_f(u[kVX], vx, u[kVY], vy, u[kVZ], vz, ph);
+  const T b2 = dot3_f(u[kBX], u[kBX], u[kBY], u[kBY], u[kBZ], u[kBZ], ph);
+  // gm1 (E - (k2 + b2) / 2)
+  T p = mul_f(ph.gm1, half_plus(-b2, half_plus(-k2, u[kPRS], ph), ph), ph);
   p = pressure_floor(p, u, rho, ph, flags);
   v[kRHO] = rho;
   v[kVX] = vx;
@@ -474,16 +493,17 @@ MHD_HD void prim_to_cons(const T v[kNV], T u[kNV], const Phys<T>& ph) {
 // B_n^2: with g = gamma p / rho, a = g + |B|^2 / rho and c_an^2 = B_n^2 / rho,
 // 2 c_f^2 = a + sqrt(a^2 - 4 g c_an^2).
 template <class T>
-MHD_HD T fast_speed2x(T rho_i, T gp, T b2, T bn2) {
-  const T g = mul_rn(gp, rho_i);
+MHD_HD T fast_speed2x(T rho_i, T gp, T b2, T bn2, const Phys<T>& ph) {
+  const T g = mul_f(gp, rho_i, ph);
   const T a = fma_rn(b2, rho_i, g);
-  return a + sqrt_h(pos_part(fma_rn(a, a, neg4(mul_rn(g, mul_rn(bn2, rho_i))))));
+  const T x = neg4(mul_f(g, mul_f(bn2, rho_i, ph), ph));
+  return add_f(a, sqrt_h(pos_part(fma_rn(a, a, x))), ph);
 }
 
 // Fast magnetosonic speed (see fast_speed2x).
 template <class T>
-MHD_HD T fast_speed(T rho_i, T gp, T b2, T bn2) {
-  return sqrt_h(half_of(fast_speed2x(rho_i, gp, b2, bn2)));
+MHD_HD T fast_speed(T rho_i, T gp, T b2, T bn2, const Phys<T>& ph) {
+  return sqrt_h(half_of(fast_speed2x(rho_i, gp, b2, bn2, ph)));
 }
 
 // max over active directions of |v_d| + c_f,d for one conservative cell.
@@ -493,18 +513,36 @@ MHD_HD T cell_max_speed(const T u[kNV], const Phys<T>& ph, int ndim, unsigned& f
   cons_to_prim(u, v, ph, flags);
   const T ri = rcp(v[kRHO]);
   const T gp = mul_rn(ph.gamma, v[kPRS]);
-  const T b2 = dot3_rn(v[kBX], v[kBX], v[kBY], v[kBY], v[kBZ], v[kBZ]);
-  T lam = tabs(v[kVX]) + fast_speed(ri, gp, b2, mul_rn(v[kBX], v[kBX]));
+  const T b2 = dot3_f(v[kBX], v[kBX], v[kBY], v[kBY], v[kBZ], v[kBZ], ph);
+  T lam = tabs(v[kVX]) + fast_speed(ri, gp, b2, mul_rn(v[kBX], v[kBX]), ph);
   if (ndim > 1)
-    lam = nan_max(lam, tabs(v[kVY]) + fast_speed(ri, gp, b2, mul_rn(v[kBY], v[kBY])));
+    lam = nan_max(lam, tabs(v[kVY]) + fast_speed(ri, gp, b2, mul_rn(v[kBY], v[kBY]), ph));
   if (ndim > 2)
-    lam = nan_max(lam, tabs(v[kVZ]) + fast_speed(ri, gp, b2, mul_rn(v[kBZ], v[kBZ])));
+    lam = nan_max(lam, tabs(v[kVZ]) + fast_speed(ri, gp, b2, mul_rn(v[kBZ], v[kBZ]), ph));
   // NaN anywhere in the cell (psi included) makes the speed NaN
   if (is_nan(v[kPSI]) || is_nan(lam)) lam = T(NAN);
   return lam;
 }
 
 #ifdef __CUDACC__
+// ph.one, ph.nzero, ph.gamma and ph.gm1im1 in registers of unknown value (see
+// add_f): through shared memory, slot[4].  Every thread of the CTA calls it.
+__device__ __forceinline__ void fp64_registers(Phys<double>& ph, double* slot) {
+  if (threadIdx.x == 0) {
+    slot[0] = 1.0;
+    slot[1] = -0.0;
+    slot[2] = ph.gamma;
+    slot[3] = ph.gm1im1;
+  }
+  __syncthreads();
+  const volatile double* v = slot;
+  ph.one = v[0];
+  ph.nzero = v[1];
+  ph.gamma = v[2];
+  ph.gm1im1 = v[3];
+}
+__device__ __forceinline__ void fp64_registers(Phys<float>&, double*) {}
+
 // ---------------------------------------------------------------------------
 // Maximum wave speed of a state (cell_max_speed over all cells): the
 // last-stage epilogue and the wave-speed kernels.  FP32 evaluates every cell.
@@ -680,7 +718,7 @@ MHD_HD float max3(float a, float b, float c) {
   return fmaxf(fmaxf(a, b), c);
 #endif
 }
-MHD_HD float half_slope_mc(float dm, float dp) {
+MHD_HD float half_slope_mc(float dm, float dp, const Phys<float>&) {
   const float c = mul_rn(0.25f, dm + dp);
   return fmaxf(min3(dm, dp, c), 0.0f) + fminf(max3(dm, dp, c), 0.0f);
 }
@@ -689,12 +727,12 @@ MHD_HD float half_slope_minmod(float dm, float dp) {
 }
 // FP64: the same value as half of limited_slope, decided and scaled on the
 // integer pipe; |dm| + |dp| is the only FP64 operation.
-MHD_HD double half_slope_mc(double dm, double dp) {
+MHD_HD double half_slope_mc(double dm, double dp, const Phys<double>& ph) {
   const long long a = dbits(dm), b = dbits(dp);
   const long long mask = 0x7fffffffffffffffll;
   const long long am = a & mask, bm = b & mask;
   const long long mb = am < bm ? am : bm;
-  const long long qr = half_bits(half_bits(dbits(bits2d(am) + bits2d(bm))));
+  const long long qr = half_bits(half_bits(dbits(add_f(bits2d(am), bits2d(bm), ph))));
   const long long h = (qr < mb ? qr : mb) | (a & ~mask);
   return (a ^ b) < 0 || am == 0 || bm == 0 ? 0.0 : bits2d(h);
 }
@@ -731,7 +769,9 @@ MHD_HD T rot3(int dir, int j, T a, T b, T c) {
 template <int dir, class T>
 MHD_HD void glm_hlld_flux(const T vl[kNV], const T vr[kNV], T ch, T half_chi,
                           const Phys<T>& ph, T F[kNV]) {
-  const T half = T(0.5);
+  auto add = [&](T a, T b) { return add_f(a, b, ph); };
+  auto sub = [&](T a, T b) { return sub_f(a, b, ph); };
+  auto mul = [&](T a, T b) { return mul_f(a, b, ph); };
   // rotate: u normal, (v, w) tangential in cyclic order; by, bz likewise
   const T uL = rot3(dir, 0, vl[kVX], vl[kVY], vl[kVZ]);
   const T vL = rot3(dir, 1, vl[kVX], vl[kVY], vl[kVZ]);
@@ -748,27 +788,28 @@ MHD_HD void glm_hlld_flux(const T vl[kNV], const T vr[kNV], T ch, T half_chi,
   const T rL = vl[kRHO], pL = vl[kPRS], rR = vr[kRHO], pR = vr[kPRS];
 
   // GLM: exact solution of the linear (B_n, psi) interface problem
-  const T bx = fma_rn(half, bnL + bnR, mul_rn(-half_chi, vr[kPSI] - vl[kPSI]));
-  const T psis = fma_rn(half, vl[kPSI] + vr[kPSI], mul_rn(T(-0.5) * ch, bnR - bnL));
-  const T bx2 = mul_rn(bx, bx);
+  const T chi = half_chi + half_chi;  // 1 / c_h
+  const T bx = half_of(fma_rn(-chi, sub(vr[kPSI], vl[kPSI]), add(bnL, bnR)));
+  const T psis = half_of(fma_rn(-ch, sub(bnR, bnL), add(vl[kPSI], vr[kPSI])));
+  const T bx2 = mul(bx, bx);
   const T nbx = -bx, nbx2 = -bx2;
 
   // total pressures; c_max, the larger fast speed: one square root of the
   // larger c_f^2 (sqrt is monotone)
   const T b2L = fma_rn(bzL, bzL, fma_rn(byL, byL, bx2));
   const T b2R = fma_rn(bzR, bzR, fma_rn(byR, byR, bx2));
-  const T ptL = fma_rn(half, b2L, pL), ptR = fma_rn(half, b2R, pR);
-  const T cf2L = fast_speed2x(rcp_h(rL), mul_rn(ph.gamma, pL), b2L, bx2);
-  const T cf2R = fast_speed2x(rcp_h(rR), mul_rn(ph.gamma, pR), b2R, bx2);
+  const T ptL = half_plus(b2L, pL, ph), ptR = half_plus(b2R, pR, ph);
+  const T cf2L = fast_speed2x(rcp_h(rL), mul(ph.gamma, pL), b2L, bx2, ph);
+  const T cf2R = fast_speed2x(rcp_h(rR), mul(ph.gamma, pR), b2R, bx2, ph);
   const T cmax = sqrt_h(half_of(tmax2(cf2L, cf2R)));
 
   // wave-speed estimates (MK05 Eq. 67) and contact speed (Eq. 38, written as
   // u_L plus a correction)
-  const T SL = tmin2(uL, uR) - cmax;
-  const T SR = tmax2(uL, uR) + cmax;
-  const T SuL = SL - uL, SuR = SR - uR;
-  const T dL = mul_rn(SuL, rL), dR = mul_rn(SuR, rR);
-  const T SM0 = fma_rn(fma_rn(dR, uR - uL, ptL - ptR), rcp_h(dR - dL), uL);
+  const T SL = sub(tmin2(uL, uR), cmax);
+  const T SR = add(tmax2(uL, uR), cmax);
+  const T SuL = sub(SL, uL), SuR = sub(SR, uR);
+  const T dL = mul(SuL, rL), dR = mul(SuR, rR);
+  const T SM0 = fma_rn(fma_rn(dR, sub(uR, uL), sub(ptL, ptR)), rcp_h(sub(dR, dL)), uL);
 
   // The upwind side a: L if (S_L > 0) or (S_R >= 0 and S_M >= 0), else R
   // (sign tests on the integer pipe in FP64: gt0 / lt0 / ge0); o: the other
@@ -789,28 +830,28 @@ MHD_HD void glm_hlld_flux(const T vl[kNV], const T vr[kNV], T ch, T half_chi,
   // the outer state) when |den| < 1e-8 p_t*, den = rho (S-u)(S-S_M) - Bx^2;
   // p_t* = p_t + rho (S-u)(S_M-u), B* = B (1 + rho (S-u)(S_M-u) / den); one
   // reciprocal for the two divisors
-  const T du = SM - u;
+  const T du = sub(SM, u);
   const T pts = fma_rn(d, du, pt);
-  const T sm = S - SM;
+  const T sm = sub(S, SM);
   const T den = fma_rn(d, sm, nbx2);
-  const T thr = mul_rn(T(1e-8), pts);
+  const T thr = mul(T(1e-8), pts);
   const bool deg = abs_lt(den, thr);
   const T dn = deg ? T(1) : den;
-  const T q = rcp_h(mul_rn(sm, dn));
-  const T smi = mul_rn(dn, q);
-  const T rs = sup ? r : mul_rn(d, smi);
-  const T k0 = deg ? T(0) : mul_rn(du, mul_rn(sm, q));
-  const T fv = mul_rn(nbx, k0), fb = mul_rn(d, k0);
+  const T q = rcp_h(mul(sm, dn));
+  const T smi = mul(dn, q);
+  const T rs = sup ? r : mul(d, smi);
+  const T k0 = deg ? T(0) : mul(du, mul(sm, q));
+  const T fv = mul(nbx, k0), fb = mul(d, k0);
   const T vs = fma_rn(by, fv, v), ws = fma_rn(bz, fv, w);
   const T bys = fma_rn(by, fb, by), bzs = fma_rn(bz, fb, bz);
-  const T vb = dot3_rn(u, bx, v, by, w, bz);
-  const T vbs = dot3_rn(SM, bx, vs, bys, ws, bzs);
+  const T vb = dot3_f(u, bx, v, by, w, bz, ph);
+  const T vbs = dot3_f(SM, bx, vs, bys, ws, bzs, ph);
   // E = rho v^2 / 2 + p / (gamma-1) + B^2 / 2, the last two from p_t; E* (S-S_M)
   // = (S-u) E + (p_t* S_M - p_t u) + Bx (v.B - v*.B*).  (rho / 2 by half_of: an
   // exponent move in FP64, the same value as 0.5 * rho)
-  const T e = fma_rn(half_of(r), dot3_rn(u, u, v, v, w, w), fma_rn(p, ph.gm1im1, pt));
-  const T ns = fma_rn(bx, vb - vbs, fma_rn(Su, e, mul_rn(du, fma_rn(d, SM, pt))));
-  const T es = sup ? e : mul_rn(ns, smi);
+  const T e = fma_rn(half_of(r), dot3_f(u, u, v, v, w, w, ph), fma_rn(p, ph.gm1im1, pt));
+  const T ns = fma_rn(bx, sub(vb, vbs), fma_rn(Su, e, mul(du, fma_rn(d, SM, pt))));
+  const T es = sup ? e : mul(ns, smi);
 
   // Inside the Alfven fan (S*_L <= 0 <= S*_R, Eq. 51: rho* S_M^2 <= B_x^2) the
   // double-star states (Eqs. 59-63).  With s = sign(B_x) on side L and
@@ -818,34 +859,34 @@ MHD_HD void glm_hlld_flux(const T vl[kNV], const T vr[kNV], T ch, T half_chi,
   // of side a: v** = v* + X, B** = B* + s sqrt(rho*) X, X = (sqrt(rho*_o)
   // (v*_o - v*) + s (B*_o - B*)) / (sqrt(rho*) + sqrt(rho*_o)).  Skipped where
   // no lane of the warp is inside the fan.
-  const T ru = mul_rn(rs, SM);
+  const T ru = mul(rs, SM);
   T vF = vs, wF = ws, byF = bys, bzF = bzs, eF = es, vbF = vbs;
-  if (!sup && !lt_ieee(bx2, mul_rn(ru, SM))) {
+  if (!sup && !lt_ieee(bx2, mul(ru, SM))) {
     const T uo = useL ? uR : uL, vo = useL ? vR : vL, wo = useL ? wR : wL;
     const T byo = useL ? byR : byL, bzo = useL ? bzR : bzL;
     const T So = useL ? SR : SL, dO = useL ? dR : dL;
-    const T smo = So - SM;
+    const T smo = sub(So, SM);
     const T deno = fma_rn(dO, smo, nbx2);
     const bool dego = abs_lt(deno, thr);
     const T dno = dego ? T(1) : deno;
-    const T qo = rcp_h(mul_rn(smo, dno));
-    const T rso = mul_rn(dO, mul_rn(dno, qo));
-    const T k0o = dego ? T(0) : mul_rn(SM - uo, mul_rn(smo, qo));
-    const T fvo = mul_rn(nbx, k0o), fbo = mul_rn(dO, k0o);
+    const T qo = rcp_h(mul(smo, dno));
+    const T rso = mul(dO, mul(dno, qo));
+    const T k0o = dego ? T(0) : mul(sub(SM, uo), mul(smo, qo));
+    const T fvo = mul(nbx, k0o), fbo = mul(dO, k0o);
     const T vso = fma_rn(byo, fvo, vo), wso = fma_rn(bzo, fvo, wo);
     const T byso = fma_rn(byo, fbo, byo), bzso = fma_rn(bzo, fbo, bzo);
     const T sqa = sqrt_h(rs), sqo = sqrt_h(rso);
-    const T isum = rcp_h(sqa + sqo);
+    const T isum = rcp_h(add(sqa, sqo));
     const auto sg = sign_of(ge0(bx) != useL, T(0));
-    const T Xv = mul_rn(fma_rn(sqo, vso - vs, sign_mul(byso - bys, sg)), isum);
-    const T Xw = mul_rn(fma_rn(sqo, wso - ws, sign_mul(bzso - bzs, sg)), isum);
+    const T Xv = mul(fma_rn(sqo, sub(vso, vs), sign_mul(sub(byso, bys), sg)), isum);
+    const T Xw = mul(fma_rn(sqo, sub(wso, ws), sign_mul(sub(bzso, bzs), sg)), isum);
     const T sqs = sign_mul(sqa, sg);
-    vF = vs + Xv;
-    wF = ws + Xw;
+    vF = add(vs, Xv);
+    wF = add(ws, Xw);
     byF = fma_rn(sqs, Xv, bys);
     bzF = fma_rn(sqs, Xw, bzs);
-    vbF = dot3_rn(SM, bx, vF, byF, wF, bzF);
-    eF = fma_rn(sqs, vbF - vbs, es);
+    vbF = dot3_f(SM, bx, vF, byF, wF, bzF, ph);
+    eF = fma_rn(sqs, sub(vbF, vbs), es);
   }
 
   // HLLD's fan fluxes F_a + S_a (U*_a - U_a) + S*_a (U**_a - U*_a) (Eqs.
@@ -853,19 +894,19 @@ MHD_HD void glm_hlld_flux(const T vl[kNV], const T vr[kNV], T ch, T half_chi,
   // flux of the state on the interface with normal velocity S_M and total
   // pressure p_t* -- except the induction terms of a degenerate star state,
   // which keeps B* = B: there B (u - S_M) is left over.
-  const T f1 = fma_rn(ru, SM, pts + nbx2);
-  const T f2 = fma_rn(ru, vF, mul_rn(nbx, byF));
-  const T f3 = fma_rn(ru, wF, mul_rn(nbx, bzF));
-  T f4 = fma_rn(byF, SM, mul_rn(nbx, vF));
-  T f5 = fma_rn(bzF, SM, mul_rn(nbx, wF));
+  const T f1 = fma_rn(ru, SM, add(pts, nbx2));
+  const T f2 = fma_rn(ru, vF, mul(nbx, byF));
+  const T f3 = fma_rn(ru, wF, mul(nbx, bzF));
+  T f4 = fma_rn(byF, SM, mul(nbx, vF));
+  T f5 = fma_rn(bzF, SM, mul(nbx, wF));
   if (deg) {
     f4 = fma_rn(-by, du, f4);
     f5 = fma_rn(-bz, du, f5);
   }
 
   F[kRHO] = ru;
-  F[kPRS] = fma_rn(eF + pts, SM, mul_rn(nbx, vbF));
-  F[kPSI] = mul_rn(mul_rn(ch, ch), bx);
+  F[kPRS] = fma_rn(add(eF, pts), SM, mul(nbx, vbF));
+  F[kPSI] = mul(ch, mul(ch, bx));
   // un-rotate: component m of a vector gets rotated slot j = (m - dir) mod 3
 #pragma unroll
   for (int m = 0; m < 3; ++m) {

@@ -242,25 +242,26 @@ struct TileGeom {
 // sh apart.
 template <class T>
 __device__ __forceinline__ void cell_slopes(const T* m, int sm, const T* c, int sc, const T* p,
-                                            int sp, int lim, T* h, int sh) {
+                                            int sp, int lim, const Phys<T>& ph, T* h, int sh) {
   T sig[kNV];
   if (lim == kLimMC) {
 #pragma unroll
     for (int k = 0; k < kNV; ++k) {
       const T q = c[k * sc];
-      sig[k] = half_slope_mc(q - m[k * sm], p[k * sp] - q);
+      sig[k] = half_slope_mc(sub_f(q, m[k * sm], ph), sub_f(p[k * sp], q, ph), ph);
     }
   } else if (lim == kLimMinmod) {
 #pragma unroll
     for (int k = 0; k < kNV; ++k) {
       const T q = c[k * sc];
-      sig[k] = half_slope_minmod(q - m[k * sm], p[k * sp] - q);
+      sig[k] = half_slope_minmod(sub_f(q, m[k * sm], ph), sub_f(p[k * sp], q, ph));
     }
   } else {
 #pragma unroll
     for (int k = 0; k < kNV; ++k) sig[k] = T(0);
   }
-  const bool ok = gt0(c[kRHO * sc] - tabs(sig[kRHO])) && gt0(c[kPRS * sc] - tabs(sig[kPRS]));
+  const bool ok = gt0(sub_f(c[kRHO * sc], tabs(sig[kRHO]), ph)) &&
+                  gt0(sub_f(c[kPRS * sc], tabs(sig[kPRS]), ph));
   if (!ok) {
 #pragma unroll
     for (int k = 0; k < kNV; ++k) sig[k] = T(0);
@@ -270,7 +271,8 @@ __device__ __forceinline__ void cell_slopes(const T* m, int sm, const T* c, int 
 }
 
 // One tile (bx, by, bz) of one RK stage; called by every thread of a CTA of
-// NW warps.  smem_raw: TileGeom::WORDS elements of T; wmax: NW doubles.
+// NW warps.  smem_raw: TileGeom::WORDS elements of T; wmax: NW doubles,
+// konst (FP64): 4 doubles.
 // CT (constrained transport, 3-D only): face-normal fields from p.bw, only
 // rho, m and E are updated (psi is written as 0; the magnetic field is left to
 // the face update), the face / cell electric fields go to p.ctf, and the last
@@ -279,7 +281,7 @@ __device__ __forceinline__ void cell_slopes(const T* m, int sm, const T* c, int 
 template <class T, int TY, int NW, int STAGE, bool ZACT, bool CT = false, bool HALO = false>
 __device__ __forceinline__ void stage_tile(const StageParams<T>& p, const StepScalars& sc,
                                            int bx, int by, int bz, unsigned char* smem_raw,
-                                           double* wmax) {
+                                           double* wmax, double* konst = nullptr) {
   using G = TileGeom<TY, ZACT>;
   constexpr int NT = NW * 32;
   constexpr int TX = G::TX;
@@ -315,7 +317,13 @@ __device__ __forceinline__ void stage_tile(const StageParams<T>& p, const StepSc
   // even where fluxes are not finite
   const bool frozen = !(sc.dt != 0.0);
   const int lim = p.limiter;
-  const Phys<T> ph = p.ph;
+  Phys<T> ph = p.ph;
+  if constexpr (NW > 1) {
+    fp64_registers(ph, konst);
+  } else {  // one-warp 1-D kernels wait for latency: the plain operations
+    ph.one = T(1);
+    ph.nzero = T(-0.0);
+  }
   unsigned flags = 0;  // of the wave-speed conversions (not counted)
 
   auto slot = [](int zz) { return ZACT ? ((zz % 3) + 3) % 3 : 0; };
@@ -437,11 +445,11 @@ __device__ __forceinline__ void stage_tile(const StageParams<T>& p, const StepSc
         dst = sys + j;
         ds = G::SYN;
       }
-      cell_slopes(m, G::PS, c, G::PS, pp, G::PS, lim, dst, ds);
+      cell_slopes(m, G::PS, c, G::PS, pp, G::PS, lim, ph, dst, ds);
     }
     if (ZACT && owner)
       cell_slopes(cur + oidx, G::PS, ring_plane(k + 1) + oidx, G::PS, ring_plane(k + 2) + oidx,
-                  G::PS, lim, zS + oidx, G::NINT);
+                  G::PS, lim, ph, zS + oidx, G::NINT);
     __syncthreads();
 
     // ---- C: fluxes --------------------------------------------------------
@@ -465,8 +473,8 @@ __device__ __forceinline__ void stage_tile(const StageParams<T>& p, const StepSc
         const T* gb = ga + 1;                        // half slope of cell fi
 #pragma unroll
         for (int q = 0; q < kNV; ++q) {
-          vl[q] = a[q * G::PS] + ga[q * G::SXN];
-          vr[q] = b[q * G::PS] - gb[q * G::SXN];
+          vl[q] = add_f(a[q * G::PS], ga[q * G::SXN], ph);
+          vr[q] = sub_f(b[q * G::PS], gb[q * G::SXN], ph);
         }
         if constexpr (CT) ct_face_field(vl, vr, 0, bface(0, k, r, fi));
         out = Fx + r * (TX + 1) + fi;
@@ -480,8 +488,8 @@ __device__ __forceinline__ void stage_tile(const StageParams<T>& p, const StepSc
         const T* gb = ga + TX;                       // half slope of row fj
 #pragma unroll
         for (int q = 0; q < kNV; ++q) {
-          vl[q] = a[q * G::PS] + ga[q * G::SYN];
-          vr[q] = b[q * G::PS] - gb[q * G::SYN];
+          vl[q] = add_f(a[q * G::PS], ga[q * G::SYN], ph);
+          vr[q] = sub_f(b[q * G::PS], gb[q * G::SYN], ph);
         }
         if constexpr (CT) ct_face_field(vl, vr, 1, bface(1, k, fj, c));
         out = Fy + j;
@@ -503,7 +511,7 @@ __device__ __forceinline__ void stage_tile(const StageParams<T>& p, const StepSc
 #pragma unroll
         for (int q = 0; q < kNV; ++q) {
           vl[q] = zP[q * G::NINT + oidx];
-          vr[q] = c[q * G::PS] - zS[q * G::NINT + oidx];
+          vr[q] = sub_f(c[q * G::PS], zS[q * G::NINT + oidx], ph);
         }
         if constexpr (CT) {
           ct_face_field(vl, vr, 2, bface(2, k + 1, orow, ocol));
@@ -516,13 +524,13 @@ __device__ __forceinline__ void stage_tile(const StageParams<T>& p, const StepSc
           glm_hlld_flux<2>(vl, vr, ch, half_chi, ph, F);
 #pragma unroll
           for (int q = 0; q < kNV; ++q) {
-            dUz[q] = F[q] - zF[q * G::NINT + oidx];
+            dUz[q] = sub_f(F[q], zF[q * G::NINT + oidx], ph);
             zF[q * G::NINT + oidx] = F[q];
           }
         }
 #pragma unroll
         for (int q = 0; q < kNV; ++q)
-          zP[q * G::NINT + oidx] = c[q * G::PS] + zS[q * G::NINT + oidx];
+          zP[q * G::NINT + oidx] = add_f(c[q * G::PS], zS[q * G::NINT + oidx], ph);
       }
     }
     __syncthreads();
@@ -541,18 +549,25 @@ __device__ __forceinline__ void stage_tile(const StageParams<T>& p, const StepSc
           const T* fx = Fx + q * G::FXN + orow * (TX + 1) + ocol;
           // sums of products with their rounding fixed (mul_rn / fma_rn), so
           // every instantiation of this tile code gives the same bits
-          T du = mul_rn(fx[1] - fx[0], dtdx);
+          T du = mul_f(sub_f(fx[1], fx[0], ph), dtdx, ph);
           if constexpr (G::GY > 0) {
             const T* fy = Fy + q * G::FYN + orow * TX + ocol;
-            du = fma_rn(fy[TX] - fy[0], dtdy, du);
+            du = fma_rn(sub_f(fy[TX], fy[0], ph), dtdy, du);
           }
           if constexpr (ZACT) du = fma_rn(dUz[q], dtdz, du);
           if (frozen) du = T(0);
-          const T s1 = p.win[q * p.sv + off] - du;
-          if constexpr (STAGE == 1) {
-            unew[q] = s1;
+          unew[q] = sub_f(p.win[q * p.sv + off], du, ph);
+        }
+        if constexpr (STAGE != 1) {
+          // RK2: (U^n + s) / 2, the same value with one operation less
+          if (p.a_n == T(0.5) && p.a_w == T(0.5)) {
+#pragma unroll
+            for (int q = 0; q < kNV; ++q)
+              unew[q] = half_of(add_f(p.un[q * p.sv + off], unew[q], ph));
           } else {
-            unew[q] = fma_rn(p.a_n, p.un[q * p.sv + off], mul_rn(p.a_w, s1));
+#pragma unroll
+            for (int q = 0; q < kNV; ++q)
+              unew[q] = fma_rn(p.a_n, p.un[q * p.sv + off], mul_f(p.a_w, unew[q], ph));
           }
         }
         if constexpr (CT) {
@@ -601,9 +616,10 @@ __global__ void __launch_bounds__(NW * 32, sizeof(T) == 4 && ZACT ? 2 : 1)
     rk_stage_kernel(const StageParams<T> p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ double wmax[NW];
+  __shared__ double konst[4];
   const StepScalars sc = *p.sc;
   stage_tile<T, TY, NW, STAGE, ZACT, CT, HALO>(p, sc, blockIdx.x, blockIdx.y, blockIdx.z,
-                                               smem_raw, wmax);
+                                               smem_raw, wmax, konst);
 }
 
 }  // namespace mhd

@@ -44,33 +44,55 @@ template <> struct WenoEps<float> { static constexpr float v = 1e-18f; };
 // FP64 multiplies the unnormalised weights by e0 e1 e2 (no reciprocal per
 // stencil): P_k = e0 e1 e2 + tau prod_{j != k} e_j, and one reciprocal of the
 // product of the two faces' denominators serves both faces: 51 FP64 operations
-// (61 from scaled second and first differences formed separately: the FP64
-// kernel is bound by its FP64 unit; one 256^3 SSP-RK3 step @@).  In FP32 these
+// (61 from scaled second and first differences formed separately: one SSP-RK3
+// step of a 256^3 box 277 -> 223 ms; with the register operands of add_f 205).  In FP32 these
 // products of epsilons underflow (a uniform variable has beta = 0), so FP32
 // takes the reciprocals 1 / e_k and one per face, with D_k = a_k / 12 and
 // G_k = g_k / 4.
-__device__ __forceinline__ void wenoz_pair(const double f[5], double& minus, double& plus) {
-  const double d0 = f[1] - f[0], d1 = f[2] - f[1], d2 = f[3] - f[2], d3 = f[4] - f[3];
-  const double a0 = d1 - d0, a1 = d2 - d1, a2 = d3 - d2;
-  const double g0 = fma(3.0, d1, -d0), g1 = d1 + d2, g2 = fma(-3.0, d2, d3);
-  constexpr double c = 13.0 / 3.0, eps = 4.0 * WenoEps<double>::v;
-  const double e0 = fma(g0, g0, fma(c * a0, a0, eps));
-  const double e1 = fma(g1, g1, fma(c * a1, a1, eps));
-  const double e2 = fma(g2, g2, fma(c * a2, a2, eps));
-  const double tau = tabs(e0 - e2);
-  const double E0 = e1 * e2, E2 = e0 * e1;
-  const double pi = e0 * E0;
+// Constants of the FP64 form; the kernel holds them in registers (see add_f).
+template <class T>
+struct WenoConst {
+  __device__ explicit WenoConst(const double*) {}
+};
+template <>
+struct WenoConst<double> {
+  double three, c, eps, i12;
+  __device__ explicit WenoConst(const volatile double* v)
+      : three(v[0]), c(v[1]), eps(v[2]), i12(v[3]) {}
+  __device__ static void fill(double* v) {
+    v[0] = 3.0;
+    v[1] = 13.0 / 3.0;
+    v[2] = 4.0 * WenoEps<double>::v;
+    v[3] = 1.0 / 12.0;
+  }
+};
+__device__ __forceinline__ void wenoz_pair(const double f[5], const Phys<double>& ph,
+                                           const WenoConst<double>& w, double& minus,
+                                           double& plus) {
+  auto add = [&](double a, double b) { return add_f(a, b, ph); };
+  auto sub = [&](double a, double b) { return sub_f(a, b, ph); };
+  auto mul = [&](double a, double b) { return mul_f(a, b, ph); };
+  const double d0 = sub(f[1], f[0]), d1 = sub(f[2], f[1]), d2 = sub(f[3], f[2]);
+  const double d3 = sub(f[4], f[3]);
+  const double a0 = sub(d1, d0), a1 = sub(d2, d1), a2 = sub(d3, d2);
+  const double g0 = fma(w.three, d1, -d0), g1 = add(d1, d2), g2 = fma(w.three, -d2, d3);
+  const double e0 = fma(g0, g0, fma(mul(w.c, a0), a0, w.eps));
+  const double e1 = fma(g1, g1, fma(mul(w.c, a1), a1, w.eps));
+  const double e2 = fma(g2, g2, fma(mul(w.c, a2), a2, w.eps));
+  const double tau = tabs(sub(e0, e2));
+  const double E0 = mul(e1, e2), E2 = mul(e0, e1);
+  const double pi = mul(e0, E0);
   // P0, 2 P1, P2: the ideal weights are 1, 3 x 2, 3
   const double P0 = fma(tau, E0, pi), P2 = fma(tau, E2, pi);
-  const double P1 = bits2d(twice_bits(dbits(fma(tau, e0 * e2, pi))));
-  const double den_p = fma(3.0, P1 + P2, P0), den_m = fma(3.0, P1 + P0, P2);
-  const double num_p = fma(3.0, fma(P1, fma(3.0, g1, a1), P2 * fma(-3.0, g2, a2)),
-                           P0 * fma(3.0, g0, a0));
-  const double num_m = fma(3.0, fma(P1, fma(-3.0, g1, a1), P0 * fma(-3.0, g0, a0)),
-                           P2 * fma(3.0, g2, a2));
-  const double r = rcp(den_p * den_m) * (1.0 / 12.0);
-  plus = fma(num_p, den_m * r, f[2]);
-  minus = fma(num_m, den_p * r, f[2]);
+  const double P1 = bits2d(twice_bits(dbits(fma(tau, mul(e0, e2), pi))));
+  const double den_p = fma(w.three, add(P1, P2), P0), den_m = fma(w.three, add(P1, P0), P2);
+  const double num_p = fma(w.three, fma(P1, fma(w.three, g1, a1), mul(P2, fma(-w.three, g2, a2))),
+                           mul(P0, fma(w.three, g0, a0)));
+  const double num_m = fma(w.three, fma(P1, fma(-w.three, g1, a1), mul(P0, fma(-w.three, g0, a0))),
+                           mul(P2, fma(w.three, g2, a2)));
+  const double r = mul(rcp(mul(den_p, den_m)), w.i12);
+  plus = fma(num_p, mul(den_m, r), f[2]);
+  minus = fma(num_m, mul(den_p, r), f[2]);
 }
 
 // FP32: two variables at once, the same steps with every operation written out.
@@ -102,8 +124,9 @@ __device__ __forceinline__ void wenoz_pair(const f2 f[5], f2& minus, f2& plus) {
 // (variables stride[j] apart); flat fallback on non-positive face density
 // or pressure.  FP32 reconstructs the variables in pairs (0, 1) ... (6, 7).
 template <class T>
-__device__ __forceinline__ void cell_weno(const T* const c[5], const int st[5], T M[kNV],
-                                          T P[kNV]) {
+__device__ __forceinline__ void cell_weno(const T* const c[5], const int st[5],
+                                          const Phys<T>& ph, const WenoConst<T>& w,
+                                          T M[kNV], T P[kNV]) {
   if constexpr (sizeof(T) == 4) {
 #pragma unroll
     for (int k = 0; k + 1 < kNV; k += 2) {
@@ -128,7 +151,7 @@ __device__ __forceinline__ void cell_weno(const T* const c[5], const int st[5], 
       T f[5];
 #pragma unroll
       for (int j = 0; j < 5; ++j) f[j] = c[j][k * st[j]];
-      wenoz_pair(f, M[k], P[k]);
+      wenoz_pair(f, ph, w, M[k], P[k]);
     }
   }
   const bool ok = gt0(M[kRHO]) && gt0(P[kRHO]) && gt0(M[kPRS]) && gt0(P[kPRS]);
@@ -204,7 +227,17 @@ __global__ void __launch_bounds__(NW * 32, sizeof(T) == 4 && ZACT ? 2 : 1)
   const T dtdx = T(sc.dtdx[0]), dtdy = T(sc.dtdx[1]), dtdz = T(sc.dtdx[2]);
   const T damp = T(sc.damp);
   const bool frozen = !(sc.dt != 0.0);
-  const Phys<T> ph = p.ph;
+  __shared__ double konst[8];
+  Phys<T> ph = p.ph;
+  if constexpr (sizeof(T) == 8) {
+    if (threadIdx.x == 0) WenoConst<T>::fill(konst + 4);
+  }
+  fp64_registers(ph, konst);  // (synchronises)
+  if constexpr (NW == 1) {  // one-warp 1-D kernels wait for latency: the plain operations
+    ph.one = T(1);
+    ph.nzero = T(-0.0);
+  }
+  const WenoConst<T> wk(konst + 4);
   unsigned flags = 0;  // of the wave-speed conversions (not counted)
 
   auto slot = [](int zz) { return ZACT ? ((zz % 5) + 5) % 5 : 0; };
@@ -286,7 +319,7 @@ __global__ void __launch_bounds__(NW * 32, sizeof(T) == 4 && ZACT ? 2 : 1)
       c[j] = ring_plane(zc - 2 + j) + oidx;
       st[j] = G::NINT;
     }
-    cell_weno(c, st, M, P);
+    cell_weno(c, st, ph, wk, M, P);
   };
 
   // The z march: one loop body for every plane (see stage_tile in
@@ -333,7 +366,7 @@ __global__ void __launch_bounds__(NW * 32, sizeof(T) == 4 && ZACT ? 2 : 1)
         dP = yP + j0;
         ds = G::SYN;
       }
-      cell_weno(c, st, M, P);
+      cell_weno(c, st, ph, wk, M, P);
 #pragma unroll
       for (int q = 0; q < kNV; ++q) {
         dM[q * ds] = M[q];
@@ -415,7 +448,7 @@ __global__ void __launch_bounds__(NW * 32, sizeof(T) == 4 && ZACT ? 2 : 1)
           glm_hlld_flux<2>(vl, vr, ch, half_chi, ph, F);
 #pragma unroll
           for (int q = 0; q < kNV; ++q) {
-            dUz[q] = F[q] - zF[q * G::NINT + oidx];
+            dUz[q] = sub_f(F[q], zF[q * G::NINT + oidx], ph);
             zF[q * G::NINT + oidx] = F[q];
           }
         }
@@ -439,18 +472,25 @@ __global__ void __launch_bounds__(NW * 32, sizeof(T) == 4 && ZACT ? 2 : 1)
           const T* fx = Fx + q * G::FXN + orow * (TX + 1) + ocol;
           // sums of products with their rounding fixed (mul_rn / fma_rn), so
           // every instantiation of this tile code gives the same bits
-          T du = mul_rn(fx[1] - fx[0], dtdx);
+          T du = mul_f(sub_f(fx[1], fx[0], ph), dtdx, ph);
           if constexpr (G::GY > 0) {
             const T* fy = Fy + q * G::FYN + orow * TX + ocol;
-            du = fma_rn(fy[TX] - fy[0], dtdy, du);
+            du = fma_rn(sub_f(fy[TX], fy[0], ph), dtdy, du);
           }
           if constexpr (ZACT) du = fma_rn(dUz[q], dtdz, du);
           if (frozen) du = T(0);
-          const T s1 = p.win[q * p.sv + off] - du;
-          if constexpr (STAGE == 1) {
-            unew[q] = s1;
+          unew[q] = sub_f(p.win[q * p.sv + off], du, ph);
+        }
+        if constexpr (STAGE != 1) {
+          // RK2: (U^n + s) / 2, the same value with one operation less
+          if (p.a_n == T(0.5) && p.a_w == T(0.5)) {
+#pragma unroll
+            for (int q = 0; q < kNV; ++q)
+              unew[q] = half_of(add_f(p.un[q * p.sv + off], unew[q], ph));
           } else {
-            unew[q] = fma_rn(p.a_n, p.un[q * p.sv + off], mul_rn(p.a_w, s1));
+#pragma unroll
+            for (int q = 0; q < kNV; ++q)
+              unew[q] = fma_rn(p.a_n, p.un[q * p.sv + off], mul_f(p.a_w, unew[q], ph));
           }
         }
         if constexpr (CT) {
