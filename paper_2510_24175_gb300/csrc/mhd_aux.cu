@@ -15,7 +15,7 @@ Phys<T> make_phys(const Grid& g) {
   ph.gm1im1 = T(1.0 / (g.gamma - 1.0) - 1.0);
   ph.rho_floor = T(g.rho_floor);
   ph.p_floor = T(g.p_floor);
-  ph.gamma_d = g.gamma;
+  ph.gm1_d = g.gamma - 1.0;
   ph.rho_floor_d = g.rho_floor;
   ph.p_floor_d = g.p_floor;
   return ph;

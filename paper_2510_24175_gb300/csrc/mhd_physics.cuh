@@ -43,7 +43,7 @@ struct Phys {
   T gm1im1;     // 1 / (gamma - 1) - 1
   T rho_floor;
   T p_floor;
-  double gamma_d, rho_floor_d, p_floor_d;  // FP64 copies for the floor branch
+  double gm1_d, rho_floor_d, p_floor_d;  // FP64 gamma - 1 and floors for the floor branch
   T one = T(1), nzero = T(-0.0);  // operands of add_f / sub_f / mul_f
 };
 
@@ -432,10 +432,18 @@ MHD_HD float pressure_floor(float p, const float u[kNV], float rho,
                                                 const Phys<float>& ph, unsigned& flags) {
   if (p < ph.p_floor || p < 1e-3f * ph.gm1 * u[kPRS]) {
     flags |= kPressF64;
-    double r = rho;
-    double m2 = (double)u[kVX] * u[kVX] + (double)u[kVY] * u[kVY] + (double)u[kVZ] * u[kVZ];
-    double b2 = (double)u[kBX] * u[kBX] + (double)u[kBY] * u[kBY] + (double)u[kBZ] * u[kBZ];
-    double pd = (ph.gamma_d - 1.0) * ((double)u[kPRS] - 0.5 * m2 / r - 0.5 * b2);
+    // (volatile, so that no part of the branch is evaluated for every cell: one
+    // FP64 instruction holds the SM's FP64 unit for 16 clocks)
+    double e;
+#ifdef __CUDA_ARCH__
+    asm volatile("cvt.f64.f32 %0, %1;" : "=d"(e) : "f"(u[kPRS]));
+#else
+    e = u[kPRS];
+#endif
+    const double r = rho;
+    const double m2 = (double)u[kVX] * u[kVX] + (double)u[kVY] * u[kVY] + (double)u[kVZ] * u[kVZ];
+    const double b2 = (double)u[kBX] * u[kBX] + (double)u[kBY] * u[kBY] + (double)u[kBZ] * u[kBZ];
+    const double pd = ph.gm1_d * (e - 0.5 * m2 / r - 0.5 * b2);
     if (pd < ph.p_floor_d) {
       flags |= kFloorP;
       return ph.p_floor;

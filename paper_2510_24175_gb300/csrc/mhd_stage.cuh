@@ -544,6 +544,12 @@ __device__ __forceinline__ void stage_tile(const StageParams<T>& p, const StepSc
       for (int q = 0; q < kNV; ++q) unew[q] = T(0);
       if (valid) {
         const long long off = (long long)k * p.sz + (long long)gy * p.sy + gx;
+        T W[kNV], un[kNV];  // (loads first: their latency is the phase's)
+#pragma unroll
+        for (int q = 0; q < kNV; ++q) {
+          W[q] = p.win[q * p.sv + off];
+          if constexpr (STAGE != 1) un[q] = p.un[q * p.sv + off];
+        }
 #pragma unroll
         for (int q = 0; q < kNV; ++q) {
           const T* fx = Fx + q * G::FXN + orow * (TX + 1) + ocol;
@@ -556,18 +562,18 @@ __device__ __forceinline__ void stage_tile(const StageParams<T>& p, const StepSc
           }
           if constexpr (ZACT) du = fma_rn(dUz[q], dtdz, du);
           if (frozen) du = T(0);
-          unew[q] = sub_f(p.win[q * p.sv + off], du, ph);
+          unew[q] = sub_f(W[q], du, ph);
         }
         if constexpr (STAGE != 1) {
           // RK2: (U^n + s) / 2, the same value with one operation less
           if (p.a_n == T(0.5) && p.a_w == T(0.5)) {
 #pragma unroll
             for (int q = 0; q < kNV; ++q)
-              unew[q] = half_of(add_f(p.un[q * p.sv + off], unew[q], ph));
+              unew[q] = half_of(add_f(un[q], unew[q], ph));
           } else {
 #pragma unroll
             for (int q = 0; q < kNV; ++q)
-              unew[q] = fma_rn(p.a_n, p.un[q * p.sv + off], mul_f(p.a_w, unew[q], ph));
+              unew[q] = fma_rn(p.a_n, un[q], mul_f(p.a_w, unew[q], ph));
           }
         }
         if constexpr (CT) {
@@ -612,7 +618,7 @@ __device__ __forceinline__ void stage_tile(const StageParams<T>& p, const StepSc
 }
 
 template <class T, int TY, int NW, int STAGE, bool ZACT, bool CT, bool HALO = false>
-__global__ void __launch_bounds__(NW * 32, sizeof(T) == 4 && ZACT ? 2 : 1)
+__global__ void __launch_bounds__(NW * 32, 1)
     rk_stage_kernel(const StageParams<T> p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ double wmax[NW];

@@ -3,6 +3,7 @@
 #pragma once
 
 #include "mhd_internal.h"
+#include "mhd_stage_pairs.cuh"
 #include "mhd_stage_weno.cuh"
 
 namespace mhd {
@@ -49,6 +50,37 @@ static cudaError_t launch_one(const StageParams<T>& p, dim3 grid, cudaStream_t s
   return cudaGetLastError();
 }
 
+// 3-D PLM: FP64 stage_tile(), FP32 stage_tile_pairs() (mhd_stage_pairs.cuh).
+template <class T, int STAGE, bool CT, bool HALO>
+struct Plm3D {
+  using S = StageShape3D<T>;
+  static constexpr auto kernel = rk_stage_kernel<T, S::TY, S::NW, STAGE, true, CT, HALO>;
+  static constexpr size_t smem = (size_t)TileGeom<S::TY, true>::WORDS * sizeof(T);
+};
+template <int STAGE, bool CT, bool HALO>
+struct Plm3D<float, STAGE, CT, HALO> {
+  using S = StageShape3D<float>;
+  static constexpr auto kernel = rk_stage_pairs_kernel<S::TY, S::NW, STAGE, CT, HALO>;
+  static constexpr size_t smem = (size_t)PairGeom<S::TY>::WORDS * sizeof(float);
+};
+template <class T, int STAGE, bool CT = false, bool HALO = false>
+static cudaError_t launch_plm3(const StageParams<T>& p, const Grid& g, int nzc, cudaStream_t s) {
+  using K = Plm3D<T, STAGE, CT, HALO>;
+  using S = StageShape3D<T>;
+  cudaError_t e = set_smem_once<K::kernel>(K::smem);
+  if (e != cudaSuccess) return e;
+  const dim3 grid((g.n[0] + 31) / 32, (g.n[1] + S::TY - 1) / S::TY, nzc);
+  K::kernel<<<grid, S::NW * 32, K::smem, s>>>(p);
+  return cudaGetLastError();
+}
+// The FP32 kernels without halo faces address a plane with 32 bits; larger planes
+// take the halo-capable ones.  (With constrained transport such a grid needs
+// over 300 GB: it never reaches a launch.)
+template <class T>
+static bool wide_plane(const Grid& g) {
+  return sizeof(T) == 4 && (long long)g.n[0] * g.n[1] * 4 >= (1ll << 32);
+}
+
 template <class T, int TY, int NW, int STAGE, bool ZACT, bool CT = false, bool HALO = false>
 static cudaError_t launch_weno(const StageParams<T>& p, dim3 grid, cudaStream_t s) {
   using G = WenoGeom<TY, ZACT>;
@@ -93,7 +125,7 @@ void stage_shape(const Grid& g, size_t* smem, int* threads, int* ty) {
   }
   if (g.ndim == 3) {
     using S = StageShape3D<T>;
-    *smem = (size_t)TileGeom<S::TY, true>::WORDS * sizeof(T);
+    *smem = Plm3D<T, 1, false, false>::smem;
     *threads = S::NW * 32;
     *ty = S::TY;
   } else if (g.ndim == 2) {
@@ -120,22 +152,27 @@ cudaError_t prepare_stage_kernels(const Grid& g, bool ct) {
   MHD_SET1(KERN, G, TY_, NW_, 1, Z_, CT_);     \
   MHD_SET1(KERN, G, TY_, NW_, 2, Z_, CT_);     \
   MHD_SET1(KERN, G, TY_, NW_, 3, Z_, CT_)
-  using S = StageShape3D<T>;
   using WS = WenoShape3D<T>;
   using W3 = WenoGeom<WS::TY, true>;
   using W2 = WenoGeom<4, false>;
   using W1 = WenoGeom<1, false>;
-  using P3 = TileGeom<S::TY, true>;
+#define MHD_SET3D(CT_)                                                           \
+  if (e == cudaSuccess)                                                          \
+    e = set_smem_once<Plm3D<T, 1, CT_, false>::kernel>(Plm3D<T, 1, CT_, false>::smem); \
+  if (e == cudaSuccess)                                                          \
+    e = set_smem_once<Plm3D<T, 2, CT_, false>::kernel>(Plm3D<T, 2, CT_, false>::smem); \
+  if (e == cudaSuccess)                                                          \
+  e = set_smem_once<Plm3D<T, 3, CT_, false>::kernel>(Plm3D<T, 3, CT_, false>::smem)
   using P2 = TileGeom<8, false>;
   using P1 = TileGeom<1, false>;
   if (ct) {
     if (g.limiter == kLimWenoz) {
       MHD_SET3(rk_stage_weno_kernel, W3, WS::TY, WS::NW, true, true);
     } else {
-      MHD_SET3(rk_stage_kernel, P3, S::TY, S::NW, true, true);
+      MHD_SET3D(true);
     }
-  } else if (sizeof(T) == 8 && g.ndim == 3) {
-    e = prepare_stage_kernels_halo<T>(g);  // FP64 3-D GLM: the halo-capable kernels
+  } else if (g.ndim == 3 && (sizeof(T) == 8 || (wide_plane<T>(g) && g.limiter != kLimWenoz))) {
+    e = prepare_stage_kernels_halo<T>(g);  // the halo-capable kernels (see launch_stage)
   } else if (g.limiter == kLimWenoz) {
     if (g.ndim == 3) {
       if constexpr (sizeof(T) == 4) {
@@ -148,13 +185,14 @@ cudaError_t prepare_stage_kernels(const Grid& g, bool ct) {
     }
   } else if (g.ndim == 3) {
     if constexpr (sizeof(T) == 4) {
-      MHD_SET3(rk_stage_kernel, P3, S::TY, S::NW, true, false);
+      MHD_SET3D(false);
     }
   } else if (g.ndim == 2) {
     MHD_SET3(rk_stage_kernel, P2, 8, 8, false, false);
   } else {
     MHD_SET3(rk_stage_kernel, P1, 1, 1, false, false);
   }
+#undef MHD_SET3D
 #undef MHD_SET3
 #undef MHD_SET1
   return e;
@@ -223,11 +261,9 @@ cudaError_t launch_stage(const Grid& g, int stage, const T* win, const T* un, T*
       if (stage == 2) return launch_weno<T, WS::TY, WS::NW, 2, true, true>(p, grid, stream);
       return launch_weno<T, WS::TY, WS::NW, 3, true, true>(p, grid, stream);
     }
-    using S = StageShape3D<T>;
-    dim3 grid((g.n[0] + 31) / 32, (g.n[1] + S::TY - 1) / S::TY, nzc);
-    if (stage == 1) return launch_one<T, S::TY, S::NW, 1, true, true>(p, grid, stream);
-    if (stage == 2) return launch_one<T, S::TY, S::NW, 2, true, true>(p, grid, stream);
-    return launch_one<T, S::TY, S::NW, 3, true, true>(p, grid, stream);
+    if (stage == 1) return launch_plm3<T, 1, true>(p, g, nzc, stream);
+    if (stage == 2) return launch_plm3<T, 2, true>(p, g, nzc, stream);
+    return launch_plm3<T, 3, true>(p, g, nzc, stream);
   }
   if constexpr (sizeof(T) == 8) {
     // FP64 3-D GLM: always the halo-capable kernels (no halo faces here), so
@@ -259,11 +295,12 @@ cudaError_t launch_stage(const Grid& g, int stage, const T* win, const T* un, T*
   }
   if constexpr (sizeof(T) == 4) {
     if (g.ndim == 3) {
-      using S = StageShape3D<T>;
-      dim3 grid((g.n[0] + 31) / 32, (g.n[1] + S::TY - 1) / S::TY, nzc);
-      if (stage == 1) return launch_one<T, S::TY, S::NW, 1, true>(p, grid, stream);
-      if (stage == 2) return launch_one<T, S::TY, S::NW, 2, true>(p, grid, stream);
-      return launch_one<T, S::TY, S::NW, 3, true>(p, grid, stream);
+      if (wide_plane<T>(g))
+        return launch_stage_halo<T>(g, stage, win, un, uout, sc, lam_bits, floor_cnt, stream, a_n,
+                                    a_w, nullptr, est_bits, zlo, zhi, tz);
+      if (stage == 1) return launch_plm3<T, 1>(p, g, nzc, stream);
+      if (stage == 2) return launch_plm3<T, 2>(p, g, nzc, stream);
+      return launch_plm3<T, 3>(p, g, nzc, stream);
     }
   }
   if (g.ndim == 2) {
@@ -307,30 +344,25 @@ cudaError_t launch_stage_halo(const Grid& g, int stage, const T* win, const T* u
     if (stage == 2) return launch_weno<T, WS::TY, WS::NW, 2, true, false, true>(p, grid, stream);
     return launch_weno<T, WS::TY, WS::NW, 3, true, false, true>(p, grid, stream);
   }
-  using S = StageShape3D<T>;
-  dim3 grid((g.n[0] + 31) / 32, (g.n[1] + S::TY - 1) / S::TY, nzc);
-  if (stage == 1) return launch_one<T, S::TY, S::NW, 1, true, false, true>(p, grid, stream);
-  if (stage == 2) return launch_one<T, S::TY, S::NW, 2, true, false, true>(p, grid, stream);
-  return launch_one<T, S::TY, S::NW, 3, true, false, true>(p, grid, stream);
+  if (stage == 1) return launch_plm3<T, 1, false, true>(p, g, nzc, stream);
+  if (stage == 2) return launch_plm3<T, 2, false, true>(p, g, nzc, stream);
+  return launch_plm3<T, 3, false, true>(p, g, nzc, stream);
 }
 
 // The shared-memory limits of the HALO variants (set once, outside any capture).
 template <class T>
 cudaError_t prepare_stage_kernels_halo(const Grid& g) {
   cudaError_t e = cudaSuccess;
-  using S = StageShape3D<T>;
   using WS = WenoShape3D<T>;
-  using W3 = WenoGeom<WS::TY, true>;
-  using P3 = TileGeom<S::TY, true>;
-  const size_t sw = (size_t)W3::WORDS * sizeof(T), sp = (size_t)P3::WORDS * sizeof(T);
+  const size_t sw = (size_t)WenoGeom<WS::TY, true>::WORDS * sizeof(T);
   if (g.limiter == kLimWenoz) {
     if (e == cudaSuccess) e = set_smem_once<rk_stage_weno_kernel<T, WS::TY, WS::NW, 1, true, false, true>>(sw);
     if (e == cudaSuccess) e = set_smem_once<rk_stage_weno_kernel<T, WS::TY, WS::NW, 2, true, false, true>>(sw);
     if (e == cudaSuccess) e = set_smem_once<rk_stage_weno_kernel<T, WS::TY, WS::NW, 3, true, false, true>>(sw);
   } else {
-    if (e == cudaSuccess) e = set_smem_once<rk_stage_kernel<T, S::TY, S::NW, 1, true, false, true>>(sp);
-    if (e == cudaSuccess) e = set_smem_once<rk_stage_kernel<T, S::TY, S::NW, 2, true, false, true>>(sp);
-    if (e == cudaSuccess) e = set_smem_once<rk_stage_kernel<T, S::TY, S::NW, 3, true, false, true>>(sp);
+    if (e == cudaSuccess) e = set_smem_once<Plm3D<T, 1, false, true>::kernel>(Plm3D<T, 1, false, true>::smem);
+    if (e == cudaSuccess) e = set_smem_once<Plm3D<T, 2, false, true>::kernel>(Plm3D<T, 2, false, true>::smem);
+    if (e == cudaSuccess) e = set_smem_once<Plm3D<T, 3, false, true>::kernel>(Plm3D<T, 3, false, true>::smem);
   }
   return e;
 }
