@@ -410,9 +410,9 @@ int mhd_fp64_fma_rate(void* stream, unsigned warp_mask, double out[3]);
 
 /* Launch planning, on the host only (no GPU, no CUDA call): the z-chunk depth
  * *tz (planes per CTA) that the 3-D stage launches of an n[0] x n[1] x n[2]
- * grid use, for column tiles of 32 x ty cells (ty: 8 for the PLM kernels, 4
- * for WENO-Z) on nsm SMs holding ctas_per_sm stage CTAs each (1 for FP64, 2
- * for FP32), and, if span is not
+ * grid use, for column tiles of 32 x ty cells (ty: 8, or 4 for FP64
+ * WENO-Z) on nsm SMs holding ctas_per_sm stage CTAs each (1 for FP64, 2 for
+ * FP32), and, if span is not
  * NULL, the modelled duration of one launch in plane iterations.  The model:
  * the CTAs start in launch order -- every column tile's full chunks, then
  * every column tile's last, possibly shorter, chunk -- each on the slot that

@@ -111,7 +111,7 @@ __device__ __forceinline__ void ens_stage(const EnsArgs& a, unsigned char* smem,
     const int bx = (int)(j % B.ntx);
     const int by = (int)((j / B.ntx) % B.nty);
     const int bz = (int)(j / ((long long)B.ntx * B.nty));
-    stage_tile_pairs<TY, kEnsNW, STAGE, false, false>(
+    stage_tile_pairs<TY, kEnsNW, STAGE, false, false, false>(
         p, sc, bx, by, bz, reinterpret_cast<float*>(smem), wmax);
   }
 }
@@ -353,8 +353,8 @@ int mhd_ensemble_create(const mhd_config* cfgs, int nbox, void* d_workspace, siz
   cudaError_t ce = cudaMemsetAsync(e->d, 0, sizeof(EnsBox) * nbox, e->stream);
   // both instantiations: shared-memory limit and co-resident CTAs per SM
   // (the cooperative grid size)
-  e->smem[0] = (size_t)mhd::PairGeom<8>::WORDS * sizeof(float);
-  e->smem[1] = (size_t)mhd::PairGeom<4>::WORDS * sizeof(float);
+  e->smem[0] = (size_t)mhd::PairGeom<8, false>::WORDS * sizeof(float);
+  e->smem[1] = (size_t)mhd::PairGeom<4, false>::WORDS * sizeof(float);
   int per_sm[2] = {0, 0}, nsm = 0, dev = 0;
   if (ce == cudaSuccess)
     ce = cudaFuncSetAttribute(mhd::ensemble_kernel<8>,

@@ -8,19 +8,19 @@
 
 namespace mhd {
 
-// Tile shapes: 3-D grids use 32 x 8 column tiles marching in z with 16 warps
-// per CTA (8 helper warps, 8 column owners).  FP64: one CTA per SM (211 KB of
-// shared memory); the SM's FP64 unit is shared by all its warps and one warp
-// issues an FP64 instruction at most every 64 clocks, so the unit saturates
-// only when at least four warps have FP64 work.  FP32: two CTAs per SM at 64
-// registers, 32 warps: the kernel is bound by latency and issue, and with 24
-// and 16 warps per SM (80 and 128 registers) it took 56.3 and 59.4 ms against
-// 55.1 for two steps of a 512^3 box.  2-D grids use the same tile with a single
-// plane; 1-D grids a 32-cell row.
-template <class T>
+// Tile shapes of 3-D grids: column tiles of 32 x TY cells marching in z.  FP64:
+// one CTA per SM, PLM 32 x 8 with 16 warps (211 KB of shared memory), WENO-Z 32 x
+// 4 with 8 warps (167 KB); the SM's FP64 unit is shared by all its warps and one
+// warp issues an FP64 instruction at most every 64 clocks, so the unit saturates
+// only when at least four warps have FP64 work.  FP32 (PLM and WENO-Z): 32 x 8
+// with 16 warps at 64 registers, two CTAs per SM: the kernels are bound by
+// latency and issue; with 24 and 16 warps per SM the PLM kernel took 2 and 8 %
+// longer (512^3).  2-D grids use the 32 x 8 (PLM) or 32 x 4 (WENO-Z) tile with a
+// single plane; 1-D grids a 32-cell row.
+template <class T, bool WENO>
 struct StageShape3D {
-  static constexpr int TY = 8;
-    static constexpr int NW = 16;
+  static constexpr int TY = sizeof(T) == 8 && WENO ? 4 : 8;
+  static constexpr int NW = sizeof(T) == 8 && WENO ? 8 : 16;
 };
 
 // The dynamic shared-memory limit of a kernel is set once per device (a
@@ -50,28 +50,51 @@ static cudaError_t launch_one(const StageParams<T>& p, dim3 grid, cudaStream_t s
   return cudaGetLastError();
 }
 
-// 3-D PLM: FP64 stage_tile(), FP32 stage_tile_pairs() (mhd_stage_pairs.cuh).
-template <class T, int STAGE, bool CT, bool HALO>
-struct Plm3D {
-  using S = StageShape3D<T>;
-  static constexpr auto kernel = rk_stage_kernel<T, S::TY, S::NW, STAGE, true, CT, HALO>;
-  static constexpr size_t smem = (size_t)TileGeom<S::TY, true>::WORDS * sizeof(T);
+// The 3-D stage kernels: FP64 rk_stage_kernel / rk_stage_weno_kernel, FP32
+// rk_stage_pairs_kernel (mhd_stage_pairs.cuh).
+template <class T, bool WENO, int STAGE, bool CT, bool HALO>
+struct Kern3D {
+  using S = StageShape3D<T, WENO>;
+  static constexpr auto get() {
+    if constexpr (sizeof(T) == 4)
+      return rk_stage_pairs_kernel<S::TY, S::NW, STAGE, CT, HALO, WENO>;
+    else if constexpr (WENO)
+      return rk_stage_weno_kernel<T, S::TY, S::NW, STAGE, true, CT, HALO>;
+    else
+      return rk_stage_kernel<T, S::TY, S::NW, STAGE, true, CT, HALO>;
+  }
+  static constexpr size_t words() {
+    if constexpr (sizeof(T) == 4)
+      return PairGeom<S::TY, WENO>::WORDS;
+    else if constexpr (WENO)
+      return WenoGeom<S::TY, true>::WORDS;
+    else
+      return TileGeom<S::TY, true>::WORDS;
+  }
+  static constexpr auto kernel = get();
+  static constexpr size_t smem = words() * sizeof(T);
+  static cudaError_t prepare() { return set_smem_once<kernel>(smem); }
+  static cudaError_t launch(const StageParams<T>& p, const Grid& g, int nzc, cudaStream_t s) {
+    cudaError_t e = prepare();
+    if (e != cudaSuccess) return e;
+    const dim3 grid((g.n[0] + 31) / 32, (g.n[1] + S::TY - 1) / S::TY, nzc);
+    kernel<<<grid, S::NW * 32, smem, s>>>(p);
+    return cudaGetLastError();
+  }
 };
-template <int STAGE, bool CT, bool HALO>
-struct Plm3D<float, STAGE, CT, HALO> {
-  using S = StageShape3D<float>;
-  static constexpr auto kernel = rk_stage_pairs_kernel<S::TY, S::NW, STAGE, CT, HALO>;
-  static constexpr size_t smem = (size_t)PairGeom<S::TY>::WORDS * sizeof(float);
-};
-template <class T, int STAGE, bool CT = false, bool HALO = false>
-static cudaError_t launch_plm3(const StageParams<T>& p, const Grid& g, int nzc, cudaStream_t s) {
-  using K = Plm3D<T, STAGE, CT, HALO>;
-  using S = StageShape3D<T>;
-  cudaError_t e = set_smem_once<K::kernel>(K::smem);
-  if (e != cudaSuccess) return e;
-  const dim3 grid((g.n[0] + 31) / 32, (g.n[1] + S::TY - 1) / S::TY, nzc);
-  K::kernel<<<grid, S::NW * 32, K::smem, s>>>(p);
-  return cudaGetLastError();
+template <class T, bool WENO, bool CT, bool HALO>
+static cudaError_t launch_3d(int stage, const StageParams<T>& p, const Grid& g, int nzc,
+                             cudaStream_t s) {
+  if (stage == 1) return Kern3D<T, WENO, 1, CT, HALO>::launch(p, g, nzc, s);
+  if (stage == 2) return Kern3D<T, WENO, 2, CT, HALO>::launch(p, g, nzc, s);
+  return Kern3D<T, WENO, 3, CT, HALO>::launch(p, g, nzc, s);
+}
+template <class T, bool WENO, bool CT, bool HALO>
+static cudaError_t prepare_3d() {
+  cudaError_t e = Kern3D<T, WENO, 1, CT, HALO>::prepare();
+  if (e == cudaSuccess) e = Kern3D<T, WENO, 2, CT, HALO>::prepare();
+  if (e == cudaSuccess) e = Kern3D<T, WENO, 3, CT, HALO>::prepare();
+  return e;
 }
 // The FP32 kernels without halo faces address a plane with 32 bits; larger planes
 // take the halo-capable ones.  (With constrained transport such a grid needs
@@ -92,26 +115,14 @@ static cudaError_t launch_weno(const StageParams<T>& p, dim3 grid, cudaStream_t 
   return cudaGetLastError();
 }
 
-// WENO-Z tiles of 3-D grids: 32 x 4 columns.  FP64: 8 warps (the face-value
-// phase gives every warp two cells' worth of work), one CTA per SM (167 KB of
-// shared memory).  FP32: 16 warps and two CTAs per SM at 64 registers; three
-// steps of a 256^3 box with constrained transport take 36.5 ms, 38.0 and 39.6
-// with 24 and 16 warps per SM, and 40.6 on 32 x 8 tiles with one CTA of 16 warps.
-// 2-D grids use 32 x 4 tiles with a single plane.
-template <class T>
-struct WenoShape3D {
-  static constexpr int TY = 4;
-  static constexpr int NW = sizeof(T) == 8 ? 8 : 16;
-};
-
 template <class T>
 void stage_shape(const Grid& g, size_t* smem, int* threads, int* ty) {
   if (g.limiter == kLimWenoz) {
     if (g.ndim == 3) {
-      using WS = WenoShape3D<T>;
-      *smem = (size_t)WenoGeom<WS::TY, true>::WORDS * sizeof(T);
-      *threads = WS::NW * 32;
-      *ty = WS::TY;
+      using K = Kern3D<T, true, 1, false, false>;
+      *smem = K::smem;
+      *threads = K::S::NW * 32;
+      *ty = K::S::TY;
     } else if (g.ndim == 2) {
       *smem = (size_t)WenoGeom<4, false>::WORDS * sizeof(T);
       *threads = 256;
@@ -124,10 +135,10 @@ void stage_shape(const Grid& g, size_t* smem, int* threads, int* ty) {
     return;
   }
   if (g.ndim == 3) {
-    using S = StageShape3D<T>;
-    *smem = Plm3D<T, 1, false, false>::smem;
-    *threads = S::NW * 32;
-    *ty = S::TY;
+    using K = Kern3D<T, false, 1, false, false>;
+    *smem = K::smem;
+    *threads = K::S::NW * 32;
+    *ty = K::S::TY;
   } else if (g.ndim == 2) {
     *smem = (size_t)TileGeom<8, false>::WORDS * sizeof(T);
     *threads = 8 * 32;
@@ -144,55 +155,35 @@ void stage_shape(const Grid& g, size_t* smem, int* threads, int* ty) {
 // driver call later, e.g. while a stream is being captured.
 template <class T>
 cudaError_t prepare_stage_kernels(const Grid& g, bool ct) {
+  const bool weno = g.limiter == kLimWenoz;
+  if (ct) return weno ? prepare_3d<T, true, true, false>() : prepare_3d<T, false, true, false>();
+  if (g.ndim == 3) {
+    // FP64, and planes beyond 32-bit offsets: the halo-capable kernels (launch_stage)
+    if (sizeof(T) == 8 || wide_plane<T>(g)) return prepare_stage_kernels_halo<T>(g);
+    if constexpr (sizeof(T) == 4)
+      return weno ? prepare_3d<T, true, false, false>() : prepare_3d<T, false, false, false>();
+  }
   cudaError_t e = cudaSuccess;
-  // the three stages of one variant <TY, NW, 3-D, CT> with geometry G
-#define MHD_SET1(KERN, G, TY_, NW_, S_, Z_, CT_) \
-  if (e == cudaSuccess) e = set_smem_once<KERN<T, TY_, NW_, S_, Z_, CT_>>((size_t)G::WORDS * sizeof(T))
-#define MHD_SET3(KERN, G, TY_, NW_, Z_, CT_)   \
-  MHD_SET1(KERN, G, TY_, NW_, 1, Z_, CT_);     \
-  MHD_SET1(KERN, G, TY_, NW_, 2, Z_, CT_);     \
-  MHD_SET1(KERN, G, TY_, NW_, 3, Z_, CT_)
-  using WS = WenoShape3D<T>;
-  using W3 = WenoGeom<WS::TY, true>;
+  // the three stages of one variant <TY, NW> with geometry G
+#define MHD_SET1(KERN, G, TY_, NW_, S_) \
+  if (e == cudaSuccess) e = set_smem_once<KERN<T, TY_, NW_, S_, false, false>>((size_t)G::WORDS * sizeof(T))
+#define MHD_SET3(KERN, G, TY_, NW_) \
+  MHD_SET1(KERN, G, TY_, NW_, 1);   \
+  MHD_SET1(KERN, G, TY_, NW_, 2);   \
+  MHD_SET1(KERN, G, TY_, NW_, 3)
   using W2 = WenoGeom<4, false>;
   using W1 = WenoGeom<1, false>;
-#define MHD_SET3D(CT_)                                                           \
-  if (e == cudaSuccess)                                                          \
-    e = set_smem_once<Plm3D<T, 1, CT_, false>::kernel>(Plm3D<T, 1, CT_, false>::smem); \
-  if (e == cudaSuccess)                                                          \
-    e = set_smem_once<Plm3D<T, 2, CT_, false>::kernel>(Plm3D<T, 2, CT_, false>::smem); \
-  if (e == cudaSuccess)                                                          \
-  e = set_smem_once<Plm3D<T, 3, CT_, false>::kernel>(Plm3D<T, 3, CT_, false>::smem)
   using P2 = TileGeom<8, false>;
   using P1 = TileGeom<1, false>;
-  if (ct) {
-    if (g.limiter == kLimWenoz) {
-      MHD_SET3(rk_stage_weno_kernel, W3, WS::TY, WS::NW, true, true);
-    } else {
-      MHD_SET3D(true);
-    }
-  } else if (g.ndim == 3 && (sizeof(T) == 8 || (wide_plane<T>(g) && g.limiter != kLimWenoz))) {
-    e = prepare_stage_kernels_halo<T>(g);  // the halo-capable kernels (see launch_stage)
-  } else if (g.limiter == kLimWenoz) {
-    if (g.ndim == 3) {
-      if constexpr (sizeof(T) == 4) {
-        MHD_SET3(rk_stage_weno_kernel, W3, WS::TY, WS::NW, true, false);
-      }
-    } else if (g.ndim == 2) {
-      MHD_SET3(rk_stage_weno_kernel, W2, 4, 8, false, false);
-    } else {
-      MHD_SET3(rk_stage_weno_kernel, W1, 1, 1, false, false);
-    }
-  } else if (g.ndim == 3) {
-    if constexpr (sizeof(T) == 4) {
-      MHD_SET3D(false);
-    }
+  if (weno && g.ndim == 2) {
+    MHD_SET3(rk_stage_weno_kernel, W2, 4, 8);
+  } else if (weno) {
+    MHD_SET3(rk_stage_weno_kernel, W1, 1, 1);
   } else if (g.ndim == 2) {
-    MHD_SET3(rk_stage_kernel, P2, 8, 8, false, false);
+    MHD_SET3(rk_stage_kernel, P2, 8, 8);
   } else {
-    MHD_SET3(rk_stage_kernel, P1, 1, 1, false, false);
+    MHD_SET3(rk_stage_kernel, P1, 1, 1);
   }
-#undef MHD_SET3D
 #undef MHD_SET3
 #undef MHD_SET1
   return e;
@@ -254,34 +245,21 @@ cudaError_t launch_stage(const Grid& g, int stage, const T* win, const T* un, T*
   if (ctf) {
     // constrained transport: 3-D grids only (checked when the context is made)
     if (g.ndim != 3 || !bw) return cudaErrorInvalidValue;
-    if (g.limiter == kLimWenoz) {
-      using WS = WenoShape3D<T>;
-      dim3 grid((g.n[0] + 31) / 32, (g.n[1] + WS::TY - 1) / WS::TY, nzc);
-      if (stage == 1) return launch_weno<T, WS::TY, WS::NW, 1, true, true>(p, grid, stream);
-      if (stage == 2) return launch_weno<T, WS::TY, WS::NW, 2, true, true>(p, grid, stream);
-      return launch_weno<T, WS::TY, WS::NW, 3, true, true>(p, grid, stream);
-    }
-    if (stage == 1) return launch_plm3<T, 1, true>(p, g, nzc, stream);
-    if (stage == 2) return launch_plm3<T, 2, true>(p, g, nzc, stream);
-    return launch_plm3<T, 3, true>(p, g, nzc, stream);
+    return g.limiter == kLimWenoz ? launch_3d<T, true, true, false>(stage, p, g, nzc, stream)
+                                  : launch_3d<T, false, true, false>(stage, p, g, nzc, stream);
   }
-  if constexpr (sizeof(T) == 8) {
-    // FP64 3-D GLM: always the halo-capable kernels (no halo faces here), so
-    // that a grid and the blocks of its decomposition run the same code
-    if (g.ndim == 3)
+  if (g.ndim == 3) {
+    // FP64 GLM: always the halo-capable kernels (no halo faces here), so that a
+    // grid and the blocks of its decomposition run the same code; FP32 where a
+    // plane is too large for 32-bit offsets
+    if (sizeof(T) == 8 || wide_plane<T>(g))
       return launch_stage_halo<T>(g, stage, win, un, uout, sc, lam_bits, floor_cnt, stream, a_n,
                                   a_w, nullptr, est_bits, zlo, zhi, tz);
+    if constexpr (sizeof(T) == 4)
+      return g.limiter == kLimWenoz ? launch_3d<T, true, false, false>(stage, p, g, nzc, stream)
+                                    : launch_3d<T, false, false, false>(stage, p, g, nzc, stream);
   }
   if (g.limiter == kLimWenoz) {
-    if constexpr (sizeof(T) == 4) {
-      if (g.ndim == 3) {
-        using WS = WenoShape3D<T>;
-        dim3 grid((g.n[0] + 31) / 32, (g.n[1] + WS::TY - 1) / WS::TY, nzc);
-        if (stage == 1) return launch_weno<T, WS::TY, WS::NW, 1, true>(p, grid, stream);
-        if (stage == 2) return launch_weno<T, WS::TY, WS::NW, 2, true>(p, grid, stream);
-        return launch_weno<T, WS::TY, WS::NW, 3, true>(p, grid, stream);
-      }
-    }
     if (g.ndim == 2) {
       dim3 grid((g.n[0] + 31) / 32, (g.n[1] + 3) / 4, 1);
       if (stage == 1) return launch_weno<T, 4, 8, 1, false>(p, grid, stream);
@@ -292,16 +270,6 @@ cudaError_t launch_stage(const Grid& g, int stage, const T* win, const T* un, T*
     if (stage == 1) return launch_weno<T, 1, 1, 1, false>(p, grid, stream);
     if (stage == 2) return launch_weno<T, 1, 1, 2, false>(p, grid, stream);
     return launch_weno<T, 1, 1, 3, false>(p, grid, stream);
-  }
-  if constexpr (sizeof(T) == 4) {
-    if (g.ndim == 3) {
-      if (wide_plane<T>(g))
-        return launch_stage_halo<T>(g, stage, win, un, uout, sc, lam_bits, floor_cnt, stream, a_n,
-                                    a_w, nullptr, est_bits, zlo, zhi, tz);
-      if (stage == 1) return launch_plm3<T, 1>(p, g, nzc, stream);
-      if (stage == 2) return launch_plm3<T, 2>(p, g, nzc, stream);
-      return launch_plm3<T, 3>(p, g, nzc, stream);
-    }
   }
   if (g.ndim == 2) {
     dim3 grid((g.n[0] + 31) / 32, (g.n[1] + 7) / 8, 1);
@@ -337,34 +305,15 @@ cudaError_t launch_stage_halo(const Grid& g, int stage, const T* win, const T* u
     p.halo[f] = bc == kBcHalo ? halo[f] : nullptr;
   }
   const int nzc = (p.zhi - p.zlo + p.tz - 1) / p.tz;
-  if (g.limiter == kLimWenoz) {
-    using WS = WenoShape3D<T>;
-    dim3 grid((g.n[0] + 31) / 32, (g.n[1] + WS::TY - 1) / WS::TY, nzc);
-    if (stage == 1) return launch_weno<T, WS::TY, WS::NW, 1, true, false, true>(p, grid, stream);
-    if (stage == 2) return launch_weno<T, WS::TY, WS::NW, 2, true, false, true>(p, grid, stream);
-    return launch_weno<T, WS::TY, WS::NW, 3, true, false, true>(p, grid, stream);
-  }
-  if (stage == 1) return launch_plm3<T, 1, false, true>(p, g, nzc, stream);
-  if (stage == 2) return launch_plm3<T, 2, false, true>(p, g, nzc, stream);
-  return launch_plm3<T, 3, false, true>(p, g, nzc, stream);
+  return g.limiter == kLimWenoz ? launch_3d<T, true, false, true>(stage, p, g, nzc, stream)
+                                : launch_3d<T, false, false, true>(stage, p, g, nzc, stream);
 }
 
 // The shared-memory limits of the HALO variants (set once, outside any capture).
 template <class T>
 cudaError_t prepare_stage_kernels_halo(const Grid& g) {
-  cudaError_t e = cudaSuccess;
-  using WS = WenoShape3D<T>;
-  const size_t sw = (size_t)WenoGeom<WS::TY, true>::WORDS * sizeof(T);
-  if (g.limiter == kLimWenoz) {
-    if (e == cudaSuccess) e = set_smem_once<rk_stage_weno_kernel<T, WS::TY, WS::NW, 1, true, false, true>>(sw);
-    if (e == cudaSuccess) e = set_smem_once<rk_stage_weno_kernel<T, WS::TY, WS::NW, 2, true, false, true>>(sw);
-    if (e == cudaSuccess) e = set_smem_once<rk_stage_weno_kernel<T, WS::TY, WS::NW, 3, true, false, true>>(sw);
-  } else {
-    if (e == cudaSuccess) e = set_smem_once<Plm3D<T, 1, false, true>::kernel>(Plm3D<T, 1, false, true>::smem);
-    if (e == cudaSuccess) e = set_smem_once<Plm3D<T, 2, false, true>::kernel>(Plm3D<T, 2, false, true>::smem);
-    if (e == cudaSuccess) e = set_smem_once<Plm3D<T, 3, false, true>::kernel>(Plm3D<T, 3, false, true>::smem);
-  }
-  return e;
+  return g.limiter == kLimWenoz ? prepare_3d<T, true, false, true>()
+                                : prepare_3d<T, false, false, true>();
 }
 
 }  // namespace mhd

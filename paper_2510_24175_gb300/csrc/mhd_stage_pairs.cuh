@@ -1,10 +1,11 @@
-// Fused Runge-Kutta stage of 3-D FP32 grids with PLM: the phases of
-// stage_tile() (mhd_stage.cuh) on 32 x TY column tiles, arranged for the FP32
-// kernel's bounds, instruction issue and shared-memory wavefronts:
+// Fused Runge-Kutta stage of 3-D FP32 grids: the phases of stage_tile()
+// (mhd_stage.cuh) and of the WENO-Z kernel (mhd_stage_weno.cuh) on 32 x 8 column
+// tiles, arranged for the FP32 kernels' bounds, latency, instruction issue and
+// shared-memory wavefronts:
 //   * the nine variables of a cell are kept as four pairs and one value (rho
 //     vx | vy vz | Bx By | Bz p | psi), so that a cell moves in five shared-
-//     memory instructions and the slopes, face states and updates run on packed
-//     pairs;
+//     memory instructions and slopes, WENO-Z values, face states and updates run
+//     on packed pairs;
 //   * phase B stores a cell's lower and upper face states instead of its slope,
 //     and a face's flux overwrites the lower state that only that face reads (45
 //     shared-memory values per face instead of 54, and no flux arrays);
@@ -16,17 +17,20 @@
 #pragma once
 
 #include "mhd_stage.cuh"
+#include "mhd_wenoz.cuh"
 
 namespace mhd {
 
-template <int TY>
+template <int TY, bool WENO>
 struct PairGeom {
   static constexpr int TX = 32;
+  static constexpr int GH = WENO ? 3 : 2;  // ghost width
+  static constexpr int NR = WENO ? 5 : 3;  // ring planes
   static constexpr int NINT = TY * TX;
-  static constexpr int NXH = 4 * TY;  // x halo: columns -2, -1, 32, 33
-  static constexpr int NYH = 4 * TX;  // y halo: rows -2, -1, TY, TY+1
+  static constexpr int NXH = 2 * GH * TY;  // x halo: columns -GH..-1, 32..31+GH
+  static constexpr int NYH = 2 * GH * TX;  // y halo: rows -GH..-1, TY..TY+GH-1
   static constexpr int PS = NINT > NXH + NYH ? NINT : NXH + NYH;  // cells of a set
-  static constexpr int RING = 3 * kNV * PS;
+  static constexpr int RING = NR * kNV * PS;
   static constexpr int HB = kNV * PS;
   static constexpr int XN = TY * (TX + 1);  // x faces
   static constexpr int YN = (TY + 1) * TX;  // y faces
@@ -129,13 +133,56 @@ __device__ __forceinline__ void face_pair(const float m[kNV], const float q[kNV]
   add9(q, h, hi);
 }
 
+// Face values of a cell from the cells at(j) (base, index) along a direction, j =
+// 0 the cell itself: PLM (WENO = false) or WENO-Z, with the flat fallback on
+// a non-positive face density or pressure.
+template <bool WENO, int PS, class At>
+__device__ __forceinline__ void face_states(At at, int lim, float lo[kNV], float hi[kNV]) {
+  if constexpr (!WENO) {
+    float m[kNV], q[kNV], n[kNV];
+    const auto cm = at(-1), cq = at(0), cn = at(1);
+    ld9<PS>(cm.b, cm.i, m);
+    ld9<PS>(cq.b, cq.i, q);
+    ld9<PS>(cn.b, cn.i, n);
+    face_pair(m, q, n, lim, lo, hi);
+  } else {
+    decltype(at(0)) c[5] = {at(-2), at(-1), at(0), at(1), at(2)};
+#pragma unroll
+    for (int n = 0; n < 4; ++n) {
+      f2 f[5], a, b;
+#pragma unroll
+      for (int j = 0; j < 5; ++j) f[j] = f2(reinterpret_cast<const float2*>(c[j].b)[n * PS + c[j].i]);
+      wenoz_pair(f, a, b);
+      lo[2 * n] = a.v.x;
+      lo[2 * n + 1] = a.v.y;
+      hi[2 * n] = b.v.x;
+      hi[2 * n + 1] = b.v.y;
+    }
+    f2 f[5], a, b;
+#pragma unroll
+    for (int j = 0; j < 5; ++j) f[j] = f2(c[j].b[8 * PS + c[j].i]);
+    wenoz_pair(f, a, b);
+    lo[8] = a.v.x;
+    hi[8] = b.v.x;
+    if (!(lo[kRHO] > 0.0f && hi[kRHO] > 0.0f && lo[kPRS] > 0.0f && hi[kPRS] > 0.0f)) {
+      ld9<PS>(c[2].b, c[2].i, lo);
+#pragma unroll
+      for (int k = 0; k < kNV; ++k) hi[k] = lo[k];
+    }
+  }
+}
+struct CellRef {  // cell i of the set at b
+  const float* b;
+  int i;
+};
+
 // One tile (bx, by, bz) of one RK stage (see stage_tile()); smem: PairGeom words.
-template <int TY, int NW, int STAGE, bool CT, bool HALO>
+template <int TY, int NW, int STAGE, bool CT, bool HALO, bool WENO>
 __device__ __forceinline__ void stage_tile_pairs(const StageParams<float>& p,
                                                  const StepScalars& sc, int bx, int by, int bz,
                                                  float* smem, double* wmax) {
-  using G = PairGeom<TY>;
-  constexpr int NT = NW * 32, TX = G::TX, PS = G::PS, NI = G::NINT;
+  using G = PairGeom<TY, WENO>;
+  constexpr int NT = NW * 32, TX = G::TX, PS = G::PS, NI = G::NINT, GH = G::GH;
   constexpr int ZT0 = NT - NI;  // threads ZT0.. own one tile column each
   constexpr int NA = (G::NLOAD + NT - 1) / NT;
   static_assert(ZT0 >= 0, "need one thread per tile column");
@@ -164,15 +211,18 @@ __device__ __forceinline__ void stage_tile_pairs(const StageParams<float>& p,
   unsigned flags = 0;  // of the wave-speed conversions (not counted)
   SpeedMax<float> smax(ph);
 
-  auto ring_plane = [&](int zz) { return ring + ((zz + 6) % 3) * (kNV * PS); };
+  auto ring_plane = [&](int zz) { return ring + ((zz + 2 * G::NR) % G::NR) * (kNV * PS); };
+  auto wrap = [](int i, int n, int lo, int hi) {
+    return GH == 2 ? remap(i, n, lo, hi) : remap3(i, n, lo, hi);
+  };
   // in-plane offset of tile cell (r, c), remapped into the grid, in bytes
   auto plane_off = [&](int r, int c) {
-    const int gx = remap(x0 + c, nx, p.bc_lo[0], p.bc_hi[0]);
-    const int gy = remap(y0 + r, ny, p.bc_lo[1], p.bc_hi[1]);
+    const int gx = wrap(x0 + c, nx, p.bc_lo[0], p.bc_hi[0]);
+    const int gy = wrap(y0 + r, ny, p.bc_lo[1], p.bc_hi[1]);
     return (unsigned)(gy * (unsigned)nx + gx) * 4u;
   };
   auto plane_z = [&](int zz) {
-    return (long long)remap(zz, p.n[2], p.bc_lo[2], p.bc_hi[2]) * p.sz;
+    return (long long)wrap(zz, p.n[2], p.bc_lo[2], p.bc_hi[2]) * p.sz;
   };
   auto ldg = [](const float* base, unsigned off) {
     return *reinterpret_cast<const float*>(reinterpret_cast<const char*>(base) + off);
@@ -187,13 +237,14 @@ __device__ __forceinline__ void stage_tile_pairs(const StageParams<float>& p,
       r = it / TX;
       c = it - r * TX;
     } else if (it < NI + G::NXH) {
-      const int j = it - NI, q = j & 3;
-      r = j >> 2;
-      c = q < 2 ? q - 2 : TX + q - 2;
+      const int j = it - NI;
+      r = j / (2 * GH);
+      const int q = j - r * (2 * GH);
+      c = q < GH ? q - GH : TX + q - GH;
     } else {
       const int j = it - NI - G::NXH, hr = j / TX;
       c = j - hr * TX;
-      r = hr < 2 ? hr - 2 : TY + hr - 2;
+      r = hr < GH ? hr - GH : TY + hr - GH;
     }
   };
   unsigned aoff[NA];
@@ -213,7 +264,7 @@ __device__ __forceinline__ void stage_tile_pairs(const StageParams<float>& p,
       int r, c;
       load_rc(it, r, c);
       long long hs;
-      const float* a = halo_cell<2>(p, x0 + c, y0 + r, zz, hs);
+      const float* a = halo_cell<GH>(p, x0 + c, y0 + r, zz, hs);
 #pragma unroll
       for (int k = 0; k < kNV; ++k) u[k] = a[k * hs];
     } else {
@@ -254,13 +305,13 @@ __device__ __forceinline__ void stage_tile_pairs(const StageParams<float>& p,
 
   // The z march; warm-up iterations as in stage_tile().
 #pragma unroll 1
-  for (int k = z0 - 4; k < z1; ++k) {
+  for (int k = z0 - 2 * GH; k < z1; ++k) {
     const bool main = k >= z0;
-    // ---- A: loads: interior of plane k+2, halo of plane k ------------------
+    // ---- A: loads: interior of plane k+GH, halo of plane k -----------------
 #pragma unroll
     for (int a = 0; a < NA; ++a) {
       const int it = tid + a * NT;
-      if (it < (main ? G::NLOAD : NI)) load_item(it, aoff[a], k + 2, k);
+      if (it < (main ? G::NLOAD : NI)) load_item(it, aoff[a], k + GH, k);
     }
     __syncthreads();
     if (k < z0 - 2) continue;
@@ -268,32 +319,31 @@ __device__ __forceinline__ void stage_tile_pairs(const StageParams<float>& p,
 
     // ---- B: face states of x and y -----------------------------------------
     for (int it = tid; main && it < G::SX + G::SY; it += NT) {
-      float m[kNV], q[kNV], n[kNV], lo[kNV], hi[kNV];
+      float lo[kNV], hi[kNV];
       if (it < G::SX) {
         const int r = it / (TX + 2), c = it - r * (TX + 2) - 1;
-        auto ld = [&](int cc, float v[kNV]) {
-          const bool h = cc < 0 || cc >= TX;
-          ld9<PS>(h ? hb : cur, h ? r * 4 + (cc < 0 ? cc + 2 : cc - TX + 2) : r * TX + cc, v);
-        };
-        ld(c - 1, m);
-        ld(c, q);
-        ld(c + 1, n);
-        face_pair(m, q, n, p.limiter, lo, hi);
+        face_states<WENO, PS>(
+            [&](int j) {
+              const int cc = c + j;
+              const bool h = cc < 0 || cc >= TX;
+              return CellRef{h ? hb : cur, h ? r * (2 * GH) + (cc < 0 ? cc + GH : cc - TX + GH)
+                                             : r * TX + cc};
+            },
+            p.limiter, lo, hi);
         const int f = r * (TX + 1) + c;  // lower face of the cell
         if (c >= 0) st9<G::XN>(xL, f, lo);
         if (c < TX) st9<G::XN>(xU, f + 1, hi);
       } else {
-        const int j = it - G::SX;
-        const int r = j / TX - 1, c = j - (j / TX) * TX;
-        auto ld = [&](int rr, float v[kNV]) {
-          const bool h = rr < 0 || rr >= TY;
-          ld9<PS>(h ? hb : cur, h ? G::NXH + (rr < 0 ? rr + 2 : rr - TY + 2) * TX + c : rr * TX + c,
-                  v);
-        };
-        ld(r - 1, m);
-        ld(r, q);
-        ld(r + 1, n);
-        face_pair(m, q, n, p.limiter, lo, hi);
+        const int j0 = it - G::SX;
+        const int r = j0 / TX - 1, c = j0 - (j0 / TX) * TX;
+        face_states<WENO, PS>(
+            [&](int j) {
+              const int rr = r + j;
+              const bool h = rr < 0 || rr >= TY;
+              return CellRef{h ? hb : cur,
+                             h ? G::NXH + (rr < 0 ? rr + GH : rr - TY + GH) * TX + c : rr * TX + c};
+            },
+            p.limiter, lo, hi);
         const int f = r * TX + c;
         if (r >= 0) st9<G::YN>(yL, f, lo);
         if (r < TY) st9<G::YN>(yU, f + TX, hi);
@@ -326,14 +376,13 @@ __device__ __forceinline__ void stage_tile_pairs(const StageParams<float>& p,
     float dUz[kNV];
     if (owner) {
       float vl[kNV], vr[kNV], hi[kNV];
-      {
-        float m[kNV], q[kNV], n[kNV];
-        ld9<PS>(cur, oidx, m);
-        ld9<PS>(ring_plane(k + 1), oidx, q);
-        ld9<PS>(ring_plane(k + 2), oidx, n);
-        if constexpr (CT) ctc.from_prims(m, 1);
-        face_pair(m, q, n, p.limiter, vr, hi);
+      if constexpr (CT) {
+        float q[kNV];
+        ld9<PS>(cur, oidx, q);
+        ctc.from_prims(q, 1);
       }
+      face_states<WENO, PS>([&](int j) { return CellRef{ring_plane(k + 1 + j), oidx}; }, p.limiter,
+                            vr, hi);
       ld9<NI>(zP, oidx, vl);
       st9<NI>(zP, oidx, hi);
       if (k >= z0 - 1) {  // from k = z0-1 on, zP holds the upper state of cell k
@@ -419,14 +468,14 @@ __device__ __forceinline__ void stage_tile_pairs(const StageParams<float>& p,
   __syncthreads();  // the CTA may start another tile on the same shared memory
 }
 
-template <int TY, int NW, int STAGE, bool CT, bool HALO = false>
+template <int TY, int NW, int STAGE, bool CT, bool HALO, bool WENO>
 __global__ void __launch_bounds__(NW * 32, 2)
     rk_stage_pairs_kernel(const StageParams<float> p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ double wmax[NW];
   const StepScalars sc = *p.sc;
-  stage_tile_pairs<TY, NW, STAGE, CT, HALO>(p, sc, blockIdx.x, blockIdx.y, blockIdx.z,
-                                            reinterpret_cast<float*>(smem_raw), wmax);
+  stage_tile_pairs<TY, NW, STAGE, CT, HALO, WENO>(p, sc, blockIdx.x, blockIdx.y, blockIdx.z,
+                                                  reinterpret_cast<float*>(smem_raw), wmax);
 }
 
 }  // namespace mhd
