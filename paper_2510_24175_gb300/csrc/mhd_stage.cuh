@@ -318,9 +318,9 @@ __device__ __forceinline__ void stage_tile(const StageParams<T>& p, const StepSc
   const bool frozen = !(sc.dt != 0.0);
   const int lim = p.limiter;
   Phys<T> ph = p.ph;
-  if constexpr (NW > 1) {
+  if constexpr (TY > 1) {
     fp64_registers(ph, konst);
-  } else {  // one-warp 1-D kernels wait for latency: the plain operations
+  } else {  // 1-D kernels wait for latency: the plain operations
     ph.one = T(1);
     ph.nzero = T(-0.0);
   }

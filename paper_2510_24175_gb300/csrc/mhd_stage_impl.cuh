@@ -23,6 +23,13 @@ struct StageShape3D {
   static constexpr int NW = sizeof(T) == 8 && WENO ? 8 : 16;
 };
 
+// Warps of a 1-D tile.  The 36 (38) cells, 34 face states and 33 faces of a 32-cell
+// tile take two rounds of one warp, and a warp alone issues an FP64 instruction
+// every 64 clocks whether one lane is active or all are: a second warp takes the
+// second round at the same time (1024 cells, stages 1 and 2: 24 and 28 us -> 14
+// and 17.5 us).
+constexpr int kNW1 = 2;
+
 // The dynamic shared-memory limit of a kernel is set once per device (a
 // driver call per launch costs more than a small grid's kernel).  One flag
 // word per kernel: the template argument is the kernel itself.
@@ -129,7 +136,7 @@ void stage_shape(const Grid& g, size_t* smem, int* threads, int* ty) {
       *ty = 4;
     } else {
       *smem = (size_t)WenoGeom<1, false>::WORDS * sizeof(T);
-      *threads = 32;
+      *threads = kNW1 * 32;
       *ty = 1;
     }
     return;
@@ -145,7 +152,7 @@ void stage_shape(const Grid& g, size_t* smem, int* threads, int* ty) {
     *ty = 8;
   } else {
     *smem = (size_t)TileGeom<1, false>::WORDS * sizeof(T);
-    *threads = 32;
+    *threads = kNW1 * 32;
     *ty = 1;
   }
 }
@@ -178,11 +185,11 @@ cudaError_t prepare_stage_kernels(const Grid& g, bool ct) {
   if (weno && g.ndim == 2) {
     MHD_SET3(rk_stage_weno_kernel, W2, 4, 8);
   } else if (weno) {
-    MHD_SET3(rk_stage_weno_kernel, W1, 1, 1);
+    MHD_SET3(rk_stage_weno_kernel, W1, 1, kNW1);
   } else if (g.ndim == 2) {
     MHD_SET3(rk_stage_kernel, P2, 8, 8);
   } else {
-    MHD_SET3(rk_stage_kernel, P1, 1, 1);
+    MHD_SET3(rk_stage_kernel, P1, 1, kNW1);
   }
 #undef MHD_SET3
 #undef MHD_SET1
@@ -267,9 +274,9 @@ cudaError_t launch_stage(const Grid& g, int stage, const T* win, const T* un, T*
       return launch_weno<T, 4, 8, 3, false>(p, grid, stream);
     }
     dim3 grid((g.n[0] + 31) / 32, 1, 1);
-    if (stage == 1) return launch_weno<T, 1, 1, 1, false>(p, grid, stream);
-    if (stage == 2) return launch_weno<T, 1, 1, 2, false>(p, grid, stream);
-    return launch_weno<T, 1, 1, 3, false>(p, grid, stream);
+    if (stage == 1) return launch_weno<T, 1, kNW1, 1, false>(p, grid, stream);
+    if (stage == 2) return launch_weno<T, 1, kNW1, 2, false>(p, grid, stream);
+    return launch_weno<T, 1, kNW1, 3, false>(p, grid, stream);
   }
   if (g.ndim == 2) {
     dim3 grid((g.n[0] + 31) / 32, (g.n[1] + 7) / 8, 1);
@@ -278,9 +285,9 @@ cudaError_t launch_stage(const Grid& g, int stage, const T* win, const T* un, T*
     return launch_one<T, 8, 8, 3, false>(p, grid, stream);
   }
   dim3 grid((g.n[0] + 31) / 32, 1, 1);
-  if (stage == 1) return launch_one<T, 1, 1, 1, false>(p, grid, stream);
-  if (stage == 2) return launch_one<T, 1, 1, 2, false>(p, grid, stream);
-  return launch_one<T, 1, 1, 3, false>(p, grid, stream);
+  if (stage == 1) return launch_one<T, 1, kNW1, 1, false>(p, grid, stream);
+  if (stage == 2) return launch_one<T, 1, kNW1, 2, false>(p, grid, stream);
+  return launch_one<T, 1, kNW1, 3, false>(p, grid, stream);
 }
 
 // Halo faces (3-D GLM grids with kBcHalo sides): the HALO variants of the

@@ -133,7 +133,7 @@ __global__ void __launch_bounds__(NW * 32, sizeof(T) == 4 && ZACT ? 2 : 1)
     if (threadIdx.x == 0) WenoConst<T>::fill(konst + 4);
   }
   fp64_registers(ph, konst);  // (synchronises)
-  if constexpr (NW == 1) {  // one-warp 1-D kernels wait for latency: the plain operations
+  if constexpr (TY == 1) {  // 1-D kernels wait for latency: the plain operations
     ph.one = T(1);
     ph.nzero = T(-0.0);
   }
