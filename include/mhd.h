@@ -419,7 +419,9 @@ int mhd_fp64_fma_rate(void* stream, unsigned warp_mask, double out[3]);
  * frees first, and a CTA takes its planes plus one for its warm-up; the
  * depth is the candidate (256, 192, 128, 96, 80, 64, 56, 48, 40, 32, 24, 20,
  * 16, 12, 8, 4; at most n[2], or 4) with the shortest launch, the deeper one
- * on a tie.  A grid with an extent of 1 is not 3-D: *tz = 1.  The paper has
+ * on a tie.  A grid with an extent of 1 is not 3-D: *tz = 1.  (FP64 PLM contexts
+ * with GLM cleaning plan 16 x 16 tiles in the same way, with the depths 3 and 2
+ * as well, and take them when their launch is no longer.)  The paper has
  * no counterpart: this is how the library spreads its stage launches over
  * the SMs.  Errors: MHD_ERR_INVALID (an extent, ty, nsm or ctas_per_sm below
  * 1, n or tz NULL; message in mhd_last_error(NULL)). */

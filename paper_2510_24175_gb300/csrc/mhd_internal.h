@@ -25,6 +25,7 @@ struct Grid {
   int limiter;
   double gamma, rho_floor, p_floor;
   double dx[3];
+  int tx;                // 3-D tile width of the stage kernel: 32, or 16 (FP64 PLM, GLM)
   int tz;                // z planes per CTA of the stage kernel
   int nsm;               // SM count of the device
 };

@@ -6,8 +6,8 @@
 // Tzeferacos 2010, Eq. 27) and the next step's max-wave-speed reduction;
 // STAGE 3 (SSP-RK3 middle stage): the combination without the epilogue.
 //
-// Decomposition: a CTA owns a 32 x TY column tile in (x, y) and marches in z
-// over p.tz planes.  Ghost zones are never stored: the boundary calculation
+// Decomposition: a CTA owns a TX x TY column tile in (x, y) (32 x 8 or 16 x 16 in
+// 3-D) and marches in z over p.tz planes.  Ghost zones are never stored: the boundary calculation
 // is an index remap at load time (periodic: wrap; outflow: clamp to the
 // nearest interior cell), so the state arrays are interior-only SoA.
 //
@@ -204,9 +204,9 @@ __host__ __device__ __forceinline__ int remap3(int i, int n, int lo, int hi) {
   return i;
 }
 
-template <int TY, bool ZACT>
+template <int TY, bool ZACT, int TX_ = 32>
 struct TileGeom {
-  static constexpr int TX = 32;
+  static constexpr int TX = TX_;
   static constexpr int GY = TY > 1 ? 2 : 0;
   static constexpr int NINT = TY * TX;             // interior cells per plane
   static constexpr int NXH = 4 * TY;               // x halo: columns -2, -1, 32, 33
@@ -229,11 +229,13 @@ struct TileGeom {
       RING_W + HB_W + kNV * SXN + kNV * SYN + kNV * FXN + kNV * FYN + Z_W;
   // phase-A items: interior, x halo, y halo
   static constexpr int NLOAD = NINT + NXH + NYH;
-  // phase-C flux items, warp-aligned segments [x main][y][x right edge]
+  // phase-C flux items [x main][y][x right edge], each segment starting on a warp:
+  // a warp with both directions would run both fluxes one after the other, last
+  // (16 x 16 tiles without that: 256^3 step 50.9 instead of 46.4 ms)
   static constexpr int IT_X = TY * TX;
   static constexpr int IT_Y = FYN;
-  static constexpr int IT_XE = TY;
-  static constexpr int ITEMS = IT_X + IT_Y + IT_XE;
+  static constexpr int IT_XE0 = IT_X + (IT_Y + 31) / 32 * 32;
+  static constexpr int ITEMS = IT_XE0 + TY;
 };
 
 // Half slopes of the 9 primitives of one cell from its two neighbours along a
@@ -278,11 +280,12 @@ __device__ __forceinline__ void cell_slopes(const T* m, int sm, const T* c, int 
 // the face update), the face / cell electric fields go to p.ctf, and the last
 // stage has no damping and no wave-speed reduction (done after the face update).
 // HALO (3-D, not CT): ghost cells of kBcHalo sides from p.halo (halo_cell).
-template <class T, int TY, int NW, int STAGE, bool ZACT, bool CT = false, bool HALO = false>
+template <class T, int TY, int NW, int STAGE, bool ZACT, bool CT = false, bool HALO = false,
+          int TX_ = 32>
 __device__ __forceinline__ void stage_tile(const StageParams<T>& p, const StepScalars& sc,
                                            int bx, int by, int bz, unsigned char* smem_raw,
                                            double* wmax, double* konst = nullptr) {
-  using G = TileGeom<TY, ZACT>;
+  using G = TileGeom<TY, ZACT, TX_>;
   constexpr int NT = NW * 32;
   constexpr int TX = G::TX;
   constexpr int ZT0 = NT - G::NINT;  // threads ZT0.. own one tile column each
@@ -457,14 +460,15 @@ __device__ __forceinline__ void stage_tile(const StageParams<T>& p, const StepSc
       T vl[kNV], vr[kNV], F[kNV];
       T* out;
       int os;
-      const bool xdir = it < G::IT_X || it >= G::IT_X + G::IT_Y;
+      const bool xdir = it < G::IT_X || it >= G::IT_XE0;
+      if (G::IT_XE0 > G::IT_X + G::IT_Y && !xdir && it >= G::IT_X + G::IT_Y) continue;
       if (xdir) {
         int r, fi;
         if (it < G::IT_X) {
           r = it / TX;
           fi = it - r * TX;
         } else {
-          r = it - (G::IT_X + G::IT_Y);
+          r = it - G::IT_XE0;
           fi = TX;
         }
         const T* a = cell_ptr(cur, r, fi - 1);
@@ -617,15 +621,15 @@ __device__ __forceinline__ void stage_tile(const StageParams<T>& p, const StepSc
   __syncthreads();  // the CTA may start another tile on the same shared memory
 }
 
-template <class T, int TY, int NW, int STAGE, bool ZACT, bool CT, bool HALO = false>
+template <class T, int TY, int NW, int STAGE, bool ZACT, bool CT, bool HALO = false, int TX = 32>
 __global__ void __launch_bounds__(NW * 32, 1)
     rk_stage_kernel(const StageParams<T> p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ double wmax[NW];
   __shared__ double konst[4];
   const StepScalars sc = *p.sc;
-  stage_tile<T, TY, NW, STAGE, ZACT, CT, HALO>(p, sc, blockIdx.x, blockIdx.y, blockIdx.z,
-                                               smem_raw, wmax, konst);
+  stage_tile<T, TY, NW, STAGE, ZACT, CT, HALO, TX>(p, sc, blockIdx.x, blockIdx.y, blockIdx.z,
+                                                   smem_raw, wmax, konst);
 }
 
 }  // namespace mhd

@@ -59,16 +59,18 @@ static cudaError_t launch_one(const StageParams<T>& p, dim3 grid, cudaStream_t s
 
 // The 3-D stage kernels: FP64 rk_stage_kernel / rk_stage_weno_kernel, FP32
 // rk_stage_pairs_kernel (mhd_stage_pairs.cuh).
-template <class T, bool WENO, int STAGE, bool CT, bool HALO>
+// TX: 32, or 16 with 16 rows (FP64 PLM; see mhd_create's choice).
+template <class T, bool WENO, int STAGE, bool CT, bool HALO, int TX = 32>
 struct Kern3D {
   using S = StageShape3D<T, WENO>;
+  static constexpr int TY = S::TY * 32 / TX;
   static constexpr auto get() {
     if constexpr (sizeof(T) == 4)
       return rk_stage_pairs_kernel<S::TY, S::NW, STAGE, CT, HALO, WENO>;
     else if constexpr (WENO)
       return rk_stage_weno_kernel<T, S::TY, S::NW, STAGE, true, CT, HALO>;
     else
-      return rk_stage_kernel<T, S::TY, S::NW, STAGE, true, CT, HALO>;
+      return rk_stage_kernel<T, TY, S::NW, STAGE, true, CT, HALO, TX>;
   }
   static constexpr size_t words() {
     if constexpr (sizeof(T) == 4)
@@ -76,7 +78,7 @@ struct Kern3D {
     else if constexpr (WENO)
       return WenoGeom<S::TY, true>::WORDS;
     else
-      return TileGeom<S::TY, true>::WORDS;
+      return TileGeom<TY, true, TX>::WORDS;
   }
   static constexpr auto kernel = get();
   static constexpr size_t smem = words() * sizeof(T);
@@ -84,23 +86,23 @@ struct Kern3D {
   static cudaError_t launch(const StageParams<T>& p, const Grid& g, int nzc, cudaStream_t s) {
     cudaError_t e = prepare();
     if (e != cudaSuccess) return e;
-    const dim3 grid((g.n[0] + 31) / 32, (g.n[1] + S::TY - 1) / S::TY, nzc);
+    const dim3 grid((g.n[0] + TX - 1) / TX, (g.n[1] + TY - 1) / TY, nzc);
     kernel<<<grid, S::NW * 32, smem, s>>>(p);
     return cudaGetLastError();
   }
 };
-template <class T, bool WENO, bool CT, bool HALO>
+template <class T, bool WENO, bool CT, bool HALO, int TX = 32>
 static cudaError_t launch_3d(int stage, const StageParams<T>& p, const Grid& g, int nzc,
                              cudaStream_t s) {
-  if (stage == 1) return Kern3D<T, WENO, 1, CT, HALO>::launch(p, g, nzc, s);
-  if (stage == 2) return Kern3D<T, WENO, 2, CT, HALO>::launch(p, g, nzc, s);
-  return Kern3D<T, WENO, 3, CT, HALO>::launch(p, g, nzc, s);
+  if (stage == 1) return Kern3D<T, WENO, 1, CT, HALO, TX>::launch(p, g, nzc, s);
+  if (stage == 2) return Kern3D<T, WENO, 2, CT, HALO, TX>::launch(p, g, nzc, s);
+  return Kern3D<T, WENO, 3, CT, HALO, TX>::launch(p, g, nzc, s);
 }
-template <class T, bool WENO, bool CT, bool HALO>
+template <class T, bool WENO, bool CT, bool HALO, int TX = 32>
 static cudaError_t prepare_3d() {
-  cudaError_t e = Kern3D<T, WENO, 1, CT, HALO>::prepare();
-  if (e == cudaSuccess) e = Kern3D<T, WENO, 2, CT, HALO>::prepare();
-  if (e == cudaSuccess) e = Kern3D<T, WENO, 3, CT, HALO>::prepare();
+  cudaError_t e = Kern3D<T, WENO, 1, CT, HALO, TX>::prepare();
+  if (e == cudaSuccess) e = Kern3D<T, WENO, 2, CT, HALO, TX>::prepare();
+  if (e == cudaSuccess) e = Kern3D<T, WENO, 3, CT, HALO, TX>::prepare();
   return e;
 }
 // The FP32 kernels without halo faces address a plane with 32 bits; larger planes
@@ -312,6 +314,9 @@ cudaError_t launch_stage_halo(const Grid& g, int stage, const T* win, const T* u
     p.halo[f] = bc == kBcHalo ? halo[f] : nullptr;
   }
   const int nzc = (p.zhi - p.zlo + p.tz - 1) / p.tz;
+  if constexpr (sizeof(T) == 8) {
+    if (g.tx == 16) return launch_3d<T, false, false, true, 16>(stage, p, g, nzc, stream);
+  }
   return g.limiter == kLimWenoz ? launch_3d<T, true, false, true>(stage, p, g, nzc, stream)
                                 : launch_3d<T, false, false, true>(stage, p, g, nzc, stream);
 }
@@ -319,6 +324,9 @@ cudaError_t launch_stage_halo(const Grid& g, int stage, const T* win, const T* u
 // The shared-memory limits of the HALO variants (set once, outside any capture).
 template <class T>
 cudaError_t prepare_stage_kernels_halo(const Grid& g) {
+  if constexpr (sizeof(T) == 8) {
+    if (g.tx == 16) return prepare_3d<T, false, false, true, 16>();
+  }
   return g.limiter == kLimWenoz ? prepare_3d<T, true, false, true>()
                                 : prepare_3d<T, false, false, true>();
 }
