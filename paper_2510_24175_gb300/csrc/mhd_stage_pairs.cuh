@@ -37,6 +37,7 @@ struct PairGeom {
   static constexpr int WORDS = RING + HB + 2 * kNV * (XN + YN) + 2 * kNV * NINT;
   static constexpr int NLOAD = NINT + NXH + NYH;
   static constexpr int SX = TY * (TX + 2);  // x face-state items, columns -1..32
+  static constexpr int SY0 = (SX + 31) / 32 * 32;  // y items start on a warp
   static constexpr int SY = (TY + 2) * TX;  // y face-state items, rows -1..TY
   static constexpr int ITEMS = XN + YN;     // flux items: [x main][y][x right edge]
 };
@@ -318,7 +319,7 @@ __device__ __forceinline__ void stage_tile_pairs(const StageParams<float>& p,
     const float* cur = ring_plane(k);
 
     // ---- B: face states of x and y -----------------------------------------
-    for (int it = tid; main && it < G::SX + G::SY; it += NT) {
+    for (int it = tid; main && it < G::SY0 + G::SY; it += NT) {
       float lo[kNV], hi[kNV];
       if (it < G::SX) {
         const int r = it / (TX + 2), c = it - r * (TX + 2) - 1;
@@ -333,8 +334,8 @@ __device__ __forceinline__ void stage_tile_pairs(const StageParams<float>& p,
         const int f = r * (TX + 1) + c;  // lower face of the cell
         if (c >= 0) st9<G::XN>(xL, f, lo);
         if (c < TX) st9<G::XN>(xU, f + 1, hi);
-      } else {
-        const int j0 = it - G::SX;
+      } else if (it >= G::SY0) {
+        const int j0 = it - G::SY0;
         const int r = j0 / TX - 1, c = j0 - (j0 / TX) * TX;
         face_states<WENO, PS>(
             [&](int j) {
