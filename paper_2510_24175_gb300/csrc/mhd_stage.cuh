@@ -272,6 +272,14 @@ __device__ __forceinline__ void cell_slopes(const T* m, int sm, const T* c, int 
   for (int k = 0; k < kNV; ++k) h[k * sh] = sig[k];
 }
 
+// Named CTA barriers: n threads in all arrive or wait at barrier id.
+__device__ __forceinline__ void bar_sync(int id, int n) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
+}
+__device__ __forceinline__ void bar_arrive(int id, int n) {
+  asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory");
+}
+
 // One tile (bx, by, bz) of one RK stage; called by every thread of a CTA of
 // NW warps.  smem_raw: TileGeom::WORDS elements of T; wmax: NW doubles,
 // konst (FP64): 4 doubles.
@@ -411,24 +419,41 @@ __device__ __forceinline__ void stage_tile(const StageParams<T>& p, const StepSc
   // k = z0.  (Unrolling, and with it the peeling of warm-up iterations into
   // separate copies, is disabled.)
   constexpr int NWARM = ZACT ? 4 : 0;
+  // 3-D tiles with as many other threads as owners: the owners' z slopes and
+  // update (D) run at the same time as the others' loads and x, y slopes, so
+  // the FP64 unit has work while loads are in flight
+  constexpr bool kRoles = ZACT && ZT0 >= G::NINT;
   SpeedMax<T> smax(ph);  // last stage: the new state's maximum wave speed
 #pragma unroll 1
   for (int k = z0 - NWARM; k < z1; ++k) {
     const bool main = k >= z0;
     // ---- A: loads ---------------------------------------------------------
+    // kRoles: the column owners are still in phase D of plane k-1 (it shares no
+    // data with A and B) when the other warps load and go on to the slopes
+    const bool roles = kRoles && main;
+    const int step = roles ? ZT0 : NT;
     const int nload = main ? G::NLOAD : G::NINT;
-    for (int it = tid; it < nload; it += NT) {
+    for (int it = roles && owner ? nload : tid; it < nload; it += step) {
       if (ZACT && it < G::NINT)
         load_item(it, k + 2, k);
       else
         load_item(it, k, k);
     }
-    __syncthreads();
+    if (!roles) {
+      __syncthreads();
+    } else if (owner) {
+      bar_sync(2, NT);  // the loads are done
+    } else {
+      bar_arrive(2, NT);
+      bar_sync(1, ZT0);
+    }
     if (ZACT && k < z0 - 2) continue;
     const T* cur = ring_plane(k);
 
     // ---- B: slopes --------------------------------------------------------
-    for (int it = tid; main && it < G::SXN + G::SYN; it += NT) {
+    constexpr int kSlopes = G::SXN + G::SYN;
+    const int send = roles && !owner ? min(kSlopes, 2 * ZT0) : kSlopes;
+    for (int it = roles && owner ? 2 * ZT0 + oidx : tid; main && it < send; it += step) {
       T* dst;
       int ds;
       const T *m, *c, *pp;
