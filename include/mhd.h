@@ -410,8 +410,8 @@ int mhd_fp64_fma_rate(void* stream, unsigned warp_mask, double out[3]);
 
 /* Launch planning, on the host only (no GPU, no CUDA call): the z-chunk depth
  * *tz (planes per CTA) that the 3-D stage launches of an n[0] x n[1] x n[2]
- * grid use, for column tiles of 32 x ty cells (ty: 8, or 4 for FP64
- * WENO-Z) on nsm SMs holding ctas_per_sm stage CTAs each (1 for FP64, 2 for
+ * grid use, for column tiles of 32 x ty cells (ty: 8 for the 3-D kernels)
+ * on nsm SMs holding ctas_per_sm stage CTAs each (1 for FP64, 2 for
  * FP32), and, if span is not
  * NULL, the modelled duration of one launch in plane iterations.  The model:
  * the CTAs start in launch order -- every column tile's full chunks, then
@@ -419,9 +419,10 @@ int mhd_fp64_fma_rate(void* stream, unsigned warp_mask, double out[3]);
  * frees first, and a CTA takes its planes plus one for its warm-up; the
  * depth is the candidate (256, 192, 128, 96, 80, 64, 56, 48, 40, 32, 24, 20,
  * 16, 12, 8, 4; at most n[2], or 4) with the shortest launch, the deeper one
- * on a tie.  A grid with an extent of 1 is not 3-D: *tz = 1.  (FP64 PLM contexts
- * with GLM cleaning plan 16 x 16 tiles in the same way, with the depths 3 and 2
- * as well, and take them when their launch is no longer.)  The paper has
+ * on a tie.  A grid with an extent of 1 is not 3-D: *tz = 1.  (FP64
+ * contexts plan a second tile in the same way -- PLM with GLM cleaning 16 x 16
+ * cells, with the depths 3 and 2 as well; WENO-Z 32 x 4 -- and take it when its
+ * launch is no longer.)  The paper has
  * no counterpart: this is how the library spreads its stage launches over
  * the SMs.  Errors: MHD_ERR_INVALID (an extent, ty, nsm or ctas_per_sm below
  * 1, n or tz NULL; message in mhd_last_error(NULL)). */

@@ -246,11 +246,33 @@ static int plan_tz(long long cols, int nz, long long slots, double* span_out, in
   return best;
 }
 
-static int choose_tz(const mhd::Grid& g, int ctas_per_sm, int ty, double* span = nullptr) {
+static int choose_tz(const mhd::Grid& g, int ctas_per_sm, double* span = nullptr) {
   if (g.ndim < 3) return 1;
-  const int wy = ty * 32 / g.tx;
-  const long long cols = (long long)((g.n[0] + g.tx - 1) / g.tx) * ((g.n[1] + wy - 1) / wy);
+  const long long cols =
+      (long long)((g.n[0] + g.tx - 1) / g.tx) * ((g.n[1] + g.ty - 1) / g.ty);
   return plan_tz(cols, g.n[2], (long long)g.nsm * ctas_per_sm, span, g.tx == 32 ? 4 : 2);
+}
+
+// The 3-D column tile and z-chunk depth of a grid: 32 x 8 (ty), or for FP64 the
+// reconstruction's other shape where its launch is modelled no longer.
+// PLM (GLM cleaning): 16 x 16, which pads fewer columns when nx ends in the first
+// half of a 32-cell tile, and whose thinner chunks (2 and 3 planes) spread a small
+// grid over the SMs.  At equal plans it is 1.3 % faster (256^3, one step 46.4 against
+// 47.0 ms; fewer halo conversions); 48^3: 536 -> 425 us.
+// WENO-Z: 32 x 4, for short last rows of tiles; a plane of it takes 0.54 of a 32 x 8
+// one (256^3, one RK3 step 102.5 against 94.4 ms for the same cells).
+static void choose_tile(mhd::Grid& g, int ctas_per_sm, int ty, bool glm, bool fp64) {
+  double span = 0.0, other_span = 0.0;
+  g.tx = 32;
+  g.ty = ty;
+  g.tz = choose_tz(g, ctas_per_sm, &span);
+  const bool weno = g.limiter == MHD_LIM_WENOZ;
+  if (g.ndim < 3 || !fp64 || (!weno && !glm)) return;
+  mhd::Grid o = g;
+  o.tx = weno ? 32 : 16;
+  o.ty = weno ? 4 : 16;
+  o.tz = choose_tz(o, ctas_per_sm, &other_span);
+  if ((weno ? 0.54 : 1.0) * other_span <= span) g = o;
 }
 
 int mhd_plan_z_chunks(const int n[3], int ty, int nsm, int ctas_per_sm, int* tz,
@@ -434,26 +456,11 @@ int mhd_create(const mhd_config* cfg, void* d_workspace, size_t bytes, void* str
   else
     mhd::stage_shape<float>(c->grid, &smem, &threads, &ty);
   const int per_sm = (int)(228 * 1024 / (smem + 1024));
-  double span = 0.0;
-  c->grid.tx = 32;
-  c->grid.tz = choose_tz(c->grid, per_sm < 1 ? 1 : per_sm, ty, &span);
-  if (c->esize == 8 && c->grid.ndim == 3 && c->grid.limiter != MHD_LIM_WENOZ &&
-      cfg->divb == MHD_DIVB_GLM) {
-    // 16 x 16 tiles instead of 32 x 8 where they take no longer: fewer columns
-    // are padded when nx ends in the first half of a 32-cell tile, and thinner
-    // chunks (2 and 3 planes) spread a small grid over the SMs.  At equal plans
-    // they are 1.3 % faster (256^3, one step 46.4 against 47.0 ms; fewer halo
-    // conversions); 48^3: 536 -> 425 us.
-    mhd::Grid g16 = c->grid;
-    g16.tx = 16;
-    double span16 = 0.0;
-    g16.tz = choose_tz(g16, per_sm < 1 ? 1 : per_sm, ty, &span16);
-    if (span16 <= span) c->grid = g16;
-  }
+  choose_tile(c->grid, per_sm < 1 ? 1 : per_sm, ty, cfg->divb == MHD_DIVB_GLM, c->esize == 8);
   {
     mhd::Grid gh = c->grid;  // the half-depth grid of mhd_step_host's last stage
     gh.n[2] = (gh.n[2] + 1) / 2;
-    c->tz_half = choose_tz(gh, per_sm < 1 ? 1 : per_sm, ty);
+    c->tz_half = choose_tz(gh, per_sm < 1 ? 1 : per_sm);
   }
   {
     // kernel attributes now, so that no later launch (a captured one in

@@ -25,7 +25,7 @@ struct Grid {
   int limiter;
   double gamma, rho_floor, p_floor;
   double dx[3];
-  int tx;                // 3-D tile width of the stage kernel: 32, or 16 (FP64 PLM, GLM)
+  int tx, ty;            // 3-D column tile of the stage kernel (see mhd_create)
   int tz;                // z planes per CTA of the stage kernel
   int nsm;               // SM count of the device
 };

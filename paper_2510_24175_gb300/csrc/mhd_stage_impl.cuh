@@ -8,20 +8,21 @@
 
 namespace mhd {
 
-// Tile shapes of 3-D grids: column tiles of 32 x TY cells marching in z.  FP64:
-// one CTA per SM, PLM 32 x 8 with 16 warps (211 KB of shared memory), WENO-Z 32 x
-// 4 with 8 warps (167 KB); the SM's FP64 unit is shared by all its warps and one
-// warp issues an FP64 instruction at most every 64 clocks, so the unit saturates
-// only when at least four warps have FP64 work.  FP32 (PLM and WENO-Z): 32 x 8
-// with 16 warps at 64 registers, two CTAs per SM: the kernels are bound by
-// latency and issue; with 24 and 16 warps per SM the PLM kernel took 2 and 8 %
-// longer (512^3).  2-D grids use the 32 x 8 (PLM) or 32 x 4 (WENO-Z) tile with a
-// single plane; 1-D grids a 32-cell row.
+// Tiles of 3-D grids: columns of TX x TY cells marching in z (mhd_create picks the
+// shape).  FP64: one CTA per SM; the SM's FP64 unit is shared by all its warps and
+// one warp issues an FP64 instruction at most every 64 clocks, so the unit
+// saturates only when at least four warps have FP64 work.  PLM: 32 x 8 or 16 x 16
+// (211 KB of shared memory), 16 warps of 128 registers (12 of 168: 256^3 step 46.8
+// instead of 44.0 ms).  WENO-Z: 32 x 8 (226 KB), 12 warps (16: 100 instead of 96 ms
+// per RK3 step of 256^3), or 32 x 4 with 8 warps.  FP32 (PLM and WENO-Z): 32 x 8
+// with 16 warps at 64 registers, two CTAs per SM: the kernels are bound by latency
+// and issue; with 24 and 16 warps per SM the PLM kernel took 2 and 8 % longer
+// (512^3).  2-D grids use the 32 x 8 (PLM) or 32 x 4 (WENO-Z) tile with a single
+// plane; 1-D grids a 32-cell row.
 template <class T, bool WENO>
-struct StageShape3D {
-  static constexpr int TY = sizeof(T) == 8 && WENO ? 4 : 8;
-  static constexpr int NW = sizeof(T) == 8 && WENO ? 8 : 16;
-};
+constexpr int stage_warps(int ty) {
+  return sizeof(T) == 8 && WENO ? (ty == 4 ? 8 : 12) : 16;
+}
 
 // Warps of a 1-D tile.  The 36 (38) cells, 34 face states and 33 faces of a 32-cell
 // tile take two rounds of one warp, and a warp alone issues an FP64 instruction
@@ -57,52 +58,52 @@ static cudaError_t launch_one(const StageParams<T>& p, dim3 grid, cudaStream_t s
   return cudaGetLastError();
 }
 
+template <class T, bool WENO, int TX, int TY>
+constexpr size_t smem_3d() {
+  if constexpr (sizeof(T) == 4)
+    return PairGeom<TY, WENO>::WORDS * sizeof(T);
+  else if constexpr (WENO)
+    return WenoGeom<TY, true>::WORDS * sizeof(T);
+  else
+    return TileGeom<TY, true, TX>::WORDS * sizeof(T);
+}
+
 // The 3-D stage kernels: FP64 rk_stage_kernel / rk_stage_weno_kernel, FP32
 // rk_stage_pairs_kernel (mhd_stage_pairs.cuh).
-// TX: 32, or 16 with 16 rows (FP64 PLM; see mhd_create's choice).
-template <class T, bool WENO, int STAGE, bool CT, bool HALO, int TX = 32>
+template <class T, bool WENO, int STAGE, bool CT, bool HALO, int TX = 32, int TY = 8>
 struct Kern3D {
-  using S = StageShape3D<T, WENO>;
-  static constexpr int TY = S::TY * 32 / TX;
+  static constexpr int NW = stage_warps<T, WENO>(TY);
   static constexpr auto get() {
     if constexpr (sizeof(T) == 4)
-      return rk_stage_pairs_kernel<S::TY, S::NW, STAGE, CT, HALO, WENO>;
+      return rk_stage_pairs_kernel<TY, NW, STAGE, CT, HALO, WENO>;
     else if constexpr (WENO)
-      return rk_stage_weno_kernel<T, S::TY, S::NW, STAGE, true, CT, HALO>;
+      return rk_stage_weno_kernel<T, TY, NW, STAGE, true, CT, HALO>;
     else
-      return rk_stage_kernel<T, TY, S::NW, STAGE, true, CT, HALO, TX>;
-  }
-  static constexpr size_t words() {
-    if constexpr (sizeof(T) == 4)
-      return PairGeom<S::TY, WENO>::WORDS;
-    else if constexpr (WENO)
-      return WenoGeom<S::TY, true>::WORDS;
-    else
-      return TileGeom<TY, true, TX>::WORDS;
+      return rk_stage_kernel<T, TY, NW, STAGE, true, CT, HALO, TX>;
   }
   static constexpr auto kernel = get();
-  static constexpr size_t smem = words() * sizeof(T);
+  static constexpr size_t smem = smem_3d<T, WENO, TX, TY>();
   static cudaError_t prepare() { return set_smem_once<kernel>(smem); }
   static cudaError_t launch(const StageParams<T>& p, const Grid& g, int nzc, cudaStream_t s) {
     cudaError_t e = prepare();
     if (e != cudaSuccess) return e;
     const dim3 grid((g.n[0] + TX - 1) / TX, (g.n[1] + TY - 1) / TY, nzc);
-    kernel<<<grid, S::NW * 32, smem, s>>>(p);
+    kernel<<<grid, NW * 32, smem, s>>>(p);
     return cudaGetLastError();
   }
 };
-template <class T, bool WENO, bool CT, bool HALO, int TX = 32>
+template <class T, bool WENO, bool CT, bool HALO, int TX = 32, int TY = 8>
 static cudaError_t launch_3d(int stage, const StageParams<T>& p, const Grid& g, int nzc,
                              cudaStream_t s) {
-  if (stage == 1) return Kern3D<T, WENO, 1, CT, HALO, TX>::launch(p, g, nzc, s);
-  if (stage == 2) return Kern3D<T, WENO, 2, CT, HALO, TX>::launch(p, g, nzc, s);
-  return Kern3D<T, WENO, 3, CT, HALO, TX>::launch(p, g, nzc, s);
+  if (stage == 1) return Kern3D<T, WENO, 1, CT, HALO, TX, TY>::launch(p, g, nzc, s);
+  if (stage == 2) return Kern3D<T, WENO, 2, CT, HALO, TX, TY>::launch(p, g, nzc, s);
+  return Kern3D<T, WENO, 3, CT, HALO, TX, TY>::launch(p, g, nzc, s);
 }
-template <class T, bool WENO, bool CT, bool HALO, int TX = 32>
+template <class T, bool WENO, bool CT, bool HALO, int TX = 32, int TY = 8>
 static cudaError_t prepare_3d() {
-  cudaError_t e = Kern3D<T, WENO, 1, CT, HALO, TX>::prepare();
-  if (e == cudaSuccess) e = Kern3D<T, WENO, 2, CT, HALO, TX>::prepare();
-  if (e == cudaSuccess) e = Kern3D<T, WENO, 3, CT, HALO, TX>::prepare();
+  cudaError_t e = Kern3D<T, WENO, 1, CT, HALO, TX, TY>::prepare();
+  if (e == cudaSuccess) e = Kern3D<T, WENO, 2, CT, HALO, TX, TY>::prepare();
+  if (e == cudaSuccess) e = Kern3D<T, WENO, 3, CT, HALO, TX, TY>::prepare();
   return e;
 }
 // The FP32 kernels without halo faces address a plane with 32 bits; larger planes
@@ -128,10 +129,9 @@ template <class T>
 void stage_shape(const Grid& g, size_t* smem, int* threads, int* ty) {
   if (g.limiter == kLimWenoz) {
     if (g.ndim == 3) {
-      using K = Kern3D<T, true, 1, false, false>;
-      *smem = K::smem;
-      *threads = K::S::NW * 32;
-      *ty = K::S::TY;
+      *smem = smem_3d<T, true, 32, 8>();
+      *threads = stage_warps<T, true>(8) * 32;
+      *ty = 8;
     } else if (g.ndim == 2) {
       *smem = (size_t)WenoGeom<4, false>::WORDS * sizeof(T);
       *threads = 256;
@@ -144,10 +144,9 @@ void stage_shape(const Grid& g, size_t* smem, int* threads, int* ty) {
     return;
   }
   if (g.ndim == 3) {
-    using K = Kern3D<T, false, 1, false, false>;
-    *smem = K::smem;
-    *threads = K::S::NW * 32;
-    *ty = K::S::TY;
+    *smem = smem_3d<T, false, 32, 8>();
+    *threads = stage_warps<T, false>(8) * 32;
+    *ty = 8;
   } else if (g.ndim == 2) {
     *smem = (size_t)TileGeom<8, false>::WORDS * sizeof(T);
     *threads = 8 * 32;
@@ -165,6 +164,9 @@ void stage_shape(const Grid& g, size_t* smem, int* threads, int* ty) {
 template <class T>
 cudaError_t prepare_stage_kernels(const Grid& g, bool ct) {
   const bool weno = g.limiter == kLimWenoz;
+  if constexpr (sizeof(T) == 8) {
+    if (ct && g.ty == 4) return prepare_3d<T, true, true, false, 32, 4>();
+  }
   if (ct) return weno ? prepare_3d<T, true, true, false>() : prepare_3d<T, false, true, false>();
   if (g.ndim == 3) {
     // FP64, and planes beyond 32-bit offsets: the halo-capable kernels (launch_stage)
@@ -254,6 +256,9 @@ cudaError_t launch_stage(const Grid& g, int stage, const T* win, const T* un, T*
   if (ctf) {
     // constrained transport: 3-D grids only (checked when the context is made)
     if (g.ndim != 3 || !bw) return cudaErrorInvalidValue;
+    if constexpr (sizeof(T) == 8) {
+      if (g.ty == 4) return launch_3d<T, true, true, false, 32, 4>(stage, p, g, nzc, stream);
+    }
     return g.limiter == kLimWenoz ? launch_3d<T, true, true, false>(stage, p, g, nzc, stream)
                                   : launch_3d<T, false, true, false>(stage, p, g, nzc, stream);
   }
@@ -315,7 +320,8 @@ cudaError_t launch_stage_halo(const Grid& g, int stage, const T* win, const T* u
   }
   const int nzc = (p.zhi - p.zlo + p.tz - 1) / p.tz;
   if constexpr (sizeof(T) == 8) {
-    if (g.tx == 16) return launch_3d<T, false, false, true, 16>(stage, p, g, nzc, stream);
+    if (g.tx == 16) return launch_3d<T, false, false, true, 16, 16>(stage, p, g, nzc, stream);
+    if (g.ty == 4) return launch_3d<T, true, false, true, 32, 4>(stage, p, g, nzc, stream);
   }
   return g.limiter == kLimWenoz ? launch_3d<T, true, false, true>(stage, p, g, nzc, stream)
                                 : launch_3d<T, false, false, true>(stage, p, g, nzc, stream);
@@ -325,7 +331,8 @@ cudaError_t launch_stage_halo(const Grid& g, int stage, const T* win, const T* u
 template <class T>
 cudaError_t prepare_stage_kernels_halo(const Grid& g) {
   if constexpr (sizeof(T) == 8) {
-    if (g.tx == 16) return prepare_3d<T, false, false, true, 16>();
+    if (g.tx == 16) return prepare_3d<T, false, false, true, 16, 16>();
+    if (g.ty == 4) return prepare_3d<T, true, false, true, 32, 4>();
   }
   return g.limiter == kLimWenoz ? prepare_3d<T, true, false, true>()
                                 : prepare_3d<T, false, false, true>();
