@@ -8,9 +8,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <algorithm>
-#include <functional>
 #include <new>
-#include <queue>
 #include <vector>
 
 #include "mhd_ctx.h"
@@ -210,17 +208,14 @@ static double launch_span(long long cols, int nz, int tz, long long slots) {
   const double a = tz + 1.0, b = (double)(nz - (chunks - 1) * tz) + 1.0;
   const long long n1 = cols * (chunks - 1);
   const long long q = n1 / slots, r = n1 % slots;  // full chunks per slot
-  std::priority_queue<double, std::vector<double>, std::greater<double>> freed;
-  double span = 0.0;
-  for (long long s = 0; s < slots; ++s) {
-    const double t = (s < r ? q + 1 : q) * a;
-    freed.push(t);
-    span = std::max(span, t);
-  }
-  for (long long c = 0; c < cols; ++c) {
-    const double t = freed.top() + b;
-    freed.pop();
-    freed.push(t);
+  // a last chunk starts on the slot that frees first: slots free at qa + ib and
+  // (q+1)a + jb, taken in the order of these times
+  double even = (double)q * a, odd = even + a;
+  double span = r ? odd : (q ? even : 0.0);
+  for (long long c = 0; c < cols;) {
+    double& t = r && odd < even ? odd : even;
+    c += &t == &odd ? r : slots - r;
+    t += b;
     span = std::max(span, t);
   }
   return span;
