@@ -138,8 +138,6 @@ MHD_HD T dot3_f(T a0, T b0, T a1, T b1, T a2, T b2, const Phys<T>& ph) {
   return fma_rn(a2, b2, fma_rn(a1, b1, mul_f(a0, b0, ph)));
 }
 
-MHD_HD double trsqrt(double x) { return rsqrt(x); }
-MHD_HD float trsqrt(float x) { return rsqrtf(x); }
 MHD_HD float tsqrt(float x) {
 #ifdef __CUDA_ARCH__
   return x > 0.0f ? x * rsqrtf(x) : 0.0f;
@@ -151,8 +149,6 @@ MHD_HD double tabs(double x) { return fabs(x); }
 MHD_HD float tabs(float x) { return fabsf(x); }
 MHD_HD double tmin(double a, double b) { return fmin(a, b); }
 MHD_HD float tmin(float a, float b) { return fminf(a, b); }
-MHD_HD double tmax(double a, double b) { return fmax(a, b); }
-MHD_HD float tmax(float a, float b) { return fmaxf(a, b); }
 
 // Bit-pattern helpers (the host build, used only by host-side harnesses,
 // goes through memcpy).
@@ -707,23 +703,24 @@ MHD_HD double limited_slope<double>(double dm, double dp, int lim) {
 // Half the limited slope, the step from the cell value to its faces: MC
 // min(|dm|, |dp|, |dm+dp|/4), minmod min(|dm|, |dp|)/2, with the common sign, 0
 // when the signs differ.  FP32: with the central value c between dm and dp, the
-// smallest of the three where it is positive, the largest where it is negative.
+// smallest of the three where it is positive, the largest where it is negative
+// (a NaN among them passes through these and the comparison with 0 drops it: 0).
 MHD_HD float min3(float a, float b, float c) {
 #if defined(__CUDA_ARCH__) && __CUDA_ARCH__ >= 1000
   float d;
-  asm("min.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  asm("min.NaN.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
   return d;
 #else
-  return fminf(fminf(a, b), c);
+  return a != a || b != b || c != c ? a + b + c : fminf(fminf(a, b), c);
 #endif
 }
 MHD_HD float max3(float a, float b, float c) {
 #if defined(__CUDA_ARCH__) && __CUDA_ARCH__ >= 1000
   float d;
-  asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
   return d;
 #else
-  return fmaxf(fmaxf(a, b), c);
+  return a != a || b != b || c != c ? a + b + c : fmaxf(fmaxf(a, b), c);
 #endif
 }
 MHD_HD float half_slope_mc(float dm, float dp, const Phys<float>&) {
@@ -731,7 +728,7 @@ MHD_HD float half_slope_mc(float dm, float dp, const Phys<float>&) {
   return fmaxf(min3(dm, dp, c), 0.0f) + fminf(max3(dm, dp, c), 0.0f);
 }
 MHD_HD float half_slope_minmod(float dm, float dp) {
-  return mul_rn(0.5f, fmaxf(fminf(dm, dp), 0.0f) + fminf(fmaxf(dm, dp), 0.0f));
+  return mul_rn(0.5f, fmaxf(min3(dm, dp, dp), 0.0f) + fminf(max3(dm, dp, dp), 0.0f));
 }
 // FP64: the same value as half of limited_slope, decided and scaled on the
 // integer pipe; |dm| + |dp| is the only FP64 operation.
@@ -770,8 +767,8 @@ MHD_HD T rot3(int dir, int j, T a, T b, T c) {
 // operations: about 95 per face, 130 where a lane of the warp is inside the
 // Alfven fan (the form that builds both sides' star and double-star states and
 // adds up the wave jumps took about 280 with CUDA's divisions and roots).
-// Orszag-Tang 256^3 FP64: 76.4 -> 47.4 ms per step, of which the fixed-point
-// reciprocals and roots 11.  Against a quadruple-precision evaluation its
+// Orszag-Tang 256^3 FP64: 76.4 -> 47.4 ms per step (44.0 with what came after), of
+// which the fixed-point reciprocals and roots 11.  Against a quadruple-precision evaluation its
 // error is at most that of the longer form (2e-16 to 3e-15 rms of the flux,
 // random, smooth, Mach-20, low- and high-beta and degenerate face states).
 template <int dir, class T>
