@@ -255,7 +255,7 @@ static int choose_tz(const mhd::Grid& g, int ctas_per_sm, double* span = nullptr
 // grid over the SMs.  At equal plans it is 1.3 % faster (256^3, one step 46.4 against
 // 47.0 ms; fewer halo conversions); 48^3: 536 -> 425 us.
 // WENO-Z: 32 x 4, for short last rows of tiles; a plane of it takes 0.54 of a 32 x 8
-// one (256^3, one RK3 step 102.5 against 94.4 ms for the same cells).
+// one (256^3, one RK3 step 205 against 189 ms for the same cells).
 static void choose_tile(mhd::Grid& g, int ctas_per_sm, int ty, bool glm, bool fp64) {
   double span = 0.0, other_span = 0.0;
   g.tx = 32;

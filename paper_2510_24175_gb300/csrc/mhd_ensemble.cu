@@ -7,7 +7,7 @@
 //   prepare (one thread per box: CFL dt and c_h from that box's reduced wave
 //   speed) -> grid sync -> stage 1 over all tiles -> grid sync -> stage 2
 //   over all tiles (reducing each box's next wave speed) -> grid sync.
-// The tile code is the same stage_tile() the per-box launches use, so every
+// The tile code is the same stage_tile_pairs() the per-box launches use, so every
 // box evolves bitwise as it would under its own mhd_step calls.  Grid syncs
 // are cooperative-group barriers: the cooperative launch guarantees that all
 // CTAs are co-resident (the launch fails otherwise), so no wait can hang.
@@ -34,6 +34,8 @@ namespace cg = cooperative_groups;
 
 namespace mhd {
 
+// Eight warps per CTA, 128 registers, two CTAs per SM.  (64 boxes of up to 128^3, 5 steps:
+// 41.6 ms; 57.4 with scalar loads, slopes and one slope array per direction.)
 constexpr int kEnsNW = 8;
 constexpr int kEnsTYs[2] = {8, 4};  // the tile heights of the two kernel instantiations
 

@@ -13,7 +13,7 @@ namespace mhd {
 // one warp issues an FP64 instruction at most every 64 clocks, so the unit
 // saturates only when at least four warps have FP64 work.  PLM: 32 x 8 or 16 x 16
 // (211 KB of shared memory), 16 warps of 128 registers (12 of 168: 256^3 step 46.8
-// instead of 44.0 ms).  WENO-Z: 32 x 8 (226 KB), 12 warps (16: 100 instead of 96 ms
+// instead of 44.0 ms).  WENO-Z: 32 x 8 (226 KB), 12 warps (16: 199 instead of 192 ms
 // per RK3 step of 256^3), or 32 x 4 with 8 warps.  FP32 (PLM and WENO-Z): 32 x 8
 // with 16 warps at 64 registers, two CTAs per SM: the kernels are bound by latency
 // and issue; with 24 and 16 warps per SM the PLM kernel took 2 and 8 % longer

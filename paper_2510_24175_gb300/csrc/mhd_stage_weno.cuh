@@ -13,6 +13,12 @@
 //      the z face k+1/2;
 //   D  flux divergence + Runge-Kutta combination (+ damping and the wave-speed
 //      reduction in the last stage).
+// A face's flux overwrites the minus value that only this face reads, and the
+// owners keep their z values in registers from B to C, so a 32 x 8 FP64 tile fits
+// in shared memory (226 KB).  Bound by the FP64 unit: Orszag-Tang 256^3, a step of
+// three stages 189 ms (335 with 32 x 4 tiles, scaled second differences, CUDA's
+// divisions and roots and the longer HLLD).  FP64 grids and the 1-D and 2-D FP32
+// ones (3-D FP32: mhd_stage_pairs.cuh).
 #pragma once
 
 #include "mhd_stage.cuh"
@@ -227,7 +233,7 @@ __global__ void __launch_bounds__(NW * 32, sizeof(T) == 4 && ZACT ? 2 : 1)
   // 3-D tiles: the warps without columns take the first kB rounds of the x, y
   // values and the first kC of the fluxes, the owners the rest besides their z
   // work, so that no phase ends in a round of a few warps (dealt out evenly with
-  // z on top: 256^3 RK3 step 96.1 instead of 94.4 ms)
+  // z on top: 256^3 RK3 step 192 instead of 189 ms)
   constexpr bool kDeal = ZACT && ZT0 > 0;
   constexpr int kB = (G::SXN + G::SYN + G::NINT + NT - 1) / NT;
   constexpr int kC = (G::ITEMS + G::NINT + NT - 1) / NT;
