@@ -48,12 +48,12 @@ sys.path.insert(0, ROOT)
 # smsp__inst_executed_pipe_fp64 x 32 / cells over the timed steps of this
 # bench's Orszag-Tang 256^3 run (profiles/).  They change whenever the kernel
 # does.
-FP64_INST_PER_CELL = {1: 1183.0, 2: 1211.0}
+FP64_INST_PER_CELL = {1: 688.3, 2: 711.5}
 # DRAM bytes per cell of the stage kernel's launches (ncu dram__bytes_read +
 # dram__bytes_write over the timed steps of this bench's 256^3 FP64 and 512^3
 # FP32 runs, profiles/); reported as the roofline's traffic per launch.  Set
 # to None whenever the kernel changes until they are captured again.
-TRAFFIC_BYTES_PER_CELL = {8: {1: 151.9, 2: 224.4}, 4: {1: 75.65, 2: 111.64}}
+TRAFFIC_BYTES_PER_CELL = {8: {1: 150.7, 2: 223.5}, 4: {1: 76.0, 2: 111.8}}
 # Nominal FP64 peak: 2 lanes/clk/SM x 152 SMs x 2.07 GHz = 629 G
 # lane-instructions/s (1.26 TFLOP/s counting an FMA as 2).  The measured one,
 # mhd_fp64_fma_rate in the same run, is reported beside it (about 1.68
@@ -64,15 +64,15 @@ FP64_PEAK_GINST = 2 * 152 * 2.07
 # / cells, turbulent box 512^3, stage 1 / stage 2; profiles/) and the issue
 # peak they run against: 4 warp-instructions per clock per SM (one per
 # scheduler) x 152 SMs x 2.07 GHz.
-FP32_WARP_INST_PER_CELL = {1: 74.19, 2: 80.10}
+FP32_WARP_INST_PER_CELL = {1: 53.59, 2: 57.05}
 ISSUE_PEAK_GINST = 4 * 152 * 2.07
 # FP64-pipe lane-instructions per cell of the FP64 WENO-Z stage kernel (ncu,
 # Orszag-Tang 256^3; first / middle / last SSP-RK3 stage).
-WENO_FP64_INST_PER_CELL = {"stage1": 3511.2, "stage_mid": 3529.2, "stage2": 3530.3}
+WENO_FP64_INST_PER_CELL = {"stage1": 2057.8, "stage_mid": 2076.7, "stage2": 2079.9}
 # Warp-instructions per cell of the FP32 WENO-Z stage kernel (ncu
 # smsp__inst_executed / cells, Orszag-Tang 256^3; first / middle / last
 # SSP-RK3 stage).
-WENO_FP32_WARP_INST_PER_CELL = {"stage1": 126.87, "stage_mid": 128.31, "stage2": 133.00}
+WENO_FP32_WARP_INST_PER_CELL = {"stage1": 106.62, "stage_mid": 107.62, "stage2": 110.86}
 # Algorithmic HBM bytes per cell: stage 1 reads U^n and writes U1 (18 words),
 # stage 2 reads U1 and U^n and writes U^{n+1} (27 words).
 WORDS_STAGE = {1: 18, 2: 27}
@@ -302,7 +302,8 @@ def roofline_of(prof, ncell, esize, hbm_peak, peak_kind, fp64, fma=None):
     tb = TRAFFIC_BYTES_PER_CELL.get(esize) if TRAFFIC_BYTES_PER_CELL else None
     traffic = ncell * (tb[1] * n1 + tb[2] * n2) / max(n1 + n2, 1) if tb else None
     hbm = {"bound": "hbm", "achieved": bytes_launch / (avg_ms * 1e-3) / 1e9, "peak": hbm_peak,
-           "unit": "GB/s", "traffic": traffic, "kernel": "rk_stage_kernel",
+           "unit": "GB/s", "traffic": traffic,
+           "kernel": "rk_stage_kernel" if esize == 8 else "rk_stage_pairs_kernel",
            "avg_launch_ms": avg_ms, "bytes_per_launch": bytes_launch,
            "peak_source": peak_kind}
     hbm["frac"] = hbm["achieved"] / hbm_peak
@@ -472,7 +473,7 @@ def main():
         ach32 = winst / ((t1 + t2) * 1e-3) / 1e9
         issue32 = {"bound": "alu", "achieved": ach32, "peak": ISSUE_PEAK_GINST,
                    "unit": "G warp-inst/s", "frac": ach32 / ISSUE_PEAK_GINST,
-                   "kernel": "rk_stage_kernel",
+                   "kernel": "rk_stage_pairs_kernel",
                    "peak_source": "4 warp-instructions/clk/SM (instruction issue) x 152 SMs x "
                                   "2.07 GHz; the FP32 kernel is issue-bound (ncu)"}
         fp32 = {"workload": f"turbulent_box_{args.n32}^3_fp32", "value": world * N32 * K / (ms32 * 1e-3),
@@ -606,14 +607,14 @@ def main():
                         paper_scheme[key]["roofline_issue"] = {
                             "bound": "alu", "achieved": ach, "peak": ISSUE_PEAK_GINST,
                             "unit": "G warp-inst/s", "frac": ach / ISSUE_PEAK_GINST,
-                            "kernel": "rk_stage_weno_kernel",
+                            "kernel": "rk_stage_pairs_kernel",
                             "warp_inst_per_cell": WENO_FP32_WARP_INST_PER_CELL}
                     nbytes = pw.ncell * 4 * sum(WORDS_STAGE_RK3[c] * profw[c][0]
                                                 for c in WORDS_STAGE_RK3)
                     achb = nbytes / (ms_k * 1e-3) / 1e9
                     paper_scheme[key]["roofline"] = {
                         "bound": "hbm", "achieved": achb, "peak": hbm_peak, "unit": "GB/s",
-                        "frac": achb / hbm_peak, "kernel": "rk_stage_weno_kernel",
+                        "frac": achb / hbm_peak, "kernel": "rk_stage_pairs_kernel",
                         "peak_source": peak_kind}
                 launches += sum(c for c, _ in profw.values())
                 if divb == m.MHD_DIVB_CT:  # edge, face and cell kernels per stage record
