@@ -95,7 +95,7 @@ __device__ __forceinline__ int ens_find(const EnsBox* boxes, int nbox, long long
   return lo;
 }
 
-template <int TY, int STAGE>
+template <int TY, int STAGE, bool WIDE>
 __device__ __forceinline__ void ens_stage(const EnsArgs& a, unsigned char* smem, double* wmax) {
   for (long long it = blockIdx.x; it < a.nitems; it += gridDim.x) {
     const int bi = ens_find(a.boxes, a.nbox, it);
@@ -113,16 +113,17 @@ __device__ __forceinline__ void ens_stage(const EnsArgs& a, unsigned char* smem,
     const int bx = (int)(j % B.ntx);
     const int by = (int)((j / B.ntx) % B.nty);
     const int bz = (int)(j / ((long long)B.ntx * B.nty));
-    stage_tile_pairs<TY, kEnsNW, STAGE, false, false, false>(
+    stage_tile_pairs<TY, kEnsNW, STAGE, false, WIDE, false>(
         p, sc, bx, by, bz, reinterpret_cast<float*>(smem), wmax);
   }
 }
 
 // 8 warps per CTA, two CTAs per SM: with 12 and 16 warps per CTA (80 and 64
 // registers, the per-box kernel's shape) the persistent kernel, which also keeps
-// a box's parameters, spills 500 bytes a thread and takes 56.0 and 56.6 ms for
-// five steps of 64 boxes against 49.5.
-template <int TY>
+// a box's parameters, spilled 500 bytes a thread and took 56.0 and 56.6 ms for
+// five steps of 64 boxes against 49.5 (41.6 with paired values).  WIDE: a box has
+// planes beyond 32-bit offsets (the tile code's 64-bit form).
+template <int TY, bool WIDE>
 __global__ void __launch_bounds__(kEnsNW * 32, 2) ensemble_kernel(const EnsArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ double wmax[kEnsNW];
@@ -131,11 +132,17 @@ __global__ void __launch_bounds__(kEnsNW * 32, 2) ensemble_kernel(const EnsArgs 
     const long long gt = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (gt < a.nbox) ens_prep(a.boxes[gt]);
     grid.sync();
-    ens_stage<TY, 1>(a, smem_raw, wmax);
+    ens_stage<TY, 1, WIDE>(a, smem_raw, wmax);
     grid.sync();
-    ens_stage<TY, 2>(a, smem_raw, wmax);
+    ens_stage<TY, 2, WIDE>(a, smem_raw, wmax);
     grid.sync();
   }
+}
+
+using EnsKernel = void (*)(EnsArgs);
+static EnsKernel ens_kernel(int k, bool wide) {
+  if (wide) return k ? ensemble_kernel<4, true> : ensemble_kernel<8, true>;
+  return k ? ensemble_kernel<4, false> : ensemble_kernel<8, false>;
 }
 
 }  // namespace mhd
@@ -154,6 +161,7 @@ struct mhd_ensemble {
   cudaStream_t stream;
   cudaStream_t cap;            // private stream the graph is captured on (the
                                // legacy default stream cannot be captured)
+  bool wide;                   // a box has planes of 4 GB or more
   size_t smem[2];              // per tile height (index of kEnsTYs)
   int grid_ctas[2];
   long long nitems;
@@ -259,8 +267,7 @@ static cudaError_t ens_launch(mhd_ensemble* e, int nsteps, cudaStream_t s) {
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return k ? cudaLaunchKernelEx(&cfg, mhd::ensemble_kernel<4>, a)
-           : cudaLaunchKernelEx(&cfg, mhd::ensemble_kernel<8>, a);
+  return cudaLaunchKernelEx(&cfg, mhd::ens_kernel(k, e->wide), a);
 }
 
 extern "C" {
@@ -324,6 +331,7 @@ int mhd_ensemble_create(const mhd_config* cfgs, int nbox, void* d_workspace, siz
   e->lam_ok.assign(nbox, false);
   e->tz.assign(nbox, 16);
   e->ty = 8;
+  e->wide = false;
   for (int b = 0; b < nbox; ++b) {
     mhd_ctx* c = e->ctx[b];
     EnsBox B;
@@ -339,6 +347,7 @@ int mhd_ensemble_create(const mhd_config* cfgs, int nbox, void* d_workspace, siz
     B.p.sy = c->grid.n[0];
     B.p.sz = (long long)c->grid.n[0] * c->grid.n[1];
     B.p.sv = c->grid.ncell;
+    e->wide = e->wide || B.p.sz * 4 >= (1ll << 32);
     B.p.limiter = c->grid.limiter;
     B.p.ph = mhd::make_phys<float>(c->grid);
     B.Ua = static_cast<float*>(c->Ua);
@@ -359,18 +368,18 @@ int mhd_ensemble_create(const mhd_config* cfgs, int nbox, void* d_workspace, siz
   e->smem[1] = (size_t)mhd::PairGeom<4, false>::WORDS * sizeof(float);
   int per_sm[2] = {0, 0}, nsm = 0, dev = 0;
   if (ce == cudaSuccess)
-    ce = cudaFuncSetAttribute(mhd::ensemble_kernel<8>,
+    ce = cudaFuncSetAttribute(mhd::ens_kernel(0, e->wide),
                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)e->smem[0]);
   if (ce == cudaSuccess)
-    ce = cudaFuncSetAttribute(mhd::ensemble_kernel<4>,
+    ce = cudaFuncSetAttribute(mhd::ens_kernel(1, e->wide),
                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)e->smem[1]);
   if (ce == cudaSuccess) ce = cudaGetDevice(&dev);
   if (ce == cudaSuccess) ce = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   if (ce == cudaSuccess)
-    ce = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm[0], mhd::ensemble_kernel<8>,
+    ce = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm[0], mhd::ens_kernel(0, e->wide),
                                                        mhd::kEnsNW * 32, e->smem[0]);
   if (ce == cudaSuccess)
-    ce = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm[1], mhd::ensemble_kernel<4>,
+    ce = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm[1], mhd::ens_kernel(1, e->wide),
                                                        mhd::kEnsNW * 32, e->smem[1]);
   if (ce != cudaSuccess || per_sm[0] < 1 || per_sm[1] < 1 || ens_layout(e) != MHD_OK) {
     for (auto* x : e->ctx) mhd_destroy(x);

@@ -10,14 +10,16 @@
 //     and a face's flux overwrites the lower state that only that face reads (45
 //     shared-memory values per face instead of 54, and no flux arrays);
 //   * global addresses are a warp-uniform plane and variable base plus the
-//     thread's 32-bit byte offset in the plane (launch_stage takes the HALO
-//     kernels, with 64-bit addresses, where a plane exceeds 4 GB).
+//     thread's 32-bit byte offset in the plane; the HALO form uses 64-bit ones,
+//     and grids with planes of 4 GB and more take it, with or without halo faces.
 // The arithmetic of a cell is that of every other instantiation, operation by
 // operation (packed instructions round like scalar ones).  Turbulent box 512^3, a
 // step of two stages: 24.8 ms (32.6 with scalar values, slopes in shared memory and
 // 16 warps per SM; 27.7 with 32 warps); Orszag-Tang 256^3 WENO-Z with constrained
 // transport, a step of three stages: 10.9 ms (13.6).
 #pragma once
+
+#include <type_traits>
 
 #include "mhd_stage.cuh"
 #include "mhd_wenoz.cuh"
@@ -228,10 +230,11 @@ __device__ __forceinline__ void stage_tile_pairs(const StageParams<float>& p,
   auto plane_z = [&](int zz) {
     return (long long)wrap(zz, p.n[2], p.bc_lo[2], p.bc_hi[2]) * p.sz;
   };
-  auto ldg = [](const float* base, unsigned off) {
+  using Off = std::conditional_t<HALO, unsigned long long, unsigned>;
+  auto ldg = [](const float* base, Off off) {
     return *reinterpret_cast<const float*>(reinterpret_cast<const char*>(base) + off);
   };
-  auto stg = [](float* base, unsigned off, float v) {
+  auto stg = [](float* base, Off off, float v) {
     *reinterpret_cast<float*>(reinterpret_cast<char*>(base) + off) = v;
   };
   // Load items: the tile's interior, its x halo, its y halo.  Item it: tile cell
@@ -305,7 +308,7 @@ __device__ __forceinline__ void stage_tile_pairs(const StageParams<float>& p,
   };
   CtCell<float> ctc;
   const bool valid = owner && x0 + ocol < nx && y0 + orow < ny;
-  const unsigned doff = (unsigned)((y0 + orow) * (unsigned)nx + (x0 + ocol)) * 4u;
+  const Off doff = (Off(y0 + orow) * Off(nx) + Off(x0 + ocol)) * 4u;
 
   // The z march; warm-up iterations as in stage_tile().
 #pragma unroll 1
