@@ -408,24 +408,30 @@ int mhd_ensemble_destroy(mhd_ensemble* ens);
  * MHD_ERR_CUDA (message in mhd_last_error(NULL)). */
 int mhd_fp64_fma_rate(void* stream, unsigned warp_mask, double out[3]);
 
-/* Launch planning, on the host only (no GPU, no CUDA call): the z-chunk depth
- * *tz (planes per CTA) that the 3-D stage launches of an n[0] x n[1] x n[2]
- * grid use, for column tiles of 32 x ty cells (ty: 8 for the 3-D kernels)
- * on nsm SMs holding ctas_per_sm stage CTAs each (1 for FP64, 2 for
- * FP32), and, if span is not
- * NULL, the modelled duration of one launch in plane iterations.  The model:
- * the CTAs start in launch order -- every column tile's full chunks, then
- * every column tile's last, possibly shorter, chunk -- each on the slot that
- * frees first, and a CTA takes its planes plus one for its warm-up; the
- * depth is the candidate (256, 192, 128, 96, 80, 64, 56, 48, 40, 32, 24, 20,
- * 16, 12, 8, 4; at most n[2], or 4) with the shortest launch, the deeper one
- * on a tie.  A grid with an extent of 1 is not 3-D: *tz = 1.  (FP64
- * contexts plan a second tile in the same way -- PLM with GLM cleaning 16 x 16
- * cells, with the depths 3 and 2 as well; WENO-Z 32 x 4 -- and take it when its
- * launch is no longer.)  The paper has
- * no counterpart: this is how the library spreads its stage launches over
- * the SMs.  Errors: MHD_ERR_INVALID (an extent, ty, nsm or ctas_per_sm below
- * 1, n or tz NULL; message in mhd_last_error(NULL)). */
+/* Launch planning, on the host only (no GPU, no CUDA call).
+ * mhd_plan_stage: the stage launches that a context of this configuration
+ * makes on nsm SMs, the plan that mhd_create takes: plan[0] x plan[1] cells of a
+ * column tile, plan[2] z planes per CTA, plan[3] warps per CTA, plan[4] CTAs per
+ * SM that the plan counts on, and, if span is not NULL, the modelled duration
+ * of one launch in plane iterations of such a tile.  3-D grids take 32 x 8
+ * tiles; FP64 ones also plan a second tile (PLM with GLM cleaning 16 x 16, with
+ * the depths 3 and 2 as well; WENO-Z 32 x 4, a plane of it counted as 0.54) and
+ * take it when its launch is no longer.  Errors: MHD_ERR_INVALID (a
+ * configuration that mhd_create refuses, nsm < 1, plan NULL; message in
+ * mhd_last_error(NULL)).
+ * mhd_plan_z_chunks: the depth alone, for given tiles of 32 x ty cells: *tz
+ * (planes per CTA) for an n[0] x n[1] x n[2] grid on nsm SMs holding
+ * ctas_per_sm CTAs each, and, if span is not NULL, the modelled duration.  The
+ * model of both: the CTAs start in launch order -- every column tile's full
+ * chunks, then every column tile's last, possibly shorter, chunk -- each on the
+ * slot that frees first, and a CTA takes its planes plus one for its warm-up;
+ * the depth is the candidate (256, 192, 128, 96, 80, 64, 56, 48, 40, 32, 24,
+ * 20, 16, 12, 8, 4; at most n[2], or 4) with the shortest launch, the deeper
+ * one on a tie.  A grid with an extent of 1 is not 3-D: *tz = 1.  The paper has
+ * no counterpart: this is how the library spreads its stage launches over the
+ * SMs.  Errors: MHD_ERR_INVALID (an extent, ty, nsm or ctas_per_sm below 1, n or
+ * tz NULL; message in mhd_last_error(NULL)). */
+int mhd_plan_stage(const mhd_config* cfg, int nsm, int plan[5], double* span);
 int mhd_plan_z_chunks(const int n[3], int ty, int nsm, int ctas_per_sm, int* tz,
                       double* span);
 
@@ -433,7 +439,7 @@ int mhd_plan_z_chunks(const int n[3], int ty, int nsm, int ctas_per_sm, int* tz,
  * message of the calling host thread's last failing call that has no context
  * (mhd_workspace_bytes, mhd_create, mhd_flux_batch, mhd_ensemble_create,
  * mhd_ensemble_workspace_bytes, mhd_conserved_sums_noalloc, mhd_fp64_fma_rate,
- * mhd_plan_z_chunks). */
+ * mhd_plan_stage, mhd_plan_z_chunks). */
 const char* mhd_last_error(const mhd_ctx* ctx);
 
 /* Releases the context (not the workspace). */

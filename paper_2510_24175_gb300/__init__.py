@@ -45,7 +45,8 @@ EXPORTED = ["mhd_config_default", "mhd_workspace_bytes", "mhd_create", "mhd_set_
             "mhd_ensemble_workspace_bytes", "mhd_ensemble_create", "mhd_ensemble_set_state",
             "mhd_ensemble_get_state", "mhd_ensemble_step", "mhd_ensemble_info",
             "mhd_ensemble_autotune", "mhd_ensemble_set_tiles", "mhd_ensemble_last_error",
-            "mhd_ensemble_destroy", "mhd_fp64_fma_rate", "mhd_plan_z_chunks"]
+            "mhd_ensemble_destroy", "mhd_fp64_fma_rate", "mhd_plan_stage",
+            "mhd_plan_z_chunks"]
 
 
 class MHDError(RuntimeError):
@@ -99,6 +100,7 @@ def lib():
         L.mhd_conserved_sums.argtypes = [vp, dp]
         L.mhd_flux_batch.argtypes = [vp, vp, vp, ctypes.c_longlong, i, d, d, i, vp]
         L.mhd_fp64_fma_rate.argtypes = [vp, ctypes.c_uint, ctypes.POINTER(ctypes.c_double)]
+        L.mhd_plan_stage.argtypes = [cfgp, i, ctypes.POINTER(ctypes.c_int), dp]
         L.mhd_plan_z_chunks.argtypes = [ctypes.POINTER(ctypes.c_int), i, i, i,
                                         ctypes.POINTER(ctypes.c_int), dp]
         L.mhd_adjoint_step.argtypes = [vp, vp, vp, vp, d, d]
@@ -318,11 +320,22 @@ def mhd_fp64_fma_rate(warp_mask: int = 0xFF) -> dict:
     return {"lane_fma_per_s": out[0], "lanes_per_clk_per_sm": out[1], "ms": out[2]}
 
 
+def mhd_plan_stage(cfg: mhd_config, nsm: int) -> dict:
+    """Host-only plan of a context's stage launches on nsm SMs (no GPU needed):
+    the column tile (tx, ty), planes per CTA tz, warps per CTA, CTAs counted per
+    SM, and the modelled duration of a launch in plane iterations."""
+    p = (ctypes.c_int * 5)()
+    span = ctypes.c_double(0.0)
+    _check(lib().mhd_plan_stage(ctypes.byref(cfg), int(nsm), p, ctypes.byref(span)),
+           what="mhd_plan_stage")
+    return {"tx": p[0], "ty": p[1], "tz": p[2], "warps": p[3], "ctas_per_sm": p[4],
+            "span": span.value}
+
+
 def mhd_plan_z_chunks(n, ty: int, nsm: int, ctas_per_sm: int):
-    """Host-only launch plan of the 3-D stage kernels (no GPU needed): the
-    z-chunk depth for an n[0] x n[1] x n[2] grid of 32 x ty column tiles on
-    nsm SMs with ctas_per_sm stage CTAs each, and the modelled launch
-    duration in plane iterations."""
+    """Host-only z-chunk depth of given 3-D tiles (no GPU needed): for an
+    n[0] x n[1] x n[2] grid of 32 x ty column tiles on nsm SMs with ctas_per_sm
+    stage CTAs each, and the modelled launch duration in plane iterations."""
     nn = (ctypes.c_int * 3)(*[int(x) for x in n])
     tz = ctypes.c_int(0)
     span = ctypes.c_double(0.0)

@@ -241,33 +241,66 @@ static int plan_tz(long long cols, int nz, long long slots, double* span_out, in
   return best;
 }
 
-static int choose_tz(const mhd::Grid& g, int ctas_per_sm, double* span = nullptr) {
-  if (g.ndim < 3) return 1;
+static int choose_tz(const mhd::Grid& g, double* span = nullptr) {
   const long long cols =
       (long long)((g.n[0] + g.tx - 1) / g.tx) * ((g.n[1] + g.ty - 1) / g.ty);
-  return plan_tz(cols, g.n[2], (long long)g.nsm * ctas_per_sm, span, g.tx == 32 ? 4 : 2);
+  const long long slots = (long long)g.nsm * g.per_sm;
+  if (g.ndim < 3) {
+    if (span) *span = launch_span(cols, 1, 1, slots);
+    return 1;
+  }
+  return plan_tz(cols, g.n[2], slots, span, g.tx == 32 ? 4 : 2);
 }
 
-// The 3-D column tile and z-chunk depth of a grid: 32 x 8 (ty), or for FP64 the
-// reconstruction's other shape where its launch is modelled no longer.
+// One tile shape's plan; returns the modelled span.
+static double plan_tile(mhd::Grid& g, bool fp64, int tx, int ty) {
+  size_t smem;
+  double span;
+  g.tx = tx;
+  g.ty = ty;
+  if (fp64)
+    mhd::stage_shape<double>(g, &smem, &g.warps);
+  else
+    mhd::stage_shape<float>(g, &smem, &g.warps);
+  g.per_sm = std::max(1, (int)(228 * 1024 / (smem + 1024)));
+  g.tz = choose_tz(g, &span);
+  return span;
+}
+
+// The stage launches of a grid: column tile, z-chunk depth, warps per CTA and CTAs
+// per SM.  3-D: 32 x 8 columns, or for FP64 the reconstruction's other shape where
+// its launch is modelled no longer.
 // PLM (GLM cleaning): 16 x 16, which pads fewer columns when nx ends in the first
 // half of a 32-cell tile, and whose thinner chunks (2 and 3 planes) spread a small
 // grid over the SMs.  At equal plans it is 1.3 % faster (256^3, one step 46.4 against
 // 47.0 ms; fewer halo conversions); 48^3: 536 -> 425 us.
 // WENO-Z: 32 x 4, for short last rows of tiles; a plane of it takes 0.54 of a 32 x 8
 // one (256^3, one RK3 step 205 against 189 ms for the same cells).
-static void choose_tile(mhd::Grid& g, int ctas_per_sm, int ty, bool glm, bool fp64) {
-  double span = 0.0, other_span = 0.0;
-  g.tx = 32;
-  g.ty = ty;
-  g.tz = choose_tz(g, ctas_per_sm, &span);
+// 2-D: one plane of 32 x 8 (PLM) or 32 x 4 tiles; 1-D: rows of 32.
+static double plan_stage(mhd::Grid& g, bool fp64, bool glm) {
   const bool weno = g.limiter == MHD_LIM_WENOZ;
-  if (g.ndim < 3 || !fp64 || (!weno && !glm)) return;
+  const double span = plan_tile(g, fp64, 32, g.ndim < 2 ? 1 : (g.ndim == 2 && weno ? 4 : 8));
+  if (g.ndim < 3 || !fp64 || (!weno && !glm)) return span;
   mhd::Grid o = g;
-  o.tx = weno ? 32 : 16;
-  o.ty = weno ? 4 : 16;
-  o.tz = choose_tz(o, ctas_per_sm, &other_span);
-  if ((weno ? 0.54 : 1.0) * other_span <= span) g = o;
+  const double other = weno ? plan_tile(o, fp64, 32, 4) : plan_tile(o, fp64, 16, 16);
+  if ((weno ? 0.54 : 1.0) * other > span) return span;
+  g = o;
+  return other;
+}
+
+int mhd_plan_stage(const mhd_config* cfg, int nsm, int plan[5], double* span) {
+  char msg[200];
+  int rc = validate(cfg, msg, sizeof(msg));
+  if (rc != MHD_OK) return mhd::free_fail(rc, "mhd_plan_stage: %s", msg);
+  if (nsm < 1 || !plan) return mhd::free_fail(MHD_ERR_INVALID, "mhd_plan_stage: bad argument");
+  mhd::Grid g;
+  fill_grid(cfg, &g);
+  g.nsm = nsm;
+  const double s = plan_stage(g, cfg->precision == MHD_FP64, cfg->divb == MHD_DIVB_GLM);
+  const int out[5] = {g.tx, g.ty, g.tz, g.warps, g.per_sm};
+  memcpy(plan, out, sizeof(out));
+  if (span) *span = s;
+  return MHD_OK;
 }
 
 int mhd_plan_z_chunks(const int n[3], int ty, int nsm, int ctas_per_sm, int* tz,
@@ -444,18 +477,11 @@ int mhd_create(const mhd_config* cfg, void* d_workspace, size_t bytes, void* str
       c->inv_dx_sum += 1.0 / c->grid.dx[d];
       c->dh_min = fmin(c->dh_min, c->grid.dx[d]);
     }
-  size_t smem;
-  int threads, ty;
-  if (c->esize == 8)
-    mhd::stage_shape<double>(c->grid, &smem, &threads, &ty);
-  else
-    mhd::stage_shape<float>(c->grid, &smem, &threads, &ty);
-  const int per_sm = (int)(228 * 1024 / (smem + 1024));
-  choose_tile(c->grid, per_sm < 1 ? 1 : per_sm, ty, cfg->divb == MHD_DIVB_GLM, c->esize == 8);
+  plan_stage(c->grid, c->esize == 8, cfg->divb == MHD_DIVB_GLM);
   {
     mhd::Grid gh = c->grid;  // the half-depth grid of mhd_step_host's last stage
     gh.n[2] = (gh.n[2] + 1) / 2;
-    c->tz_half = choose_tz(gh, per_sm < 1 ? 1 : per_sm);
+    c->tz_half = choose_tz(gh);
   }
   {
     // kernel attributes now, so that no later launch (a captured one in

@@ -25,8 +25,9 @@ struct Grid {
   int limiter;
   double gamma, rho_floor, p_floor;
   double dx[3];
-  int tx, ty;            // 3-D column tile of the stage kernel (see mhd_create)
+  int tx, ty;            // column tile of the stage kernel (plan_stage in mhd_api.cu)
   int tz;                // z planes per CTA of the stage kernel
+  int warps, per_sm;     // warps per CTA; CTAs per SM that the plan counts on
   int nsm;               // SM count of the device
 };
 
@@ -74,9 +75,9 @@ cudaError_t launch_ct_divb(const Grid& g, const T* b, unsigned long long* out_bi
 template <class T>
 cudaError_t prepare_stage_kernels(const Grid& g, bool ct);
 
-// Shared-memory bytes and threads of the stage kernel for this grid.
+// Shared-memory bytes and warps per CTA of the stage kernel for this grid's tile.
 template <class T>
-void stage_shape(const Grid& g, size_t* smem, int* threads, int* ty);
+void stage_shape(const Grid& g, size_t* smem, int* warps);
 
 // Auxiliary kernels (mhd_aux.cu).
 struct PrepArgs {

@@ -14,6 +14,6 @@ template cudaError_t launch_stage<float>(const Grid&, int, const float*, const f
                                          unsigned long long*, cudaStream_t, double, double,
                                          const float* const*, float*, int, int, int,
                                           unsigned int*);
-template void stage_shape<float>(const Grid&, size_t*, int*, int*);
+template void stage_shape<float>(const Grid&, size_t*, int*);
 template cudaError_t prepare_stage_kernels<float>(const Grid&, bool);
 }  // namespace mhd

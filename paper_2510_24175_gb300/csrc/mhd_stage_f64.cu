@@ -14,6 +14,6 @@ template cudaError_t launch_stage<double>(const Grid&, int, const double*, const
                                           unsigned long long*, cudaStream_t, double, double,
                                           const double* const*, double*, int, int, int,
                                           unsigned int*);
-template void stage_shape<double>(const Grid&, size_t*, int*, int*);
+template void stage_shape<double>(const Grid&, size_t*, int*);
 template cudaError_t prepare_stage_kernels<double>(const Grid&, bool);
 }  // namespace mhd

@@ -126,35 +126,18 @@ static cudaError_t launch_weno(const StageParams<T>& p, dim3 grid, cudaStream_t 
 }
 
 template <class T>
-void stage_shape(const Grid& g, size_t* smem, int* threads, int* ty) {
-  if (g.limiter == kLimWenoz) {
-    if (g.ndim == 3) {
-      *smem = smem_3d<T, true, 32, 8>();
-      *threads = stage_warps<T, true>(8) * 32;
-      *ty = 8;
-    } else if (g.ndim == 2) {
-      *smem = (size_t)WenoGeom<4, false>::WORDS * sizeof(T);
-      *threads = 256;
-      *ty = 4;
-    } else {
-      *smem = (size_t)WenoGeom<1, false>::WORDS * sizeof(T);
-      *threads = kNW1 * 32;
-      *ty = 1;
-    }
-    return;
-  }
+void stage_shape(const Grid& g, size_t* smem, int* warps) {
+  const bool weno = g.limiter == kLimWenoz;
   if (g.ndim == 3) {
-    *smem = smem_3d<T, false, 32, 8>();
-    *threads = stage_warps<T, false>(8) * 32;
-    *ty = 8;
+    *warps = weno ? stage_warps<T, true>(g.ty) : stage_warps<T, false>(g.ty);
+    *smem = weno ? (g.ty == 4 ? smem_3d<T, true, 32, 4>() : smem_3d<T, true, 32, 8>())
+                 : (g.tx == 16 ? smem_3d<T, false, 16, 16>() : smem_3d<T, false, 32, 8>());
   } else if (g.ndim == 2) {
-    *smem = (size_t)TileGeom<8, false>::WORDS * sizeof(T);
-    *threads = 8 * 32;
-    *ty = 8;
+    *warps = 8;
+    *smem = (weno ? WenoGeom<4, false>::WORDS : TileGeom<8, false>::WORDS) * sizeof(T);
   } else {
-    *smem = (size_t)TileGeom<1, false>::WORDS * sizeof(T);
-    *threads = kNW1 * 32;
-    *ty = 1;
+    *warps = kNW1;
+    *smem = (weno ? WenoGeom<1, false>::WORDS : TileGeom<1, false>::WORDS) * sizeof(T);
   }
 }
 
