@@ -56,8 +56,8 @@ FP64_INST_PER_CELL = {1: 688.3, 2: 711.5}
 TRAFFIC_BYTES_PER_CELL = {8: {1: 150.7, 2: 223.5}, 4: {1: 76.0, 2: 111.8}}
 # Nominal FP64 peak: 2 lanes/clk/SM x 152 SMs x 2.07 GHz = 629 G
 # lane-instructions/s (1.26 TFLOP/s counting an FMA as 2).  The measured one,
-# mhd_fp64_fma_rate in the same run, is reported beside it (about 1.68
-# lanes/clk/SM: the SM's FP64 unit is shared by its warps, and one warp issues
+# mhd_fp64_fma_rate in the same run, is reported beside it (1.99 lanes/clk/SM
+# for FMAs on register operands, 1.68 with a constant operand; the SM's FP64 unit is shared by its warps, and one warp issues
 # an FP64 instruction at most every 64 clocks).
 FP64_PEAK_GINST = 2 * 152 * 2.07
 # Warp-instructions per cell of the FP32 stage kernel (ncu smsp__inst_executed

@@ -399,7 +399,7 @@ int mhd_ensemble_destroy(mhd_ensemble* ens);
  * FP64 stage kernels' roofline (their bound is the SM's FP64 unit, not HBM):
  * one CTA of 8 warps per SM; every thread of the warps that warp_mask selects
  * (bit w: warp w; warp w runs on scheduler w mod 4; 0 or 0xff: all 8) runs 16
- * independent fused multiply-add chains, timed with CUDA events on `stream`
+ * independent fused multiply-add chains on register operands, timed with CUDA events on `stream`
  * (NULL: the legacy default stream) after one warm-up launch.  out[0] =
  * lane-FMAs per second over the device, out[1] = lane-FMAs per clock per SM
  * at the clock rate the device reports, out[2] = milliseconds of the timed

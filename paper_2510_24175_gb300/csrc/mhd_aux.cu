@@ -462,14 +462,24 @@ template cudaError_t launch_flux_batch<float>(const float*, const float*, float*
 
 // FP64 throughput probe: every thread of the warps selected by warp_mask
 // (bit w: warp w of the 8) runs 16 independent fused multiply-add chains
-// (a <- a b + c) for `iters` rounds.  The chains converge to c / (1 - b) and
-// stay finite; the sums are stored so that no chain is dead code.
+// (a <- a b + c) for `iters` rounds, all operands in registers (b and c of a
+// value that the compiler cannot see): the unit takes an instruction with a
+// constant operand less often, and the stage kernels use the register form.  The
+// chains converge to c / (1 - b) and stay finite; the sums are stored so that no
+// chain is dead code.
 __global__ void __launch_bounds__(256, 1) fma_rate_kernel(double* out, int iters,
                                                           unsigned warp_mask) {
   double a[16];
 #pragma unroll
   for (int i = 0; i < 16; ++i) a[i] = 1.0 + 1e-9 * (threadIdx.x + i);
-  const double b = 0.999999999, c = 1e-12;
+  __shared__ double slot[2];
+  if (threadIdx.x == 0) {
+    slot[0] = 0.999999999;
+    slot[1] = 1e-12;
+  }
+  __syncthreads();
+  const volatile double* v = slot;
+  const double b = v[0], c = v[1];
   const int n = (warp_mask >> (threadIdx.x >> 5)) & 1u ? iters : 0;
   for (int it = 0; it < n; ++it) {
 #pragma unroll

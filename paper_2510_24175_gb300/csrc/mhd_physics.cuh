@@ -121,9 +121,9 @@ MHD_HD double fma_rn(double a, double b, double c) { return fma(a, b, c); }
 MHD_HD float fma_rn(float a, float b, float c) { return fmaf(a, b, c); }
 // Sums, differences and products as fused multiply-adds with the constants 1
 // and -0 (exact, so each rounds once, as the plain operation does).  The FP64
-// unit takes a fused multiply-add with three register operands every 16.8
-// clocks per SM, but an addition, a multiplication or a fused multiply-add with
-// a constant operand only every 19.9.  The kernels therefore hold ph.one and
+// unit takes a fused multiply-add of a warp with three register operands every
+// 16.1 clocks, but an addition, a multiplication or a fused multiply-add with
+// a constant operand only every 19.1.  The kernels therefore hold ph.one and
 // ph.nzero in registers whose values the compiler cannot see (fp64_registers);
 // elsewhere they are plain constants.  FP32 uses the plain operations.
 MHD_HD double add_f(double a, double b, const Phys<double>& ph) { return fma(a, ph.one, b); }
@@ -172,11 +172,11 @@ MHD_HD double bits2d(long long b) {
 }
 
 // FP64 reciprocal and square root without FP64 instructions.  The SM's FP64
-// unit issues 1.68 lanes per clock against 128 for the integer and FP32
-// pipes, which idle beside it.  Clocks per warp and SM with the pipes full:
-// CUDA's correctly rounded reciprocal 83.5, this one 21.8; CUDA's square root
-// 141, this one 26.2 (a fused multiply-add takes 15.6).  A single-precision seed of the significand (relative
-// error < 2^-21) is corrected in 64-bit fixed point: the residual against the
+// unit issues 2 lanes per clock against 128 for the integer and FP32 pipes, which
+// idle beside it.  Time per warp and SM with the pipes full, in fused
+// multiply-adds: CUDA's correctly rounded reciprocal 5.4, this one 1.4; CUDA's
+// square root 9.0, this one 1.7.  A single-precision seed of the significand
+// (relative error < 2^-21) is corrected in 64-bit fixed point: the residual against the
 // full significand is exact to 2^-62, and the first- and second-order terms of
 // the correction leave less than 2^-61, so the rounded result is within 0.51
 // ulp.  Both need a biased exponent in [64, 1982] (in_fixed_range); other
