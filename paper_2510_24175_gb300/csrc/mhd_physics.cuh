@@ -184,12 +184,14 @@ MHD_HD double bits2d(long long b) {
 // take the CUDA function behind a branch.
 MHD_HD bool in_fixed_range(uint32_t hi) { return ((hi >> 20) & 0x7ffu) - 64u < 1919u; }
 
-MHD_HD double rcp_fixed(double x) {
+// seed: the single-precision reciprocal (square root: reciprocal root) function.
+template <class Seed>
+MHD_HD double rcp_fixed(double x, Seed seed) {
   const uint64_t b = (uint64_t)dbits(x);
   const uint32_t hi = (uint32_t)(b >> 32), lo = (uint32_t)b;
   // significand in [1, 2): xh 2^-31 + xl 2^-63
   const uint32_t xh = 0x80000000u | (hi << 11) | (lo >> 21), xl = lo << 11;
-  const float r0 = seed_rcp(bits_f32(0x3f800000u | ((xh >> 8) & 0x7fffffu)));
+  const float r0 = seed(bits_f32(0x3f800000u | ((xh >> 8) & 0x7fffffu)));
   const float r = fminf(fmaxf(r0, 0.5f), 0.99999994f);
   const uint32_t y = (f32_bits(r) << 8) | 0x80000000u;  // seed, units 2^-32
   const int32_t yh = (int32_t)(y >> 1);                 // the same, units 2^-31
@@ -204,14 +206,15 @@ MHD_HD double rcp_fixed(double x) {
   return bits2d((int64_t)((m + ex) | (b & 0x8000000000000000ull)));
 }
 
-MHD_HD double sqrt_fixed(double x) {
+template <class Seed>
+MHD_HD double sqrt_fixed(double x, Seed seed) {
   const uint64_t b = (uint64_t)dbits(x);
   const uint32_t hi = (uint32_t)(b >> 32);
   const uint32_t odd = ((hi >> 20) & 1u) ^ 1u;  // odd exponent: significand in [2, 4)
   // m in [1, 4), units 2^-62
   const uint64_t m = ((b & 0x000fffffffffffffull) | 0x0010000000000000ull) << (10 + odd);
   const float f = bits_f32((0x3f800000u + (odd << 23)) | (uint32_t)((b >> 29) & 0x7fffffu));
-  const float y0 = fminf(fmaxf(seed_rsqrt(f), 0.5f), 0.99999994f);
+  const float y0 = fminf(fmaxf(seed(f), 0.5f), 0.99999994f);
   const float s0 = fminf(fmaxf(f * y0, 1.0f), 1.9999999f);
   const uint32_t t = (f32_bits(s0) << 8) | 0x80000000u;                  // units 2^-31
   const int32_t yh = (int32_t)(((f32_bits(y0) << 8) | 0x80000000u) >> 1);  // units 2^-31
@@ -225,6 +228,13 @@ MHD_HD double sqrt_fixed(double x) {
   const uint64_t s = (q + 0x200u) >> 10;  // [2^52, 2^53]
   const uint64_t ex = (uint64_t)((((hi >> 20) + 1023u) >> 1) - 1u) << 52;
   return bits2d((int64_t)(s + ex));
+}
+
+MHD_HD double rcp_fixed(double x) {
+  return rcp_fixed(x, [](float f) { return seed_rcp(f); });
+}
+MHD_HD double sqrt_fixed(double x) {
+  return sqrt_fixed(x, [](float f) { return seed_rsqrt(f); });
 }
 
 // (The CUDA functions as volatile asm: otherwise the compiler evaluates them
