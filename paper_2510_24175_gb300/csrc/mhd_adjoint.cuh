@@ -362,7 +362,8 @@ MHD_HD void glm_hlld_flux_vjp(const T vl[kNV], const T vr[kNV], int dir, T ch, T
 }
 
 // Limited slope and its (piecewise constant) partial derivatives with
-// respect to the one-sided differences dm, dp.
+// respect to the one-sided differences dm, dp (what limited_slope_c encodes; for
+// the host tests, as slope_code_d).
 template <class T>
 MHD_HD T limited_slope_d(T dm, T dp, int lim, T& ddm, T& ddp) {
   ddm = T(0);

@@ -679,7 +679,9 @@ struct SpeedMax<double> {
 #endif
 
 // Limited slope (van Leer 1977): 0 when the one-sided differences disagree in
-// sign; minmod = smaller magnitude; MC = min(2|dm|, 2|dp|, |dm+dp|/2).
+// sign; minmod = smaller magnitude; MC = min(2|dm|, 2|dp|, |dm+dp|/2).  The kernels
+// take half of it (half_slope_mc, half_slope_minmod) or it with a derivative code
+// (limited_slope_c); the host tests compare with this one.
 template <class T>
 MHD_HD T limited_slope(T dm, T dp, int lim) {
   if (lim == kLimFlat || !(dm * dp > T(0))) return T(0);
@@ -740,8 +742,9 @@ MHD_HD float half_slope_mc(float dm, float dp, const Phys<float>&) {
 MHD_HD float half_slope_minmod(float dm, float dp) {
   return mul_rn(0.5f, fmaxf(min3(dm, dp, dp), 0.0f) + fminf(max3(dm, dp, dp), 0.0f));
 }
-// FP64: the same value as half of limited_slope, decided and scaled on the
-// integer pipe; |dm| + |dp| is the only FP64 operation.
+// FP64: decided and scaled on the integer pipe; |dm| + |dp| is the only FP64
+// operation.  (A NaN difference orders above infinity there: the slope is then the
+// other difference's.)
 MHD_HD double half_slope_mc(double dm, double dp, const Phys<double>& ph) {
   const long long a = dbits(dm), b = dbits(dp);
   const long long mask = 0x7fffffffffffffffll;
