@@ -138,13 +138,6 @@ MHD_HD T dot3_f(T a0, T b0, T a1, T b1, T a2, T b2, const Phys<T>& ph) {
   return fma_rn(a2, b2, fma_rn(a1, b1, mul_f(a0, b0, ph)));
 }
 
-MHD_HD float tsqrt(float x) {
-#ifdef __CUDA_ARCH__
-  return x > 0.0f ? x * rsqrtf(x) : 0.0f;
-#else
-  return sqrtf(x);
-#endif
-}
 MHD_HD double tabs(double x) { return fabs(x); }
 MHD_HD float tabs(float x) { return fabsf(x); }
 MHD_HD double tmin(double a, double b) { return fmin(a, b); }

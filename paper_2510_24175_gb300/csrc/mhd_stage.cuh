@@ -407,6 +407,7 @@ __device__ __forceinline__ void stage_tile(const StageParams<T>& p, const StepSc
     if (r < 0 || r >= TY) return yh + (r < 0 ? r + 2 : r - TY + 2) * TX + c;
     return cur + r * TX + c;
   };
+  static_assert(sizeof(T) == 8 || !ZACT, "3-D FP32: mhd_stage_pairs.cuh");
   static_assert(!CT || ZACT, "constrained transport is 3-D only");
   static_assert(!HALO || (ZACT && !CT), "halo faces: 3-D GLM kernels only");
   // staggered normal field on the lower d-face of tile cell (r, c) of plane zz

@@ -93,13 +93,14 @@ struct WenoGeom {
 
 // CT: constrained transport, HALO: halo faces, as in stage_tile() (mhd_stage.cuh).
 template <class T, int TY, int NW, int STAGE, bool ZACT, bool CT, bool HALO = false>
-__global__ void __launch_bounds__(NW * 32, sizeof(T) == 4 && ZACT ? 2 : 1)
+__global__ void __launch_bounds__(NW * 32, 1)
     rk_stage_weno_kernel(const StageParams<T> p) {
   using G = WenoGeom<TY, ZACT>;
   constexpr int NT = NW * 32;
   constexpr int TX = G::TX;
   constexpr int ZT0 = NT - G::NINT;
   static_assert(ZT0 >= 0, "need one thread per tile column");
+  static_assert(sizeof(T) == 8 || !ZACT, "3-D FP32: mhd_stage_pairs.cuh");
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ double wmax[NW];
   T* ring = reinterpret_cast<T*>(smem_raw);
