@@ -28,8 +28,16 @@ constexpr int stage_warps(int ty) {
 // tile take two rounds of one warp, and a warp alone issues an FP64 instruction
 // every 64 clocks whether one lane is active or all are: a second warp takes the
 // second round at the same time (1024 cells, stages 1 and 2: 24 and 28 us -> 14
-// and 17.5 us).
+// and 17.5 us).  FP32 grids of more tiles than the GPU has schedulers take one
+// warp: their schedulers have other tiles to issue from, and the second warp costs
+// its own prologue and barriers (PLM, 20 steps: 512 tiles 0.22 ms with two warps,
+// 0.25 with one; 1024 tiles 0.27, 0.26; 2048 tiles 0.43, 0.34; eight steps of
+// 32768 tiles 1.45, 0.98).
 constexpr int kNW1 = 2;
+template <class T>
+constexpr bool one_warp(const Grid& g) {
+  return sizeof(T) == 4 && g.ndim == 1 && (g.n[0] + 31) / 32 > 4 * g.nsm;
+}
 
 // The dynamic shared-memory limit of a kernel is set once per device (a
 // driver call per launch costs more than a small grid's kernel).  One flag
@@ -136,7 +144,7 @@ void stage_shape(const Grid& g, size_t* smem, int* warps) {
     *warps = 8;
     *smem = (weno ? WenoGeom<4, false>::WORDS : TileGeom<8, false>::WORDS) * sizeof(T);
   } else {
-    *warps = kNW1;
+    *warps = one_warp<T>(g) ? 1 : kNW1;
     *smem = (weno ? WenoGeom<1, false>::WORDS : TileGeom<1, false>::WORDS) * sizeof(T);
   }
 }
@@ -169,6 +177,16 @@ cudaError_t prepare_stage_kernels(const Grid& g, bool ct) {
   using W1 = WenoGeom<1, false>;
   using P2 = TileGeom<8, false>;
   using P1 = TileGeom<1, false>;
+  if constexpr (sizeof(T) == 4) {
+    if (weno && g.warps == 1) {
+      MHD_SET3(rk_stage_weno_kernel, W1, 1, 1);
+      return e;
+    }
+    if (g.warps == 1) {
+      MHD_SET3(rk_stage_kernel, P1, 1, 1);
+      return e;
+    }
+  }
   if (weno && g.ndim == 2) {
     MHD_SET3(rk_stage_weno_kernel, W2, 4, 8);
   } else if (weno) {
@@ -264,6 +282,13 @@ cudaError_t launch_stage(const Grid& g, int stage, const T* win, const T* un, T*
       return launch_weno<T, 4, 8, 3, false>(p, grid, stream);
     }
     dim3 grid((g.n[0] + 31) / 32, 1, 1);
+    if constexpr (sizeof(T) == 4) {
+      if (g.warps == 1) {
+        if (stage == 1) return launch_weno<T, 1, 1, 1, false>(p, grid, stream);
+        if (stage == 2) return launch_weno<T, 1, 1, 2, false>(p, grid, stream);
+        return launch_weno<T, 1, 1, 3, false>(p, grid, stream);
+      }
+    }
     if (stage == 1) return launch_weno<T, 1, kNW1, 1, false>(p, grid, stream);
     if (stage == 2) return launch_weno<T, 1, kNW1, 2, false>(p, grid, stream);
     return launch_weno<T, 1, kNW1, 3, false>(p, grid, stream);
@@ -275,6 +300,13 @@ cudaError_t launch_stage(const Grid& g, int stage, const T* win, const T* un, T*
     return launch_one<T, 8, 8, 3, false>(p, grid, stream);
   }
   dim3 grid((g.n[0] + 31) / 32, 1, 1);
+  if constexpr (sizeof(T) == 4) {
+    if (g.warps == 1) {
+      if (stage == 1) return launch_one<T, 1, 1, 1, false>(p, grid, stream);
+      if (stage == 2) return launch_one<T, 1, 1, 2, false>(p, grid, stream);
+      return launch_one<T, 1, 1, 3, false>(p, grid, stream);
+    }
+  }
   if (stage == 1) return launch_one<T, 1, kNW1, 1, false>(p, grid, stream);
   if (stage == 2) return launch_one<T, 1, kNW1, 2, false>(p, grid, stream);
   return launch_one<T, 1, kNW1, 3, false>(p, grid, stream);

@@ -62,6 +62,14 @@ def test_plans_of_named_grids(n, limiter, prec, tile):
     assert (p["tx"], p["ty"], p["tz"]) == tile
 
 
+@pytest.mark.parametrize("n,prec,warps", [(32 * 608, m.MHD_FP32, 2), (32 * 608 + 1, m.MHD_FP32, 1),
+                                          (1 << 20, m.MHD_FP32, 1), (1 << 20, m.MHD_FP64, 2)])
+@pytest.mark.parametrize("limiter", [MC, WZ])
+def test_warps_of_1d_tiles(n, prec, warps, limiter):
+    assert m.mhd_plan_stage(m.Config(n=(n, 1, 1), limiter=limiter, precision=prec).c(),
+                            152)["warps"] == warps
+
+
 def test_bad_arguments_are_rejected():
     ok = m.Config(n=(8, 8, 8)).c()
     for cfg, nsm in [(ok, 0), (m.Config(n=(8, 1, 8)).c(), 152),
