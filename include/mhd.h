@@ -416,6 +416,7 @@ int mhd_fp64_fma_rate(void* stream, unsigned warp_mask, double out[3]);
  * of one launch in plane iterations of such a tile.  3-D grids take 32 x 8
  * tiles; FP64 ones also plan a second tile (PLM with GLM cleaning 16 x 16, with
  * the depths 3 and 2 as well; WENO-Z 32 x 4, a plane of it counted as 0.54) and
+ * FP32 WENO-Z ones one CTA per SM beside two (a plane counted as 0.59), and
  * take it when its launch is no longer.  1-D FP32 grids of more than 4 nsm tiles
  * take one warp per tile, other 1-D grids two.  Errors: MHD_ERR_INVALID (a
  * configuration that mhd_create refuses, nsm < 1, plan NULL; message in

@@ -253,7 +253,7 @@ static int choose_tz(const mhd::Grid& g, double* span = nullptr) {
 }
 
 // One tile shape's plan; returns the modelled span.
-static double plan_tile(mhd::Grid& g, bool fp64, int tx, int ty) {
+static double plan_tile(mhd::Grid& g, bool fp64, int tx, int ty, int per_sm = 2) {
   size_t smem;
   double span;
   g.tx = tx;
@@ -262,7 +262,7 @@ static double plan_tile(mhd::Grid& g, bool fp64, int tx, int ty) {
     mhd::stage_shape<double>(g, &smem, &g.warps);
   else
     mhd::stage_shape<float>(g, &smem, &g.warps);
-  g.per_sm = std::max(1, (int)(228 * 1024 / (smem + 1024)));
+  g.per_sm = std::max(1, std::min(per_sm, (int)(228 * 1024 / (smem + 1024))));
   g.tz = choose_tz(g, &span);
   return span;
 }
@@ -276,14 +276,23 @@ static double plan_tile(mhd::Grid& g, bool fp64, int tx, int ty) {
 // 47.0 ms; fewer halo conversions); 48^3: 536 -> 425 us.
 // WENO-Z: 32 x 4, for short last rows of tiles; a plane of it takes 0.54 of a 32 x 8
 // one (256^3, one RK3 step 205 against 189 ms for the same cells).
+// FP32 WENO-Z: the same tile at one CTA per SM and 128 registers, whose CTAs are
+// faster than two that share an SM and spill, where the plan does not need the
+// second slot (RK3 with GLM, ten steps: 48^3 0.99 against 1.21 ms, 96 x 96 x 48 2.48
+// against 3.18, 88^3 3.85 against 4.48; with constrained transport 1.61 times the span
+// is even, 1.8 times 4-12 % slower).  Large grids fill both slots: 256^3, 22.2 ms for
+// three steps against 25.9.
 // 2-D: one plane of 32 x 8 (PLM) or 32 x 4 tiles; 1-D: rows of 32.
 static double plan_stage(mhd::Grid& g, bool fp64, bool glm) {
   const bool weno = g.limiter == MHD_LIM_WENOZ;
   const double span = plan_tile(g, fp64, 32, g.ndim < 2 ? 1 : (g.ndim == 2 && weno ? 4 : 8));
-  if (g.ndim < 3 || !fp64 || (!weno && !glm)) return span;
+  if (g.ndim < 3 || (!weno && (!fp64 || !glm))) return span;
   mhd::Grid o = g;
-  const double other = weno ? plan_tile(o, fp64, 32, 4) : plan_tile(o, fp64, 16, 16);
-  if ((weno ? 0.54 : 1.0) * other > span) return span;
+  // the other shape's weight: its time a plane over the first one's
+  const double w = !fp64 ? 0.59 : (weno ? 0.54 : 1.0);
+  const double other = !fp64 ? plan_tile(o, fp64, 32, 8, 1)
+                             : (weno ? plan_tile(o, fp64, 32, 4) : plan_tile(o, fp64, 16, 16));
+  if (w * other > span) return span;
   g = o;
   return other;
 }

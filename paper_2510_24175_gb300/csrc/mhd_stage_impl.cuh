@@ -17,7 +17,8 @@ namespace mhd {
 // per RK3 step of 256^3), or 32 x 4 with 8 warps.  FP32 (PLM and WENO-Z): 32 x 8
 // with 16 warps at 64 registers, two CTAs per SM: the kernels are bound by latency
 // and issue; with 24 and 16 warps per SM the PLM kernel took 2 and 8 % longer
-// (512^3).  2-D grids use the 32 x 8 (PLM) or 32 x 4 (WENO-Z) tile with a single
+// (512^3).  WENO-Z launches that do not fill two CTAs per SM take one of 128
+// registers (plan_stage).  2-D grids use the 32 x 8 (PLM) or 32 x 4 (WENO-Z) tile with a single
 // plane; 1-D grids a 32-cell row.
 template <class T, bool WENO>
 constexpr int stage_warps(int ty) {
@@ -78,12 +79,13 @@ constexpr size_t smem_3d() {
 
 // The 3-D stage kernels: FP64 rk_stage_kernel / rk_stage_weno_kernel, FP32
 // rk_stage_pairs_kernel (mhd_stage_pairs.cuh).
-template <class T, bool WENO, int STAGE, bool CT, bool HALO, int TX = 32, int TY = 8>
+template <class T, bool WENO, int STAGE, bool CT, bool HALO, int TX = 32, int TY = 8,
+          int PER_SM = 2>
 struct Kern3D {
   static constexpr int NW = stage_warps<T, WENO>(TY);
   static constexpr auto get() {
     if constexpr (sizeof(T) == 4)
-      return rk_stage_pairs_kernel<TY, NW, STAGE, CT, HALO, WENO>;
+      return rk_stage_pairs_kernel<TY, NW, STAGE, CT, HALO, WENO, PER_SM>;
     else if constexpr (WENO)
       return rk_stage_weno_kernel<T, TY, NW, STAGE, true, CT, HALO>;
     else
@@ -100,18 +102,24 @@ struct Kern3D {
     return cudaGetLastError();
   }
 };
-template <class T, bool WENO, bool CT, bool HALO, int TX = 32, int TY = 8>
+template <class T, bool WENO, bool CT, bool HALO, int TX = 32, int TY = 8, int PER_SM = 2>
 static cudaError_t launch_3d(int stage, const StageParams<T>& p, const Grid& g, int nzc,
                              cudaStream_t s) {
-  if (stage == 1) return Kern3D<T, WENO, 1, CT, HALO, TX, TY>::launch(p, g, nzc, s);
-  if (stage == 2) return Kern3D<T, WENO, 2, CT, HALO, TX, TY>::launch(p, g, nzc, s);
-  return Kern3D<T, WENO, 3, CT, HALO, TX, TY>::launch(p, g, nzc, s);
+  if constexpr (sizeof(T) == 4 && WENO && PER_SM == 2) {
+    if (g.per_sm == 1) return launch_3d<T, WENO, CT, HALO, TX, TY, 1>(stage, p, g, nzc, s);
+  }
+  if (stage == 1) return Kern3D<T, WENO, 1, CT, HALO, TX, TY, PER_SM>::launch(p, g, nzc, s);
+  if (stage == 2) return Kern3D<T, WENO, 2, CT, HALO, TX, TY, PER_SM>::launch(p, g, nzc, s);
+  return Kern3D<T, WENO, 3, CT, HALO, TX, TY, PER_SM>::launch(p, g, nzc, s);
 }
-template <class T, bool WENO, bool CT, bool HALO, int TX = 32, int TY = 8>
-static cudaError_t prepare_3d() {
-  cudaError_t e = Kern3D<T, WENO, 1, CT, HALO, TX, TY>::prepare();
-  if (e == cudaSuccess) e = Kern3D<T, WENO, 2, CT, HALO, TX, TY>::prepare();
-  if (e == cudaSuccess) e = Kern3D<T, WENO, 3, CT, HALO, TX, TY>::prepare();
+template <class T, bool WENO, bool CT, bool HALO, int TX = 32, int TY = 8, int PER_SM = 2>
+static cudaError_t prepare_3d(const Grid& g) {
+  if constexpr (sizeof(T) == 4 && WENO && PER_SM == 2) {
+    if (g.per_sm == 1) return prepare_3d<T, WENO, CT, HALO, TX, TY, 1>(g);
+  }
+  cudaError_t e = Kern3D<T, WENO, 1, CT, HALO, TX, TY, PER_SM>::prepare();
+  if (e == cudaSuccess) e = Kern3D<T, WENO, 2, CT, HALO, TX, TY, PER_SM>::prepare();
+  if (e == cudaSuccess) e = Kern3D<T, WENO, 3, CT, HALO, TX, TY, PER_SM>::prepare();
   return e;
 }
 // The FP32 kernels without halo faces address a plane with 32 bits; larger planes
@@ -156,14 +164,14 @@ template <class T>
 cudaError_t prepare_stage_kernels(const Grid& g, bool ct) {
   const bool weno = g.limiter == kLimWenoz;
   if constexpr (sizeof(T) == 8) {
-    if (ct && g.ty == 4) return prepare_3d<T, true, true, false, 32, 4>();
+    if (ct && g.ty == 4) return prepare_3d<T, true, true, false, 32, 4>(g);
   }
-  if (ct) return weno ? prepare_3d<T, true, true, false>() : prepare_3d<T, false, true, false>();
+  if (ct) return weno ? prepare_3d<T, true, true, false>(g) : prepare_3d<T, false, true, false>(g);
   if (g.ndim == 3) {
     // FP64, and planes beyond 32-bit offsets: the halo-capable kernels (launch_stage)
     if (sizeof(T) == 8 || wide_plane<T>(g)) return prepare_stage_kernels_halo<T>(g);
     if constexpr (sizeof(T) == 4)
-      return weno ? prepare_3d<T, true, false, false>() : prepare_3d<T, false, false, false>();
+      return weno ? prepare_3d<T, true, false, false>(g) : prepare_3d<T, false, false, false>(g);
   }
   cudaError_t e = cudaSuccess;
   // the three stages of one variant <TY, NW> with geometry G
@@ -346,11 +354,11 @@ cudaError_t launch_stage_halo(const Grid& g, int stage, const T* win, const T* u
 template <class T>
 cudaError_t prepare_stage_kernels_halo(const Grid& g) {
   if constexpr (sizeof(T) == 8) {
-    if (g.tx == 16) return prepare_3d<T, false, false, true, 16, 16>();
-    if (g.ty == 4) return prepare_3d<T, true, false, true, 32, 4>();
+    if (g.tx == 16) return prepare_3d<T, false, false, true, 16, 16>(g);
+    if (g.ty == 4) return prepare_3d<T, true, false, true, 32, 4>(g);
   }
-  return g.limiter == kLimWenoz ? prepare_3d<T, true, false, true>()
-                                : prepare_3d<T, false, false, true>();
+  return g.limiter == kLimWenoz ? prepare_3d<T, true, false, true>(g)
+                                : prepare_3d<T, false, false, true>(g);
 }
 
 }  // namespace mhd

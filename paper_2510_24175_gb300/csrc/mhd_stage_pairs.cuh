@@ -475,8 +475,9 @@ __device__ __forceinline__ void stage_tile_pairs(const StageParams<float>& p,
   __syncthreads();  // the CTA may start another tile on the same shared memory
 }
 
-template <int TY, int NW, int STAGE, bool CT, bool HALO, bool WENO>
-__global__ void __launch_bounds__(NW * 32, 2)
+// PER_SM: CTAs per SM (2: 64 registers a thread, 1: 128).
+template <int TY, int NW, int STAGE, bool CT, bool HALO, bool WENO, int PER_SM>
+__global__ void __launch_bounds__(NW * 32, PER_SM)
     rk_stage_pairs_kernel(const StageParams<float> p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ double wmax[NW];

@@ -20,6 +20,10 @@ SHAPES = {
                                       (32, 4, CANDIDATES, 0.54, 8, 1)],
     (m.MHD_FP32, MC, m.MHD_DIVB_GLM): [(32, 8, CANDIDATES, 1.0, 16, 2)],
     (m.MHD_FP32, MC, m.MHD_DIVB_CT): [(32, 8, CANDIDATES, 1.0, 16, 2)],
+    (m.MHD_FP32, WZ, m.MHD_DIVB_GLM): [(32, 8, CANDIDATES, 1.0, 16, 2),
+                                       (32, 8, CANDIDATES, 0.59, 16, 1)],
+    (m.MHD_FP32, WZ, m.MHD_DIVB_CT): [(32, 8, CANDIDATES, 1.0, 16, 2),
+                                      (32, 8, CANDIDATES, 0.59, 16, 1)],
 }
 
 
@@ -46,8 +50,8 @@ def test_plan_is_the_shortest_simulated_launch(key):
         cfg = m.Config(n=n, precision=key[0], limiter=key[1], divb=key[2]).c()
         got = m.mhd_plan_stage(cfg, nsm)
         assert got == expected(n, SHAPES[key], nsm), (n, nsm)
-        taken.add((got["tx"], got["ty"]))
-    assert taken == {s[:2] for s in SHAPES[key]}
+        taken.add((got["tx"], got["ty"], got["ctas_per_sm"]))
+    assert taken == {s[:2] + s[5:] for s in SHAPES[key]}
 
 
 @pytest.mark.parametrize("n,limiter,prec,tile", [
