@@ -526,8 +526,11 @@ MHD_HD T cell_max_speed(const T u[kNV], const Phys<T>& ph, int ndim, unsigned& f
     lam = nan_max(lam, tabs(v[kVY]) + fast_speed(ri, gp, b2, mul_rn(v[kBY], v[kBY]), ph));
   if (ndim > 2)
     lam = nan_max(lam, tabs(v[kVZ]) + fast_speed(ri, gp, b2, mul_rn(v[kBZ], v[kBZ]), ph));
-  // NaN anywhere in the cell (psi included) makes the speed NaN
-  if (is_nan(v[kPSI]) || is_nan(lam)) lam = T(NAN);
+  // NaN anywhere in the cell (psi included) makes the speed NaN, and so does an
+  // overflow of a^2 (see fast_speed2x): the discriminant is then minus infinity or
+  // NaN, which the positive part turns into a finite, wrong speed
+  const T a = mul_rn(gp + b2, ri);
+  if (is_nan(v[kPSI]) || is_nan(lam) || !(mul_rn(a, a) < T(INFINITY))) lam = T(NAN);
   return lam;
 }
 
