@@ -155,7 +155,10 @@ int mhd_divb_max(mhd_ctx* ctx, double* out);
 
 /* CFL time step of the current state (Section 3.2's explicit scheme; the rule
  * is lambda = max over cells and active d of |v_d| + c_f,d, c_h = lambda,
- * dt = cfl / (c_h sum_d 1/dx_d)).  Synchronises.  Either pointer may be NULL. */
+ * dt = cfl / (c_h sum_d 1/dx_d)).  Synchronises.  Either pointer may be NULL.
+ * Steps need the squares of the squared fast speeds in range: where they overflow
+ * lambda is NaN, and a step whose c_h is lambda is refused (MHD_ERR_NONFINITE) for
+ * lambda below 2^-34 (FP32) or 2^-262 (FP64). */
 int mhd_dt(mhd_ctx* ctx, double* dt, double* ch);
 
 /* One Runge-Kutta step (Section 3.2: every stage runs the five steps listed
@@ -215,7 +218,8 @@ int mhd_step_record(mhd_ctx* ctx, double* d_out);
  * reduction are not counted:
  *   counters[0]: density floor (rho < rho_floor: rho = rho_floor);
  *   counters[1]: pressure floor (p < p_floor: p = p_floor);
- *   counters[2]: device status bits (non-zero: a non-finite dt or c_h);
+ *   counters[2]: device status bits (non-zero: a non-finite dt or c_h, or a
+ *                maximum wave speed below 2^-34 (FP32) or 2^-262 (FP64));
  *   counters[3]: MHD_FP32 only: cells whose FP32 pressure fell below p_floor
  *                or below 1e-3 (gamma-1) E and was recomputed in FP64 (the
  *                floor decision then taken in FP64). */

@@ -748,6 +748,7 @@ static int launch_prepare(mhd_ctx* c, double dt, double ch) {
   a.ch_req = ch;
   a.cfl = c->cfg.cfl;
   a.inv_dx_sum = c->inv_dx_sum;
+  a.lam_min = mhd::speed_min(c->esize == 8);
   a.t_end = c->cfg.t_end;
   a.glm_alpha = c->cfg.glm_alpha;
   a.dh_min = c->dh_min;

@@ -26,7 +26,7 @@ template Phys<float> make_phys<float>(const Grid&);
 // ---------------------------------------------------------------- prepare --
 // One thread.  dt rule: c_h = lambda (max |v_d| + c_f,d of the state),
 // dt = cfl / (c_h sum_active 1/dx_d), clamped so the step ends at t_end.
-// A non-finite or non-positive dt / c_h sets status bit 1 and turns the step
+// A non-finite or non-positive dt / c_h, or lambda below lam_min, sets status bit 1 and turns the step
 // into a no-op (dt = 0, damping 1), so the state is preserved for inspection.
 __global__ void prep_kernel(const PrepArgs a, StepScalars* sc, unsigned long long* lam_bits,
                             unsigned int* est_bits, unsigned int* status) {
@@ -39,7 +39,8 @@ __global__ void prep_kernel(const PrepArgs a, StepScalars* sc, unsigned long lon
     dt = a.cfl / (ch * a.inv_dx_sum);
     if (a.t_end > 0.0) dt = fmin(dt, a.t_end - t);
   }
-  bool bad = !(ch > 0.0) || !(ch < INFINITY) || !(dt >= 0.0) || !(dt < INFINITY);
+  bool bad = !(ch > 0.0) || !(ch < INFINITY) || !(dt >= 0.0) || !(dt < INFINITY) ||
+             (!(a.ch_req > 0.0) && lam < a.lam_min);
   if (bad) {
     atomicOr(status, 1u);
     dt = 0.0;

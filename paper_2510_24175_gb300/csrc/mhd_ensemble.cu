@@ -69,7 +69,7 @@ __device__ __forceinline__ void ens_prep(EnsBox& b) {
   const double t = b.sc.t;
   double dt = b.cfl / (ch * b.inv_dx_sum);
   if (b.t_end > 0.0) dt = fmin(dt, b.t_end - t);
-  if (!(ch > 0.0) || !(ch < INFINITY) || !(dt >= 0.0) || !(dt < INFINITY)) {
+  if (!(ch >= speed_min(false)) || !(ch < INFINITY) || !(dt >= 0.0) || !(dt < INFINITY)) {
     atomicOr(&b.status, 1u);
     dt = 0.0;
     ch = 1.0;

@@ -83,9 +83,13 @@ void stage_shape(const Grid& g, size_t* smem, int* warps);
 struct PrepArgs {
   double dt_req, ch_req;  // > 0: use as given
   double cfl, inv_dx_sum, t_end, glm_alpha, dh_min;
+  double lam_min;  // smallest wave speed of a step (speed_min)
   double dx[3];
   int active[3];
 };
+// The fourth power of a smaller wave speed, the square of the fast speed's a, has
+// fewer than 13 (FP32) or 26 (FP64) bits left in the subnormal range.
+__host__ __device__ inline double speed_min(bool fp64) { return fp64 ? 0x1p-262 : 0x1p-34; }
 cudaError_t launch_prep(const PrepArgs& a, StepScalars* sc, unsigned long long* lam_bits,
                         unsigned int* est_bits, unsigned int* status, cudaStream_t stream);
 // out[0..3] = (t, dt, c_h, steps) of the last step (device array).
