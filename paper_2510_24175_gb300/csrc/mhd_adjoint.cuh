@@ -60,8 +60,9 @@ MHD_HD void glm_hlld_flux_vjp(const T vl[kNV], const T vr[kNV], int dir, T ch, T
   const T SuL = SL - uL, SuR = SR - uR;
   const T dL = SuL * rL, dR = SuR * rR;
   const T Di = rcp(dR - dL);
-  const T NDi = (dR * (uR - uL) + (ptL - ptR)) * Di;
-  const T SM0 = uL + NDi;
+  const bool hL = mag_ge(dL, dR);
+  const T nh = ((hL ? dR : dL) * (uR - uL) + (ptL - ptR)) * Di;
+  const T SM0 = (hL ? uL : uR) + nh;
 
   const bool sup = gt0(SL) || lt0(SR);
   const bool useL = gt0(SL) || (!lt0(SR) && ge0(SM0));
@@ -70,7 +71,7 @@ MHD_HD void glm_hlld_flux_vjp(const T vl[kNV], const T vr[kNV], int dir, T ch, T
   const T pt = useL ? ptL : ptR, S = useL ? SL : SR, Su = useL ? SuL : SuR;
   const T d = useL ? dL : dR;
   const T SM = sup ? u : SM0;
-  const T du = SM - u;
+  const T du = useL == hL && !sup ? nh : SM - u;
   const T pts = d * du + pt;
   const T sm = S - SM;
   const T den = d * sm - bx2;
@@ -283,14 +284,14 @@ MHD_HD void glm_hlld_flux_vjp(const T vl[kNV], const T vr[kNV], int dir, T ch, T
   T dL_ = useL ? d_ : do_, dR_ = useL ? do_ : d_;
   T SL_ = useL ? S_ : So_, SR_ = useL ? So_ : S_;
   T SuL_ = useL ? Su_ : T(0), SuR_ = useL ? T(0) : Su_;
-  // S_M = u_L + (d_R (u_R - u_L) + pt_L - pt_R) / (d_R - d_L)
+  // S_M = (d_R u_R - d_L u_L + pt_L - pt_R) / (d_R - d_L); S_M - u_L and u_R - S_M from nh
   {
     const T n_ = SM_ * Di;
-    const T ndr = n_ * dR, nd = n_ * NDi;
-    uL_ += SM_ - ndr;
-    uR_ += ndr;
-    dR_ += n_ * (uR - uL) - nd;
-    dL_ += nd;
+    const T dw = uR - uL;
+    uL_ -= n_ * dL;
+    uR_ += n_ * dR;
+    dR_ += n_ * (hL ? dw - nh : -nh);
+    dL_ += n_ * (hL ? nh : dw + nh);
     ptL_ += n_;
     ptR_ -= n_;
   }
