@@ -48,7 +48,7 @@ sys.path.insert(0, ROOT)
 # smsp__inst_executed_pipe_fp64 x 32 / cells over the timed steps of this
 # bench's Orszag-Tang 256^3 run (profiles/).  They change whenever the kernel
 # does.
-FP64_INST_PER_CELL = {1: 688.3, 2: 711.5}
+FP64_INST_PER_CELL = {1: 692.7, 2: 713.8}
 # DRAM bytes per cell of the stage kernel's launches (ncu dram__bytes_read +
 # dram__bytes_write over the timed steps of this bench's 256^3 FP64 and 512^3
 # FP32 runs, profiles/); reported as the roofline's traffic per launch.  Set
@@ -57,22 +57,23 @@ TRAFFIC_BYTES_PER_CELL = {8: {1: 150.7, 2: 223.5}, 4: {1: 76.0, 2: 111.8}}
 # Nominal FP64 peak: 2 lanes/clk/SM x 152 SMs x 2.07 GHz = 629 G
 # lane-instructions/s (1.26 TFLOP/s counting an FMA as 2).  The measured one,
 # mhd_fp64_fma_rate in the same run, is reported beside it (1.99 lanes/clk/SM
-# for FMAs on register operands, 1.68 with a constant operand; the SM's FP64 unit is shared by its warps, and one warp issues
-# an FP64 instruction at most every 64 clocks).
+# for FMAs on register operands, 1.68 with a constant operand; the SM's FP64 unit
+# is shared by its warps, and one warp issues an FP64 instruction at most every
+# 64 clocks).
 FP64_PEAK_GINST = 2 * 152 * 2.07
 # Warp-instructions per cell of the FP32 stage kernel (ncu smsp__inst_executed
 # / cells, turbulent box 512^3, stage 1 / stage 2; profiles/) and the issue
 # peak they run against: 4 warp-instructions per clock per SM (one per
 # scheduler) x 152 SMs x 2.07 GHz.
-FP32_WARP_INST_PER_CELL = {1: 53.59, 2: 57.05}
+FP32_WARP_INST_PER_CELL = {1: 55.20, 2: 59.05}
 ISSUE_PEAK_GINST = 4 * 152 * 2.07
 # FP64-pipe lane-instructions per cell of the FP64 WENO-Z stage kernel (ncu,
 # Orszag-Tang 256^3; first / middle / last SSP-RK3 stage).
-WENO_FP64_INST_PER_CELL = {"stage1": 2057.8, "stage_mid": 2076.7, "stage2": 2079.9}
+WENO_FP64_INST_PER_CELL = {"stage1": 2060.0, "stage_mid": 2080.0, "stage2": 2084.3}
 # Warp-instructions per cell of the FP32 WENO-Z stage kernel (ncu
 # smsp__inst_executed / cells, Orszag-Tang 256^3; first / middle / last
 # SSP-RK3 stage).
-WENO_FP32_WARP_INST_PER_CELL = {"stage1": 106.62, "stage_mid": 107.62, "stage2": 110.86}
+WENO_FP32_WARP_INST_PER_CELL = {"stage1": 107.69, "stage_mid": 109.21, "stage2": 112.87}
 # Algorithmic HBM bytes per cell: stage 1 reads U^n and writes U1 (18 words),
 # stage 2 reads U1 and U^n and writes U^{n+1} (27 words).
 WORDS_STAGE = {1: 18, 2: 27}

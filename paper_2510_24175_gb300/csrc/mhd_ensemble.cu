@@ -35,7 +35,7 @@ namespace cg = cooperative_groups;
 namespace mhd {
 
 // Eight warps per CTA, 128 registers, two CTAs per SM.  (64 boxes of up to 128^3, 5 steps:
-// 41.8 ms; 57.4 with scalar loads, slopes and one slope array per direction.)
+// 42.6 ms; 57.4 with scalar loads, slopes and one slope array per direction.)
 constexpr int kEnsNW = 8;
 constexpr int kEnsTYs[2] = {8, 4};  // the tile heights of the two kernel instantiations
 
@@ -121,7 +121,7 @@ __device__ __forceinline__ void ens_stage(const EnsArgs& a, unsigned char* smem,
 // 8 warps per CTA, two CTAs per SM: with 12 and 16 warps per CTA (80 and 64
 // registers, the per-box kernel's shape) the persistent kernel, which also keeps
 // a box's parameters, spilled 500 bytes a thread and took 56.0 and 56.6 ms for
-// five steps of 64 boxes against 49.5 (41.8 with paired values).  WIDE: a box has
+// five steps of 64 boxes against 49.5 (42.6 with paired values).  WIDE: a box has
 // planes beyond 32-bit offsets (the tile code's 64-bit form).
 template <int TY, bool WIDE>
 __global__ void __launch_bounds__(kEnsNW * 32, 2) ensemble_kernel(const EnsArgs a) {

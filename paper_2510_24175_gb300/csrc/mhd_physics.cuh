@@ -793,13 +793,14 @@ MHD_HD T rot3(int dir, int j, T a, T b, T c) {
 // every kernel and at every call site it is inlined into (the results of
 // decomposed and undecomposed runs must agree bit for bit).
 // FP64 is bound by the SM's FP64 unit, so the solver is arranged for few FP64
-// operations: about 95 per face, 130 where a lane of the warp is inside the
+// operations: about 96 per face, 131 where a lane of the warp is inside the
 // Alfven fan (the form that builds both sides' star and double-star states and
 // adds up the wave jumps took about 280 with CUDA's divisions and roots).
-// Orszag-Tang 256^3 FP64: 76.4 -> 47.4 ms per step (44.0 with what came after), of
-// which the fixed-point reciprocals and roots 11.  Against a quadruple-precision evaluation its
-// error is at most that of the longer form (2e-16 to 3e-15 rms of the flux,
-// random, smooth, Mach-20, low- and high-beta and degenerate face states).
+// Orszag-Tang 256^3 FP64: 76.4 -> 47.4 ms per step (45.0 with what came after), of
+// which the fixed-point reciprocals and roots 11.  Against a quadruple-precision
+// evaluation its error is at most that of the longer form (2e-16 to 3e-15 rms of
+// the flux, random, smooth, Mach-20, low- and high-beta and degenerate face states;
+// for density contrasts see du below).
 template <int dir, class T>
 MHD_HD void glm_hlld_flux(const T vl[kNV], const T vr[kNV], T ch, T half_chi,
                           const Phys<T>& ph, T F[kNV]) {

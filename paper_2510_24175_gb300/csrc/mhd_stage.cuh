@@ -25,7 +25,7 @@
 //
 // This kernel runs FP64 grids and the 1-D and 2-D FP32 ones (3-D FP32:
 // mhd_stage_pairs.cuh).  In FP64 it is bound by the SM's FP64 unit, 88 % of whose
-// cycles it uses (Orszag-Tang 256^3, a step of two stages 44.0 ms); the sums,
+// cycles it uses (Orszag-Tang 256^3, a step of two stages 45.0 ms); the sums,
 // differences and products run as fused multiply-adds on register operands (add_f),
 // and in 3-D phase D of a plane runs at the same time as A and B of the next (kRoles).
 #pragma once

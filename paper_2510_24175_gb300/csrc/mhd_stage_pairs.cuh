@@ -14,7 +14,7 @@
 //     and grids with planes of 4 GB and more take it, with or without halo faces.
 // The arithmetic of a cell is that of every other instantiation, operation by
 // operation (packed instructions round like scalar ones).  Turbulent box 512^3, a
-// step of two stages: 24.9 ms (32.6 with scalar values, slopes in shared memory and
+// step of two stages: 25.1 ms (32.6 with scalar values, slopes in shared memory and
 // 16 warps per SM; 27.7 with 32 warps); Orszag-Tang 256^3 WENO-Z with constrained
 // transport, a step of three stages: 11.0 ms (13.6).
 #pragma once
